@@ -37,6 +37,7 @@
 // depend on scheduling.
 #include <math.h>
 
+#include <algorithm>
 #include <atomic>
 
 #include "gbs_internal.cuh"
@@ -1224,9 +1225,17 @@ __global__ void pairing_select_kernel(const PairingSelect S) {
 
 // ---- repeated-row route (Kan's moment identity; see RepLaunch) ----------
 
+// The modes split into low ones (the fastest digits, as many as give at most
+// kRepLow digit combinations) and high ones; the low ones again into two
+// groups of T1 and T2 combinations.
+constexpr int kRepLow = 256;
 struct RepWarp {
   double2 B[kRepMaxDistinct * kRepMaxDistinct];  // B_v, row stride kRepMaxDistinct
-  double x[kRepMaxDistinct][32];                  // x_j of each lane's current term (column = lane)
+  double2 C[kRepLow];           // x^T B_v x / 2 over the low modes, per combination
+  double2 S1[kMaxN + 2];        // per combination of the first group: its x . y, plus the high modes' share
+  double2 S2[kRepLow / 2];      // per combination of the second group: its x . y
+  double2 y[kRepMaxDistinct];   // B_v x over the high modes, per low mode
+  double w[kRepLow];            // prod (-1)^nu_j C(c_j, nu_j) over the low modes
   int c[kRepMaxDistinct];                         // multiplicities c_j
   int mode[kRepMaxDistinct];                      // distinct modes v_j
 };
@@ -1256,62 +1265,154 @@ __device__ __forceinline__ void store_warp_partial(Comp<double> re, Comp<double>
   }
 }
 
-// Terms t0 + q, q = lane, lane + 32, ... < count, for D distinct modes: digits
-// nu_j of t (mixed radix c_j + 1, j = 0 fastest), x_j = c_j - 2 nu_j (kept in
-// the lane's own column of W.x), the weight prod (-1)^nu_j C(c_j, nu_j),
-// Q = x^T B_v x / 2 evaluated as sum_j x_j (B_jj x_j / 2 + sum_{k>j} B_jk x_k)
-// (x integer, so every product with x is one rounding), Q^h by squaring, and
-// the term times 2 / (2^n h!) (1 / (2^n h!) for the middle term
-// t = (T - 1) / 2, which is its own mirror).
+// s + e += v (Knuth's two-sum; e gathers the rounding errors).
+__device__ __forceinline__ void sum_add(Comp<double>& a, double v) {
+  const double s = a.hi + v;
+  const double b = s - a.hi;
+  a.lo += (a.hi - (s - b)) + (v - b);
+  a.hi = s;
+}
+
+// Terms t0 <= t < t0 + count for D distinct modes: digits nu_j of t (mixed
+// radix c_j + 1, j = 0 fastest), x_j = c_j - 2 nu_j, the weight prod (-1)^nu_j
+// C(c_j, nu_j), Q = x^T B_v x / 2, Q^h by squaring, and the term times
+// 2 / (2^n h!) (1 / (2^n h!) for the middle term t = (T - 1) / 2, which is its
+// own mirror).
+//
+// Q = C[l] + (x . y over the low modes) + (the high modes alone), l the low
+// digits: C depends on the pattern only, y and the high share on the high
+// digits only, and x . y splits over the two groups of low modes. So a term
+// forms its Q in three complex additions from tables instead of the d^2 / 2
+// multiply-adds of the quadratic form, and takes 41 FP64 operations at h = 12
+// where it took 170 (d = 8); the tables add about a quarter. The FP64 pipe
+// bounds it: 512 patterns of n = 24 in 8 modes (2^15 terms each) went from
+// 3.5 to 1.75 ms (whole call). The sum keeps its rounding errors (Knuth's two-sum, once a
+// component and term), as it did.
 __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN + 1], int D, int h, int t0,
                                           int count, int T, double scale, int lane, Comp<double>& re,
                                           Comp<double>& im, double& kap) {
-  for (int q = lane; q < count; q += 32) {
-    const int t = t0 + q;
-    int rem = t;
-    double w = 1.0;
-    for (int j = 0; j < D; ++j) {
-      const int cj = W.c[j];
-      const int nu = rem % (cj + 1);
+  const unsigned FULL = 0xffffffffu;
+  // low modes [0, dl), the first group [0, d1)
+  int dl = 1, TL = W.c[0] + 1;
+  while (dl < D && TL * (W.c[dl] + 1) <= kRepLow) TL *= W.c[dl++] + 1;
+  int d1 = 1, T1 = W.c[0] + 1;
+  while (d1 < dl && T1 * (W.c[d1] + 1) <= 32) T1 *= W.c[d1++] + 1;
+  const int T2 = TL / T1;
+  for (int l = lane; l < TL; l += 32) {
+    double w = 1.0, qr = 0.0, qi = 0.0;
+    int rem = l;
+    for (int j = 0; j < dl; ++j) {
+      const int cj = W.c[j], nu = rem % (cj + 1);
       rem /= (cj + 1);
-      W.x[j][lane] = (double)(cj - 2 * nu);
-      const double bw = (double)binom[cj][nu];
+      const double xj = (double)(cj - 2 * nu), bw = (double)binom[cj][nu], hx = 0.5 * xj;
       w *= (nu & 1) ? -bw : bw;
-    }
-    double qr = 0.0, qi = 0.0;
-    for (int j = 0; j < D; ++j) {
-      const double xj = W.x[j][lane];
       const double2 bjj = W.B[j * kRepMaxDistinct + j];
-      const double hx = 0.5 * xj;
       double sr = bjj.x * hx, si = bjj.y * hx;
-      for (int k = j + 1; k < D; ++k) {
+      int rk = rem;
+      for (int k = j + 1; k < dl; ++k) {
+        const int ck = W.c[k];
+        const double xk = (double)(ck - 2 * (rk % (ck + 1)));
+        rk /= (ck + 1);
         const double2 b = W.B[j * kRepMaxDistinct + k];
-        const double xk = W.x[k][lane];
         sr = fma(b.x, xk, sr);
         si = fma(b.y, xk, si);
       }
       qr = fma(xj, sr, qr);
       qi = fma(xj, si, qi);
     }
-    double pr = 1.0, pi = 0.0, br = qr, bi = qi;
-    for (int e = h; e > 0; e >>= 1) {
-      if (e & 1) {
-        const double tr = fma(pr, br, -pi * bi);
-        pi = fma(pr, bi, pi * br);
-        pr = tr;
-      }
-      if (e > 1) {
-        const double tr = fma(br, br, -bi * bi);
-        bi = 2.0 * br * bi;
-        br = tr;
+    W.w[l] = w;
+    W.C[l] = make_double2(qr, qi);
+  }
+  double kp = 0.0;
+  for (int H = t0 / TL; (int64_t)H * TL < t0 + count; ++H) {
+    const int base = H * TL;
+    // the high digits' weight; lane j < dl takes y_j, lane j >= dl the high
+    // mode j's x_j (B_jj x_j / 2 + sum_{k > j} B_jk x_k)
+    double wh = 1.0, ar = 0.0, ai = 0.0, xl = 0.0;
+    int rem = H;
+    for (int j = dl; j < D; ++j) {
+      const int cj = W.c[j], nu = rem % (cj + 1);
+      rem /= (cj + 1);
+      const double xj = (double)(cj - 2 * nu), bw = (double)binom[cj][nu];
+      wh *= (nu & 1) ? -bw : bw;
+      if (lane <= j) {
+        const double2 b = W.B[lane * kRepMaxDistinct + j];
+        const double f = (lane == j) ? 0.5 * xj : xj;
+        ar = fma(b.x, f, ar);
+        ai = fma(b.y, f, ai);
+        if (lane == j) xl = xj;
       }
     }
-    const double f = w * ((2 * t + 1 == T) ? scale : 2.0 * scale);
-    const double vr = f * pr, vi = f * pi;
-    comp_add<double>(re, vr);
-    comp_add<double>(im, vi);
-    kap += fabs(vr) + fabs(vi);
+    __syncwarp();
+    if (lane < dl) W.y[lane] = make_double2(ar, ai);
+    // lanes outside [dl, D) hold xl = 0
+    double hr = ar * xl, hi = ai * xl;
+    for (int off = 8; off > 0; off >>= 1) {
+      hr += __shfl_xor_sync(FULL, hr, off);
+      hi += __shfl_xor_sync(FULL, hi, off);
+    }
+    hr = __shfl_sync(FULL, hr, 0);
+    hi = __shfl_sync(FULL, hi, 0);
+    __syncwarp();
+    for (int l = lane; l < T1 + T2; l += 32) {
+      const bool first = l < T1;
+      int r = first ? l : l - T1;
+      double sr = first ? hr : 0.0, si = first ? hi : 0.0;
+      for (int j = first ? 0 : d1; j < (first ? d1 : dl); ++j) {
+        const int cj = W.c[j];
+        const double xj = (double)(cj - 2 * (r % (cj + 1)));
+        r /= (cj + 1);
+        const double2 y = W.y[j];
+        sr = fma(xj, y.x, sr);
+        si = fma(xj, y.y, si);
+      }
+      (first ? W.S1[l] : W.S2[l - T1]) = make_double2(sr, si);
+    }
+    __syncwarp();
+    const int end = min(TL, t0 + count - base);
+    for (int l = max(t0 - base, 0) + lane; l < end; l += 32) {
+      const int l2 = l / T1, l1 = l - l2 * T1;
+      const double2 c = W.C[l], s1 = W.S1[l1], s2 = W.S2[l2];
+      const double qr = c.x + (s1.x + s2.x), qi = c.y + (s1.y + s2.y);
+      double pr = 1.0, pi = 0.0, br = qr, bi = qi;
+      bool one = true;  // p = 1 (uniform: the exponent is)
+      for (int e = h; e > 0; e >>= 1) {
+        if (e & 1) {
+          if (one) {
+            pr = br;
+            pi = bi;
+            one = false;
+          } else {
+            const double tr = fma(pr, br, -pi * bi);
+            pi = fma(pr, bi, pi * br);
+            pr = tr;
+          }
+        }
+        if (e > 1) {
+          const double tr = fma(br, br, -bi * bi);
+          bi = (br + br) * bi;
+          br = tr;
+        }
+      }
+      double f = W.w[l];
+      if (2 * (base + l) + 1 == T) f *= 0.5;
+      const double vr = f * pr, vi = f * pi;
+      sum_add(re, wh * vr);
+      sum_add(im, wh * vi);
+      kp = fma(fabs(wh), fabs(vr) + fabs(vi), kp);
+    }
+    __syncwarp();
   }
+  // the common factor 2 / (2^n h!)
+  const double g = 2.0 * scale;
+  auto scaled = [&](Comp<double>& a) {
+    const double p = a.hi * g;
+    a.lo = fma(a.hi, g, -p) + a.lo * g;
+    a.hi = p;
+  };
+  scaled(re);
+  scaled(im);
+  kap += kp * g;
 }
 
 // Persistent warps over repeated-row work items. Per item: the matrix's index
@@ -1319,7 +1420,8 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
 // __match_any_sync (order of first occurrence), B_v gathered into the warp's
 // shared slot, then the item's terms.
 __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
-  __shared__ RepWarp ws[4];
+  extern __shared__ __align__(16) unsigned char rep_smem[];
+  RepWarp* ws = reinterpret_cast<RepWarp*>(rep_smem);
   __shared__ int binom[kMaxN + 1][kMaxN + 1];
   // the grid covers the reservation; with no item (no bunched pattern) every
   // block leaves before building its table (uniform over the block)
@@ -1519,10 +1621,18 @@ cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  constexpr int smem = 4 * (int)sizeof(RepWarp);
+  static std::atomic<int> done[64];
+  if (!done[dev].load(std::memory_order_acquire)) {
+    const cudaError_t e = cudaFuncSetAttribute(haf_repeated_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    done[dev].store(1, std::memory_order_release);
+  }
   int blocks = (R.n_items + 3) / 4;
-  const int cap = (sms > 0 ? sms : 1) * 8;
+  const int cap = (sms > 0 ? sms : 1) * (int)std::min<size_t>(8, (size_t)220 * 1024 / smem);
   if (blocks > cap) blocks = cap;
-  haf_repeated_kernel<<<blocks, 128, 0, st>>>(R);
+  haf_repeated_kernel<<<blocks, 128, smem, st>>>(R);
   return cudaGetLastError();
 }
 
