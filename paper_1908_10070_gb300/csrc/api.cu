@@ -242,6 +242,38 @@ bool shape_fits(int precision, int warp_bytes, int maxn) {
   return true;
 }
 
+// Launch shape of the terms kernel: the most warps (one block per SM, up to
+// kTermsWarps) whose shared memory holds every lane group of orders <= n.
+// Measured on 4096 patterns of n = 16 and 80 of n = 28 and 30 (all outputs):
+// 6 / 8 / 10 / 12 warps 4.17 / 3.62 / 3.36 / 3.46 ms at n = 16; at n = 28 no
+// more than 6 fit. Rounds per item 1 / 2 / 4 / 8: 3.57 / 3.41 / 3.36 / 3.36 ms
+// and 77.7 / 62.3 / 54.9 / 52.1 ms (few subsets in an item leave the series,
+// one lane per subset, mostly idle); small batches halve them as needed.
+constexpr int kTermsWarps = 10;
+static TuneCfg terms_cfg(int n) {
+  static const int optin = [] {  // thread-safe one-time initialisation
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || v <= 0) {
+      cudaGetLastError();
+      v = 232448;  // 227 KB, the GB300 opt-in limit
+    }
+    return v;
+  }();
+  TuneCfg c;
+  const int h = std::max(n / 2, 1);
+  c.rounds = 8;
+  for (int w = kTermsWarps; w >= 1; --w) {
+    c.warps_per_block = w;
+    c.warp_bytes = ((optin - 4096) / w) & ~127;
+    bool fits = true;
+    for (int v = 1; v <= h; ++v)
+      for (int s = 1; s <= v; ++s) fits = fits && terms_lanes(s, v, c.warp_bytes, h) != 0;
+    if (fits) break;
+  }
+  return c;
+}
+
 int64_t binom64(int a, int b) {
   if (b < 0 || b > a) return 0;
   int64_t r = 1;
@@ -267,7 +299,7 @@ static int64_t key_cost(int key) {
 }
 
 void Planner::init(const int* n, int batch, int precision, int warp_bytes, const int* rounds_for_n,
-                   int64_t whole_reserve) {
+                   int64_t whole_reserve, bool terms) {
   n_ = n;
   batch_ = batch;
   const int cb = complex_bytes(precision);
@@ -293,7 +325,7 @@ void Planner::init(const int* n, int batch, int precision, int warp_bytes, const
       total_ += nwhole_[v];
     }
     for (int sz = 1; sz <= h; ++sz) {
-      const int G = 32 / lanes_for(2 * sz, h, warp_bytes, stage_h, cb);
+      const int G = 32 / (terms ? terms_lanes(sz, h, warp_bytes, stage_h) : lanes_for(2 * sz, h, warp_bytes, stage_h, cb));
       const int64_t cnt = binom64(h, sz), cap = (int64_t)G * R;
       for (int64_t r0 = 0; r0 < cnt; r0 += cap) {
         ItemTemplate t;
@@ -537,7 +569,100 @@ struct BatchLayout {
   size_t perm_b = 0, ppats_b = 0, pitems_b = 0, pperm_b = 0, selpat_b = 0, probe_up_b = 0;
   size_t choff_b = 0, chpat_b = 0, up_b = 0;
   size_t probe_at = 0, chunk_at = 0;
+  // matching route: the even-order matrices by order (largest first), the
+  // tiles of the small ones, and the scratch of the large ones
+  bool match = false, terms = false;
+  TuneCfg tcfg;  // terms kernel's launch shape
+  size_t matoff_at = 0, arena_b = 0;
+  int by_order[kMaxN + 1] = {0}, first_of[kMaxN + 1] = {0}, n_order = 0, n_tiles = 0;
+  size_t order_at = 0, tiles_at = 0, tile_smem = 0, match_b = 0;
 };
+
+// Scratch of the matching route's larger orders: the matrices of a call go in
+// chunks of at most this many bytes (one matrix of order 32 takes 34 MB). A
+// chunk costs about 25 launches, against 4 ms of work in 512 MB of order 28.
+constexpr size_t kMatchBudget = (size_t)512 << 20;
+
+// Lay out the matching route for the call's orders: `order` (matrices of even
+// order >= 2, largest order first) and the tiles of orders <= kMatchSmallMax.
+static void plan_matching(const int* n, int batch, int sms, BatchLayout& U, std::vector<int>* order,
+                          std::vector<MatchTile>* tiles) {
+  for (int b = 0; b < batch; ++b)
+    if (n[b] >= 2 && !(n[b] & 1)) U.by_order[n[b]]++;
+  for (int v = kMaxN; v >= 2; v -= 2) {
+    U.first_of[v] = U.n_order;
+    U.n_order += U.by_order[v];
+  }
+  order->resize(std::max(U.n_order, 1));
+  int at[kMaxN + 1];
+  std::copy(U.first_of, U.first_of + kMaxN + 1, at);
+  for (int b = 0; b < batch; ++b)
+    if (n[b] >= 2 && !(n[b] & 1)) (*order)[at[n[b]]++] = b;
+  for (int v = kMatchSmallMax; v >= 2; v -= 2) {
+    const int cnt = U.by_order[v];
+    if (!cnt) continue;
+    MatchTile t;
+    t.n = v;
+    match_sizes(v, &t.even, &t.odd, nullptr);
+    const size_t one = 16 * ((size_t)t.even + t.odd + v * (v - 1) / 2);
+    // as many matrices side by side as fit, while the tiles still fill the
+    // SMs twice
+    t.lp = 0;
+    while (t.lp < 5 && (one << (t.lp + 1)) <= (size_t)kMatchTileBytes && (cnt >> (t.lp + 1)) >= 2 * sms) ++t.lp;
+    U.tile_smem = std::max(U.tile_smem, one << t.lp);
+    for (int k = 0; k < cnt; k += 1 << t.lp) {
+      t.first = U.first_of[v] + k;
+      t.count = std::min(1 << t.lp, cnt - k);
+      tiles->push_back(t);
+    }
+  }
+  U.n_tiles = (int)tiles->size();
+  size_t large = 0, most = 0;
+  for (int v = kMatchSmallMax + 2; v <= kMaxN; v += 2)
+    if (U.by_order[v]) {
+      large += U.by_order[v] * match_matrix_bytes(v);
+      most = match_matrix_bytes(v);
+    }
+  U.match_b = std::max(most, std::min(large, kMatchBudget));
+}
+
+// The chunks of the larger orders, each within U.match_b bytes of scratch.
+static void match_chunks(const BatchLayout& U, double* scratch, std::vector<MatchChunk>* out) {
+  MatchChunk c;
+  memset(&c, 0, sizeof(c));
+  size_t used = 0;
+  int mats = 0;
+  for (int v = kMaxN; v > kMatchSmallMax; v -= 2) {
+    const size_t one = match_matrix_bytes(v);
+    for (int done = 0; done < U.by_order[v];) {
+      const int take = (int)std::min<size_t>(U.by_order[v] - done, (U.match_b - used) / one);
+      if (take == 0) {
+        c.scratch = scratch;
+        out->push_back(c);
+        memset(&c, 0, sizeof(c));
+        used = 0;
+        mats = 0;
+        continue;
+      }
+      MatchGroup& g = c.g[c.n_groups++];
+      int odd;
+      g.n = v;
+      g.first = U.first_of[v] + done;
+      g.count = take;
+      g.begin = mats;
+      match_sizes(v, &g.even, &odd, nullptr);
+      g.off = (int64_t)(used / 16);
+      g.stride = (int64_t)(one / 16);
+      used += take * one;
+      mats += take;
+      done += take;
+    }
+  }
+  if (c.n_groups) {
+    c.scratch = scratch;
+    out->push_back(c);
+  }
+}
 
 // Plans of repeated batch shapes. The plan block depends only on the orders,
 // offsets, m and launch shapes (never on the index lists or matrices), so a
@@ -547,7 +672,7 @@ struct BatchLayout {
 // evicted least recently used, never while a call is using them, and only
 // after the device has finished every launch that read them.
 struct PlanKey {
-  int mode, precision, batch, maxn, m, device, sms, probe32;
+  int mode, precision, batch, maxn, m, device, sms, probe32, match;
   int wpb, warp_bytes, pwpb, pwarp_bytes;
   int rounds[kMaxN + 1];
   bool operator==(const PlanKey& o) const { return memcmp(this, &o, sizeof(PlanKey)) == 0; }
@@ -682,6 +807,11 @@ int run_batch(const BatchArgs& a) {
   }
   (hmode ? U.src_elems : U.idx_elems) = elems;
   const int maxn = U.maxn;
+  // FP64: the Hafnians by partial matchings; the subset sum's terms are formed
+  // (in fixed point) only for the error estimate made of their moduli. Tuning
+  // runs time the subset sum itself.
+  U.match = a.precision == GBS_FP64 && !a.cfg_override && maxn <= kMatchMaxN;
+  U.terms = U.match && a.out3 != nullptr;
   // launch shape from the largest n (it dominates the cost); rounds per n
   U.cfg = a.cfg_override ? *a.cfg_override : get_cfg(a.precision, maxn);
   const TuneCfg& cfg = U.cfg;
@@ -733,6 +863,7 @@ int run_batch(const BatchArgs& a) {
     cudaGetDevice(&key.device);
     key.sms = device_sm_count();
     key.probe32 = U.probe32;
+    key.match = (U.match ? 1 : 0) + (U.terms ? 2 : 0);
     key.wpb = cfg.warps_per_block;
     key.warp_bytes = cfg.warp_bytes;
     key.pwpb = U.pcfg.warps_per_block;
@@ -753,7 +884,7 @@ int run_batch(const BatchArgs& a) {
   unsigned char* hs = nullptr;
   if (!hit) {
     // (a kept plan's shape was checked when it was made)
-    if (!shape_fits(a.precision, cfg.warp_bytes, maxn))
+    if (!U.match && !shape_fits(a.precision, cfg.warp_bytes, maxn))
       return fail(GBS_EINVAL, "warp_bytes %d too small for n = %d", cfg.warp_bytes, maxn);
     Planner plan;
     // a few items per resident warp balance the load over all SMs; whole-matrix
@@ -765,8 +896,22 @@ int run_batch(const BatchArgs& a) {
     const int64_t want = 4LL * device_sm_count() * cfg.warps_per_block;
     const int64_t reserve = a.cfg_override ? 0
                           : (int64_t)device_sm_count() * cfg.warps_per_block / (a.precision == GBS_FP64 ? 2 : 1);
-    plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
-    if (!a.cfg_override) {
+    std::vector<int> order;
+    std::vector<MatchTile> tiles;
+    if (U.match) plan_matching(a.n, batch, device_sm_count(), U, &order, &tiles);
+    if (U.terms) {
+      U.tcfg = terms_cfg(maxn);
+      for (int v = 0; v <= kMaxN; ++v) rounds_for_n[v] = U.tcfg.rounds;
+    }
+    auto init = [&]() {
+      if (U.terms)
+        plan.init(a.n, batch, a.precision, U.tcfg.warp_bytes, rounds_for_n,
+                  (int64_t)device_sm_count() * U.tcfg.warps_per_block / 2, true);
+      else if (!U.match)
+        plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
+    };
+    init();
+    if (!a.cfg_override && (U.terms || !U.match)) {
       // A small batch gets smaller work items (fewer rounds each) for the same reason.
       for (int iter = 0; iter < 6 && plan.total() < want; ++iter) {
         bool shrunk = false;
@@ -776,7 +921,7 @@ int run_batch(const BatchArgs& a) {
             shrunk = true;
           }
         if (!shrunk) break;
-        plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
+        init();
       }
     }
     U.n_items = plan.total();
@@ -795,10 +940,10 @@ int run_batch(const BatchArgs& a) {
     }
 
     // plan block: pats | items | (pair-sum offsets) | (probe tables) | (chunk
-    // tables)
+    // tables) | (order | tiles of the matchings) | (arena offsets of the terms)
     U.pats_b = al(sizeof(PatDesc) * batch);
     U.items_b = al(sizeof(WorkItem) * std::max<int64_t>(U.n_items, 1));
-    if (a.precision == GBS_FP64)
+    if (a.precision == GBS_FP64 && !U.match)
       for (int b = 0; b < batch; ++b) {
         const int64_t q = pair_terms_elems(a.n[b]);
         if (q > 0 && 16 * (U.pt_elems + q) <= kPairTermBudget) U.pt_elems += q;
@@ -819,7 +964,8 @@ int run_batch(const BatchArgs& a) {
     // two-stage finalisation when some matrix has more than kChunkItems items
     std::vector<int> chunk_off, chunk_pat;
     int max_items = 0;
-    for (int b = 0; b < batch; ++b) max_items = std::max(max_items, plan.items_for(b));
+    if (!U.match)
+      for (int b = 0; b < batch; ++b) max_items = std::max(max_items, plan.items_for(b));
     if (max_items > kChunkItems) {
       chunk_off.resize(batch + 1);
       for (int b = 0; b < batch; ++b) {
@@ -835,14 +981,52 @@ int run_batch(const BatchArgs& a) {
     U.up_b = U.pats_b + U.items_b + U.ptoff_b + U.probe_up_b + U.choff_b + U.chpat_b;
     U.probe_at = U.pats_b + U.items_b + U.ptoff_b;
     U.chunk_at = U.probe_at + U.probe_up_b;
+    if (U.match) {
+      U.order_at = U.up_b;
+      U.tiles_at = U.order_at + al(sizeof(int) * order.size());
+      U.up_b = U.tiles_at + al(sizeof(MatchTile) * std::max<size_t>(tiles.size(), 1));
+    }
+    if (U.terms) {
+      U.matoff_at = U.up_b;
+      U.up_b += al(2 * sizeof(int64_t) * batch);
+    }
 
     int rc = pinned_acquire(U.up_b + data_b, &host_stage, &slot);
     if (rc) return rc;
     hs = (unsigned char*)host_stage;
     PatDesc* h_pats = (PatDesc*)hs;
-    plan.fill(h_pats, (WorkItem*)(hs + U.pats_b));
+    if (U.terms || !U.match) plan.fill(h_pats, (WorkItem*)(hs + U.pats_b));
+    if (U.match) {
+      memcpy(hs + U.order_at, order.data(), sizeof(int) * order.size());
+      if (!tiles.empty()) memcpy(hs + U.tiles_at, tiles.data(), sizeof(MatchTile) * tiles.size());
+    }
+    if (U.terms) {
+      // every even-order matrix's blocks, and its pair sums while they fit the
+      // budget (later matrices form A_S X A_S by the product)
+      int64_t* mat_off = (int64_t*)(hs + U.matoff_at);
+      int64_t* sum_off = mat_off + batch;
+      int64_t at = 0, sums = 0;
+      for (int b = 0; b < batch; ++b) {
+        const int v = a.n[b], h = v / 2, nb = h * (h + 1) / 2;
+        mat_off[b] = sum_off[b] = -1;
+        if (v < 2 || (v & 1)) continue;
+        mat_off[b] = at;
+        at += 4 * nb;
+        const int64_t q = v >= 6 ? 4ll * nb * pair_sums_width(h) : 0;
+        if (q > 0 && 16 * (sums + q) <= kPairTermBudget) {
+          sum_off[b] = at;
+          at += q;
+          sums += q;
+        }
+      }
+      U.arena_b = al(16 * (size_t)at);
+    }
     for (int b = 0; b < batch; ++b) {
       PatDesc& d = h_pats[b];
+      if (U.match && !U.terms) {
+        d.n = a.n[b];
+        d.item_begin = d.item_end = 0;
+      }
       if (a.mode == BatchArgs::HAFNIAN) {
         d.src_off = a.offs[b];
         d.idx_off = -1;
@@ -920,6 +1104,12 @@ int run_batch(const BatchArgs& a) {
   const size_t ctr_b = 256;
   const size_t status_b = al(sizeof(int) * batch);
   const size_t pstatus_b = n_sel ? al(sizeof(int) * n_probe) : 0;  // zeroed with ctr and status
+  const size_t ok_b = U.terms ? al(sizeof(int) * batch) : 0;       // zeroed too
+  // matchings: a partial per matrix | scratch; terms: exponents | item sums | matrix sums | arena
+  const size_t mparts_b = U.match ? al(sizeof(Partial) * batch) : 0;
+  const size_t exps_b = U.terms ? al(sizeof(int) * kExpInts * batch) : 0;
+  const size_t kparts_b = U.terms ? al(16 * std::max<int64_t>(n_items, 1)) : 0;
+  const size_t ksum_b = U.terms ? al(8 * (size_t)batch) : 0;
   // outputs in host memory (any of them sends all through device staging)
   bool out_hmem[4];
   {
@@ -936,7 +1126,8 @@ int run_batch(const BatchArgs& a) {
   const size_t mperm_b = n_sel ? al(sizeof(int) * batch) : 0;  // written by the probe's choice
   // route choice on the device: rep_half | rep_end | repeated-row partials
   const size_t droute_b = dev_rep_cap ? 2 * al(sizeof(int) * batch) + al(sizeof(Partial) * dev_rep_cap) : 0;
-  const size_t dev_b = data_b + parts_b + ctr_b + status_b + pstatus_b + outs_b + a32_b + pt_b + pparts_b + chparts_b + mperm_b + droute_b;
+  const size_t dev_b = data_b + parts_b + ctr_b + status_b + pstatus_b + outs_b + a32_b + pt_b + pparts_b + chparts_b + mperm_b + droute_b + ok_b +
+                       mparts_b + U.match_b + exps_b + kparts_b + ksum_b + U.arena_b;
   const size_t own_up_b = pe ? 0 : U.up_b;
 
   void* dmem = nullptr;
@@ -971,6 +1162,8 @@ int run_batch(const BatchArgs& a) {
   o += status_b;
   int* d_pstatus = n_sel ? (int*)(dv + o) : nullptr;
   o += pstatus_b;
+  int* d_ok = ok_b ? (int*)(dv + o) : nullptr;
+  o += ok_b;
   double* d_outs = outs_b ? (double*)(dv + o) : nullptr;
   o += outs_b;
   float* d_a32 = a32_b ? (float*)(dv + o) : nullptr;
@@ -986,6 +1179,18 @@ int run_batch(const BatchArgs& a) {
   int* d_rephalf = dev_rep_cap ? (int*)(dv + o) : nullptr;
   int* d_repend = dev_rep_cap ? (int*)(dv + o + al(sizeof(int) * batch)) : nullptr;
   Partial* d_repparts = dev_rep_cap ? (Partial*)(dv + o + 2 * al(sizeof(int) * batch)) : nullptr;
+  o += droute_b;
+  Partial* d_mparts = (Partial*)(dv + o);
+  o += mparts_b;
+  double* d_match = U.match_b ? (double*)(dv + o) : nullptr;
+  o += U.match_b;
+  int* d_exps = (int*)(dv + o);
+  o += exps_b;
+  double2* d_kparts = (double2*)(dv + o);
+  o += kparts_b;
+  double* d_ksum = (double*)(dv + o);
+  o += ksum_b;
+  int4* d_arena = (int4*)(dv + o);
 
   HafLaunch L;
   memset(&L, 0, sizeof(L));
@@ -1008,7 +1213,7 @@ int run_batch(const BatchArgs& a) {
       e = cudaMemcpyAsync(dv, hdata, data_b, cudaMemcpyHostToDevice, st);
       if (e != cudaSuccess) { ret = cuda_fail(e, "input upload"); break; }
     }
-    e = cudaMemsetAsync(d_ctr, 0, ctr_b + status_b + pstatus_b, st);
+    e = cudaMemsetAsync(d_ctr, 0, ctr_b + status_b + pstatus_b + ok_b, st);
     if (e != cudaSuccess) { ret = cuda_fail(e, "memset"); break; }
     if (d_mperm) {  // -1: the default ordering until the probe's choice replaces it
       e = cudaMemsetAsync(d_mperm, 0xff, sizeof(int) * batch, st);
@@ -1018,7 +1223,7 @@ int run_batch(const BatchArgs& a) {
       e = launch_to_float(d_src, d_a32, 2 * src_elems, st);
       if (e != cudaSuccess) { ret = cuda_fail(e, "float copy"); break; }
     }
-    if (n_items > 0) {
+    if (n_items > 0 || U.n_order > 0) {
       L.src = (a.mode == BatchArgs::HAFNIAN) ? d_src : a.B;
       L.src32 = (a.precision == GBS_MIXED) ? ((a.mode == BatchArgs::HAFNIAN) ? d_a32 : a.B32) : nullptr;
       L.idx = (a.mode == BatchArgs::PROB) ? d_idx : nullptr;
@@ -1105,9 +1310,67 @@ int run_batch(const BatchArgs& a) {
         e = launch_pairing_select(S, st);
         if (e != cudaSuccess) { ret = cuda_fail(e, "pairing choice launch"); break; }
       }
-      e = launch_pair_terms(L, st);
-      if (e != cudaSuccess) { ret = cuda_fail(e, "pair-term kernel launch"); break; }
-      if (n_items > 0) {
+      if (U.match) {
+        MatchLaunch M;
+        M.src = L.src;
+        M.idx = L.idx;
+        M.pats = d_pats;
+        M.order = (const int*)(up + U.order_at);
+        M.tiles = (const MatchTile*)(up + U.tiles_at);
+        M.skip = L.skip;
+        M.m_bound = L.m_bound;
+        M.status = d_status;
+        M.parts = d_mparts;
+        if (U.match_b) {
+          std::vector<MatchChunk> chunks;
+          match_chunks(U, d_match, &chunks);
+          for (const MatchChunk& c : chunks)
+            if ((e = launch_match_large(M, c, st)) != cudaSuccess) break;
+        }
+        if (e == cudaSuccess && U.n_tiles) e = launch_match_small(M, U.n_tiles, U.tile_smem, st);
+        if (e != cudaSuccess) { ret = cuda_fail(e, "matching kernel launch"); break; }
+        if (U.terms && n_items > 0) {
+          TermsLaunch T;
+          memset(&T, 0, sizeof(T));
+          T.src = L.src;
+          T.idx = L.idx;
+          T.pats = d_pats;
+          T.items = d_items;
+          T.n_items = (int)n_items;
+          T.batch = batch;
+          T.m_bound = L.m_bound;
+          T.perm = L.perm;
+          T.perm_off = L.perm_off;
+          T.skip = L.skip;
+          T.counter = d_ctr + 40;
+          T.status = d_status;
+          T.warp_bytes = U.tcfg.warp_bytes;
+          T.stage_h = maxn / 2;
+          T.mat = d_arena;
+          T.mat_off = (const int64_t*)(up + U.matoff_at);
+          T.sum_off = T.mat_off + batch;
+          T.exps = d_exps;
+          T.ok = d_ok;
+          T.kparts = d_kparts;
+          T.ksum = d_ksum;
+          T.n_redo = d_ctr + 41;
+          T.blocks_done = (unsigned*)(d_ctr + 42);
+          T.fp64_items = d_ctr + 43;
+          const int tw = U.tcfg.warps_per_block;
+          e = launch_terms(T, (int)std::min<int64_t>(device_sm_count(), (n_items + tw - 1) / tw), tw, st);
+          if (e != cudaSuccess) { ret = cuda_fail(e, "terms kernel launch"); break; }
+          // the matrices the fixed-point terms gave back (normally none)
+          HafLaunch L2 = L;
+          L2.skip = d_ok;
+          L2.pt = nullptr;
+          L2.pt_off = nullptr;
+          L2.n_items_dev = T.fp64_items;
+          e = launch_haf_subsets(L2, a.precision, blocks, cfg.warps_per_block, st);
+          if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
+        }
+      } else {
+        e = launch_pair_terms(L, st);
+        if (e != cudaSuccess) { ret = cuda_fail(e, "pair-term kernel launch"); break; }
         e = launch_haf_subsets(L, a.precision, blocks, cfg.warps_per_block, st);
         if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
       }
@@ -1153,7 +1416,14 @@ int run_batch(const BatchArgs& a) {
     }
     F.idx = (a.mode == BatchArgs::PROB) ? d_idx : nullptr;
     F.status = d_status;
-    if (dev_rep_cap && n_items > 0) {
+    if (U.match) {
+      F.match = d_mparts;
+      if (U.terms) {
+        F.ok = d_ok;
+        F.ksum = d_ksum;
+      }
+    }
+    if (dev_rep_cap && (n_items > 0 || U.n_order > 0)) {
       F.rep_half = d_rephalf;
       F.rep_end = d_repend;
       F.rep_parts = d_repparts;

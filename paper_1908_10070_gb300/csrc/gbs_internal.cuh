@@ -152,6 +152,55 @@ __host__ __device__ inline bool spare_tile(int N, int h, int warp_bytes, int sta
   return (32 / L) * group_bytes(N, h, cbytes, true) <= avail;
 }
 
+// ---- fixed-point terms (haf_terms.cuh): lane groups of 2 x 2 blocks ----
+__host__ __device__ inline int terms_stage_bytes(int stage_h) {
+  return stage_slots(stage_h) * stage_stride(stage_h) * 16;
+}
+// One lane group's region for subsets of s pairs of a matrix of h pairs: the
+// schedule row's matrices (s (s + 1) / 2 blocks of 64 bytes each) and the pair
+// numbers, padded so that the 8 lanes of a 16-byte access that lie in
+// different groups of fewer than 8 lanes start in different banks.
+__host__ __device__ inline int terms_group_bytes(int s, int h, int L) {
+  int units = sched_nbuf(h) * 2 * s * (s + 1) + ((s + 3) >> 2);
+  if (L < 8)
+    while ((units & 7) != L) ++units;
+  return units * 16;
+}
+// Lanes per subset of s pairs: the fewest (a power of two) whose 32 / L groups
+// fit the warp's bytes and the staging slots and are not mostly idle on the
+// C(h, s) subsets of that size; 0 if none fits.
+__host__ __device__ inline int terms_lanes(int s, int h, int warp_bytes, int stage_h) {
+  const int avail = warp_bytes - 512 - terms_stage_bytes(stage_h);
+  int c = 1;
+  for (int i = 1; i <= s; ++i) c = c * (h - s + i) / i;
+  for (int L = 32 / stage_slots(stage_h); L <= 32; L <<= 1)
+    if (32 / L < 2 * c && (32 / L) * terms_group_bytes(s, h, L) <= avail) return L;
+  return 0;
+}
+struct TermsLaunch {
+  const double* src;       // as in HafLaunch
+  const int* idx;
+  const PatDesc* pats;
+  const WorkItem* items;
+  int n_items, batch, m_bound;
+  const int* perm;
+  const int* perm_off;
+  const int* skip;         // as in HafLaunch: the repeated-row sum gives the estimate
+  int* counter;            // work-queue head, zero before launch
+  int* status;
+  int warp_bytes, stage_h;
+  int4* mat;               // limbs: per matrix its entries, and its pair sums
+  const int64_t* mat_off;  // per matrix, in int4 (-1: odd orders)
+  const int64_t* sum_off;  // -1: R_2 by the product
+  int* exps;               // kExpStride exponents per matrix
+  int* ok;                 // zero before launch; in the end 1 where the FP64 kernel has nothing to do
+  double2* kparts;         // per item: sum |f|_1 and the rounding bound
+  double* ksum;            // per matrix: sum |f|_1
+  int* n_redo;             // zero before launch
+  unsigned* blocks_done;   // zero before launch
+  int* fp64_items;         // out: items the FP64 kernel is to look at (0 or n_items)
+};
+
 struct HafLaunch {
   const double* src;       // interleaved complex source matrices
   const float* src32;      // the same rounded to float (FP32 path; may be null)
@@ -206,6 +255,12 @@ struct FinalizeLaunch {
   const int* rep_half;
   const int* rep_end;
   const Partial* rep_parts;
+  // If non-null: per matrix its Hafnian (matchings) in re_hi, im_hi; the
+  // partials of `parts` then count only for kappa, and only where ok is 0
+  // (elsewhere it is ksum, where that is given).
+  const Partial* match;
+  const int* ok;
+  const double* ksum;
   const int* batch_dev;    // if non-null, the number of entries is read here (device memory)
   const Partial* chunk_parts;  // if non-null, sum these chunk sums (chunk_off ranges) instead
   const int* chunk_off;
@@ -293,8 +348,58 @@ struct RoutePlan {
   int* n_chosen;           // zero before launch: patterns given the repeated-row sum
 };
 
+// Hafnians by partial matchings (match.cu): FP64, without the subset sum's
+// cancellation ratio. A tile is up to 2^lp matrices of one order that a block
+// holds side by side in shared memory; `even` and `odd` are the most sets an
+// even- and an odd-numbered layer of that order has.
+constexpr int kMatchMaxN = 30;       // batches with larger orders keep the subset sum
+constexpr int kMatchSmallMax = 18;   // largest order whose layers live in shared memory
+constexpr int kMatchThreads = 256;
+constexpr int kMatchTileBytes = 112 * 1024;  // two blocks an SM
+constexpr int kMatchTail = 9;        // the last layers of larger orders go back to shared memory
+struct MatchTile {
+  int n, lp, first, count;  // matrices order[first, first + count)
+  int even, odd;
+};
+struct MatchLaunch {
+  const double* src;       // interleaved complex source matrices
+  const int* idx;          // index lists (may be null when every idx_off < 0)
+  const PatDesc* pats;
+  const int* order;        // even-order matrices, by order
+  const MatchTile* tiles;
+  const int* skip;         // as in HafLaunch
+  int m_bound;             // as in HafLaunch
+  int* status;             // as in HafLaunch
+  Partial* parts;          // one per matrix
+};
+// Larger orders: the matrices of one order in a chunk. Per matrix the scratch
+// holds the packed strict upper triangle and an even and an odd layer.
+struct MatchGroup {
+  int n, first, count;     // matrices order[first, first + count)
+  int begin;               // the group's first matrix in the chunk
+  int even;                // sets of the largest even layer
+  int tasks;               // warps per matrix of one layer's launch (set by the launcher)
+  int64_t off, stride;     // complex elements in the scratch: the group's first matrix, and per matrix
+};
+constexpr int kMatchGroups = (kMatchMaxN - kMatchSmallMax) / 2;
+struct MatchChunk {
+  int n_groups;
+  double* scratch;
+  MatchGroup g[kMatchGroups];
+};
+// Most sets of an even and of an odd layer of order n, and its complex
+// multiply-adds (macs may be null).
+void match_sizes(int n, int* even, int* odd, double* macs);
+// Device scratch of one matrix of a larger order.
+size_t match_matrix_bytes(int n);
+cudaError_t launch_match_small(const MatchLaunch& L, int tiles, size_t smem, cudaStream_t st);
+cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t st);
+
 // Defined in haf_subsets.cu
 cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st);
+// The fixed-point terms: prep and pair sums, the terms, and the check.
+cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, cudaStream_t st);
+constexpr int kExpInts = 20;  // ints of TermsLaunch::exps per matrix
 cudaError_t launch_route_plan(const RoutePlan& R, cudaStream_t st);
 cudaError_t launch_haf_subsets(const HafLaunch& L, int precision, int blocks, int warps_per_block,
                                cudaStream_t st);

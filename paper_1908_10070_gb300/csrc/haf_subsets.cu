@@ -1007,6 +1007,15 @@ __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const Finalize
           const int end = F.rep_end[pb];
           sum_partials(F.rep_parts, end - (rep + kRepTermsPerItem - 1) / kRepTermsPerItem, end, lane, rh, rl,
                        ih, il, K);
+        } else if (F.match) {
+          rh = F.match[pb].re_hi;
+          ih = F.match[pb].im_hi;
+          if (F.ok != nullptr && F.ok[pb] == 0) {
+            double a = 0, b2 = 0, c2 = 0, e2 = 0;
+            sum_partials(F.parts, d.item_begin, d.item_end, lane, a, b2, c2, e2, K);
+          } else if (F.ksum != nullptr) {
+            K = F.ksum[pb];
+          }
         } else if (F.chunk_parts)
           sum_partials(F.chunk_parts, F.chunk_off[pb], F.chunk_off[pb + 1], lane, rh, rl, ih, il, K);
         else
@@ -1517,6 +1526,8 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
   }
 }
 
+#include "haf_terms.cuh"
+
 // Route choice on the device (see RoutePlan): one warp per pattern decides
 // between the subset sum and the repeated-row sum by the cost rule, then the
 // last block to finish assigns each repeated-row pattern its partial range in
@@ -1646,6 +1657,34 @@ cudaError_t launch_pair_terms(const HafLaunch& L, cudaStream_t st) {
   if (L.pt == nullptr || L.batch <= 0) return cudaSuccess;
   if (2 * L.stage_h > kMaxN) return cudaErrorInvalidValue;
   pair_terms_kernel<<<pair_terms_grid(L), 256, 0, st>>>(L);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, cudaStream_t st) {
+  static_assert(kExpInts == kExpStride, "exponent stride");
+  if (warps_per_block < 1 || warps_per_block > kMaxWarpsPerBlock) return cudaErrorInvalidValue;
+  static std::atomic<int> done[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if (!done[dev].load(std::memory_order_acquire)) {
+    cudaFuncAttributes fa;
+    e = cudaFuncGetAttributes(&fa, (const void*)haf_terms_kernel);
+    if (e != cudaSuccess) return e;
+    int optin = 0;
+    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(haf_terms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             optin - (int)fa.sharedSizeBytes);
+    if (e != cudaSuccess) return e;
+    done[dev].store(1, std::memory_order_release);
+  }
+  const int h = T.stage_h, chunks = (h * (h + 1) / 2 + kSumBlocks - 1) / kSumBlocks;
+  terms_prep_kernel<<<T.batch, 256, 0, st>>>(T);
+  if (h >= 3) terms_sums_kernel<<<(unsigned)((int64_t)T.batch * chunks), 256, 0, st>>>(T);
+  haf_terms_kernel<<<blocks, warps_per_block * 32, (size_t)warps_per_block * T.warp_bytes, st>>>(T);
+  terms_check_kernel<<<std::min((T.batch + 7) / 8, 1024), 256, 0, st>>>(T);
   return cudaGetLastError();
 }
 

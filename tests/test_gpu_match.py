@@ -1,0 +1,122 @@
+"""The FP64 batched route: Hafnians by partial matchings and the subset sum's
+terms (for kappa) in fixed point, at the sizes where they change over.
+
+Tolerances. A Hafnian by matchings is a sum of products of h = n/2 entries with
+at most n roundings on the way to each; on random matrices their effect grows
+like the square root of that: 1e-13 leaves a factor of 50 at n = 30. kappa is
+compared with the FP64 subset kernel's (gbs_hafnian_batch_noalloc, the same
+pairing for n <= 24): its Hafnian's error, kappa 2^-53 n relative, dominates:
+1e-10 as everywhere in these tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gbs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1908_10070_gb300 as g
+
+    return g
+
+
+def rand_sym(n, rng, scale=0.3):
+    A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    return scale * (A + A.T) / 2
+
+
+def haf(gbs, mats, kappa=False, noalloc=False):
+    flat, n, offs = gbs.pack_matrices(mats)
+    A = torch.from_numpy(flat).cuda()
+    out = torch.zeros(2 * len(mats), dtype=torch.float64, device="cuda")
+    kap = torch.zeros(len(mats), dtype=torch.float64, device="cuda") if kappa else None
+    (gbs.hafnian_batch_noalloc if noalloc else gbs.hafnian_batch)(A, n, offs, gbs.FP64, haf_out=out, kappa_out=kap)
+    torch.cuda.synchronize()
+    o = out.cpu().numpy()
+    return o[0::2] + 1j * o[1::2], kap.cpu().numpy() if kappa else None
+
+
+@pytest.mark.parametrize("n,count", [(2, 1), (2, 700), (4, 33), (6, 5), (10, 650), (16, 3), (16, 620), (18, 1), (18, 310),
+                                     (20, 1), (20, 3), (22, 2), (26, 1)])
+def test_matchings_match_oracle(gbs, n, count):
+    """Tiles of one and of several matrices (the last one partly filled), the
+    largest order in shared memory, the smallest ones in device memory."""
+    import oracle
+
+    rng = np.random.default_rng(n * 1000 + count)
+    mats = [rand_sym(n, rng) for _ in range(count)]
+    got, _ = haf(gbs, mats)
+    for b in sorted({0, count // 2, count - 1}):
+        ref = oracle.haf_subset(mats[b])
+        assert abs(got[b] - ref) <= 1e-13 * abs(ref), (b, got[b], ref)
+
+
+def test_matchings_ragged_batch_and_estimate_do_not_change_bits(gbs):
+    """Every order 0..30 at once, each as it is alone, and with or without kappa."""
+    rng = np.random.default_rng(7)
+    mats = [rand_sym(n, rng) for n in range(0, 31)]
+    got, _ = haf(gbs, mats)
+    with_k, kap = haf(gbs, mats, kappa=True)
+    assert np.array_equal(got, with_k)
+    assert got[0] == 1 and np.all(got[1::2] == 0) and np.all(kap[2::2] >= 1)
+    for n in (4, 18, 20, 28):
+        assert haf(gbs, [mats[n]])[0][0] == got[n]
+
+
+def scaled_rows(A, power):
+    d = np.ldexp(1.0, power * (1 - 2 * (np.arange(len(A)) % 2)))
+    return A * d[:, None] * d[None, :]
+
+
+def special(kind, n, rng):
+    A = rand_sym(n, rng)
+    if kind == "zero_row":
+        A[0, :] = A[:, 0] = 0
+    elif kind == "rows_2^15":
+        A = scaled_rows(A, 15)
+    elif kind == "rows_2^4":
+        A = scaled_rows(A, 4)
+    elif kind == "huge":
+        A = A * 1e30
+    elif kind == "tiny":
+        A = A * 1e-30
+    elif kind == "subnormal":
+        A = A * 1e-310
+    elif kind == "ones":
+        A = np.ones((n, n), complex)
+    elif kind == "permutation":
+        A = np.zeros((n, n), complex)
+        p = rng.permutation(n)
+        for i in range(0, n, 2):
+            A[p[i], p[i + 1]] = A[p[i + 1], p[i]] = 1
+    elif kind == "nan":
+        A[0, 1] = A[1, 0] = np.nan
+    elif kind == "inf":
+        A[0, 1] = A[1, 0] = np.inf
+    return A
+
+
+@pytest.mark.parametrize("kind", ["random", "zero_row", "rows_2^15", "rows_2^4", "huge", "tiny", "subnormal", "ones",
+                                  "permutation", "nan", "inf"])
+def test_terms_match_fp64_kernel(gbs, kind):
+    """kappa in fixed point against the FP64 subset kernel's, on matrices that
+    fit the fixed-point range and on ones that must be given back to it."""
+    rng = np.random.default_rng(3)
+    orders = (2, 4, 6, 8, 10, 14, 16, 18, 20, 24)
+    mats = [special(kind, n, rng) for n in orders] + [rand_sym(16, rng)]
+    h1, k1 = haf(gbs, mats, kappa=True)
+    h0, k0 = haf(gbs, mats, kappa=True, noalloc=True)
+    for a, b, ka, kb, n in zip(h1, h0, k1, k0, list(orders) + [16]):
+        if not np.isfinite(b):
+            assert not np.isfinite(a), (n, a, b)
+            continue
+        if abs(b) == 0 or not np.isfinite(kb) or abs(a) == 0:
+            # a zero Hafnian: the subset sum leaves rounding or zero there
+            assert abs(a) <= 1e-10 * max(1.0, abs(b)) or kb > 1e10, (n, a, b)
+            continue
+        if kb < 1e6:
+            assert abs(a - b) <= 1e-10 * abs(b) and abs(ka - kb) <= 1e-10 * kb, (n, a, b, ka, kb)
