@@ -120,3 +120,21 @@ def test_terms_match_fp64_kernel(gbs, kind):
             continue
         if kb < 1e6:
             assert abs(a - b) <= 1e-10 * abs(b) and abs(ka - kb) <= 1e-10 * kb, (n, a, b, ka, kb)
+
+
+@pytest.mark.parametrize("m,n,k", [(9, 14, 11), (9, 14, 12), (7, 14, 13), (6, 16, 14), (6, 16, 15), (5, 20, 17), (5, 20, 18),
+                                   (5, 20, 19)])
+def test_marginals_sum_across_prefix_lengths(gbs, m, n, k):
+    """sum_l q(x_1..x_k, l) = q(x_1..x_k): the tables in shared memory (up to 12
+    photons), in device memory, and the sets taken one by one near k = n, with
+    repeated modes. q is a sum of positive terms of about n roundings each:
+    1e-12 leaves a factor of 100."""
+    import workloads as W
+
+    K = gbs.build_kernel(W.haar_unitary(m, 17 * m + n), np.full(m, 0.7))
+    x = np.random.default_rng(n * k).integers(0, m, size=(3, k)).astype(np.int32)
+    whole = gbs.marginal_batch(K, x, n)
+    ext = np.repeat(x, m, axis=0)
+    ext = np.hstack([ext, np.tile(np.arange(m, dtype=np.int32), 3)[:, None]])
+    parts = gbs.marginal_batch(K, ext, n).reshape(3, m).sum(1)
+    assert np.all(whole > 0) and np.all(np.abs(parts - whole) <= 1e-12 * whole), (whole, parts)
