@@ -249,7 +249,6 @@ bool shape_fits(int precision, int warp_bytes, int maxn) {
 // more than 6 fit. Rounds per item 1 / 2 / 4 / 8: 3.57 / 3.41 / 3.36 / 3.36 ms
 // and 77.7 / 62.3 / 54.9 / 52.1 ms (few subsets in an item leave the series,
 // one lane per subset, mostly idle); small batches halve them as needed.
-constexpr int kTermsWarps = 10;
 static TuneCfg terms_cfg(int n) {
   static const int optin = [] {  // thread-safe one-time initialisation
     int dev = 0, v = 0;

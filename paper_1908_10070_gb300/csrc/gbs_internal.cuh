@@ -177,6 +177,7 @@ __host__ __device__ inline int terms_lanes(int s, int h, int warp_bytes, int sta
     if (32 / L < 2 * c && (32 / L) * terms_group_bytes(s, h, L) <= avail) return L;
   return 0;
 }
+constexpr int kTermsWarps = 10;  // most warps in a block (one block per SM); 204 registers a thread
 struct TermsLaunch {
   const double* src;       // as in HafLaunch
   const int* idx;

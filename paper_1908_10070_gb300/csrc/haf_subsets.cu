@@ -1662,7 +1662,7 @@ cudaError_t launch_pair_terms(const HafLaunch& L, cudaStream_t st) {
 
 cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, cudaStream_t st) {
   static_assert(kExpInts == kExpStride, "exponent stride");
-  if (warps_per_block < 1 || warps_per_block > kMaxWarpsPerBlock) return cudaErrorInvalidValue;
+  if (warps_per_block < 1 || warps_per_block > kTermsWarps) return cudaErrorInvalidValue;
   static std::atomic<int> done[64];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);

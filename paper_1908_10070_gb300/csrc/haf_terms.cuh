@@ -71,19 +71,19 @@ __device__ __forceinline__ int2 fx_pack(int hi, float lo, bool& over) {
   over |= (unsigned)(hi + (1 << kFxBits)) > (2u << kFxBits);
   return make_int2(hi, __float_as_int(lo - (q - 12582912.0f)));
 }
-// (h + 64 m) 2^-sh, 18 <= sh <= 32.
+// (h + 64 m) 2^-sh, 18 <= sh <= 31 (so h 2^-sh is below 2^44).
 __device__ __forceinline__ int2 fx_round(long long h, float m, int sh, bool& over) {
-  const long long top = (h + (1ll << (sh - 1))) >> sh;
-  over |= (unsigned long long)(top + (1ll << 28)) > (1ull << 29) || !(fabsf(m) < 0x1p30f);
+  const long long top = h >> sh;
+  over |= (unsigned)((int)(top >> 28) + 1) > 1u || !(fabsf(m) < 0x1p30f);
   const float unit = __int_as_float((127 - sh) << 23);
-  const float lo = (float)(int)(h - (top << sh)) * unit + m * (64.0f * unit);
+  const float lo = (float)((unsigned)h & ((1u << sh) - 1)) * unit + m * (64.0f * unit);
   return fx_pack((int)top, lo, over);
 }
 __device__ __forceinline__ int4 fx_entry(const Fx& c, int sh, bool& over) {
   const int2 x = fx_round(c.rh, c.rm, sh, over), y = fx_round(c.ih, c.im, sh, over);
   return make_int4(x.x, y.x, x.y, y.y);
 }
-__device__ __forceinline__ bool fx_shift_ok(int sh) { return sh >= 18 && sh <= 32; }
+__device__ __forceinline__ bool fx_shift_ok(int sh) { return sh >= 18 && sh <= 31; }
 
 // A symmetric matrix of s pairs as 2 x 2 blocks of its upper block triangle:
 // block (r, c), r < c, is number c(c-1)/2 + r, block (r, r) number
@@ -368,8 +368,15 @@ __device__ __forceinline__ longlong2 fx_tr1(const int4* __restrict__ Ra, int s, 
 }
 
 // Persistent warps over work items (as haf_subsets_kernel): a warp takes
-// 32 / L subsets of one size at a time, L lanes each.
-__global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) haf_terms_kernel(const TermsLaunch P) {
+// 32 / L subsets of one size at a time, L lanes each. Six to ten warps an SM
+// (shared memory sets the number) leave latency in sight, so loads are issued
+// ahead of their use and sums run two at a time. 4096 patterns of n = 16: this
+// kernel 2.66 -> 2.35 ms (with one load in flight, each trace summed alone);
+// with every part timed by leaving it out, products take 1.1 ms of it, their
+// rounding a third of that, traces and loads 0.6, the series 0.3, the sums over
+// lanes 0.3 (before the pairing). 80 patterns of n = 28 and 30: products 22 of
+// 40 ms, at six warps an SM.
+__global__ void __launch_bounds__(kTermsWarps * 32, 1) haf_terms_kernel(const TermsLaunch P) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Tables tab;
   __shared__ unsigned short rc[kMaxH * (kMaxH - 1) / 2];
@@ -516,29 +523,48 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) haf_terms_kernel(co
         // R_1 (and R_2 from the pair sums): the subset's blocks
         const bool have2 = sums != nullptr && h >= 3;
         const int klo = (int)(gmask & ((1u << hl) - 1)), khi = (1 << hl) + (int)(gmask >> hl);
-        for (int f = l; f < 4 * E; f += L) {
-          const int e = f >> 2, el = f & 3;
-          int r, c;
-          if (e >= D) {
-            r = c = e - D;
-          } else {
-            const int v = rc[e];
-            r = v & 255;
-            c = v >> 8;
+        // (the loads of four entries are issued before the first is used)
+        for (int f0 = l; f0 < 4 * E; f0 += 4 * L) {
+          int4 v[4], x[4], y[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int f = f0 + u * L, e = f >> 2, el = f & 3;
+            if (f < 4 * E) {
+              int r, c;
+              if (e >= D) {
+                r = c = e - D;
+              } else {
+                const int z = rc[e];
+                r = z & 255;
+                c = z >> 8;
+              }
+              const int src = blk_index(pairs[r], pairs[c], h);
+              v[u] = __ldg(mat + 4 * src + el);
+              if (have2) {
+                const int4* q = sums + ((int64_t)src * W) * 4 + el;
+                x[u] = __ldg(q + 4 * klo);
+                y[u] = __ldg(q + 4 * khi);
+              }
+            }
           }
-          const int src = blk_index(pairs[r], pairs[c], h);
-          buf[el * E + e] = __ldg(mat + 4 * src + el);
-          if (have2) {
-            const int4* q = sums + ((int64_t)src * W) * 4 + el;
-            const int4 x = __ldg(q + 4 * klo), y = __ldg(q + 4 * khi);
-            const int2 re = fx_pack(x.x + y.x, __int_as_float(x.z) + __int_as_float(y.z), over);
-            const int2 im = fx_pack(x.y + y.y, __int_as_float(x.w) + __int_as_float(y.w), over);
-            buf[4 * E + el * E + e] = make_int4(re.x, im.x, re.y, im.y);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int f = f0 + u * L, e = f >> 2, el = f & 3;
+            if (f < 4 * E) {
+              buf[el * E + e] = v[u];
+              if (have2) {
+                const int2 re = fx_pack(x[u].x + y[u].x, __int_as_float(x[u].z) + __int_as_float(y[u].z), over);
+                const int2 im = fx_pack(x[u].y + y[u].y, __int_as_float(x[u].w) + __int_as_float(y[u].w), over);
+                buf[4 * E + el * E + e] = make_int4(re.x, im.x, re.y, im.y);
+              }
+            }
           }
         }
         __syncwarp();
         longlong2* const row = stage + (staged + g) * sts;
         unsigned pw = 1;
+        longlong2 wait = make_longlong2(0, 0);
+        int wait_k = 0;  // 0: none waiting
         for (int o = 0; o < kMaxOps; ++o) {
           const SchedOp op = c_sched[h][o];
           if (op.kind == kEnd) break;
@@ -550,13 +576,38 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 1) haf_terms_kernel(co
               fx_prod(buf + op.k * 4 * E, Ra, Rb, rc, s, E, 27 + ex[ka + kb] - ex[ka] - ex[kb], l, L, over);
             pw = (pw & ~(15u << (4 * op.k))) | (unsigned)(ka + kb) << (4 * op.k);
           } else {
-            longlong2 t = (op.kind == kTr1) ? fx_tr1(Ra, s, E, l, L) : fx_tr2(Ra, Rb, s, E, l, L);
-            for (int off = L >> 1; off > 0; off >>= 1) {
-              t.x += __shfl_xor_sync(FULL, t.x, off);
-              t.y += __shfl_xor_sync(FULL, t.y, off);
+            // the lanes' shares are summed two traces at a time, as group_sum2
+            // does (half the lanes carry one, half the other); they are whole
+            // numbers, so the order does not matter
+            const longlong2 t = (op.kind == kTr1) ? fx_tr1(Ra, s, E, l, L) : fx_tr2(Ra, Rb, s, E, l, L);
+            if (L == 1) {
+              row[op.k - 1] = active ? t : make_longlong2(0, 0);
+            } else if (wait_k == 0) {
+              wait = t;
+              wait_k = op.k;
+            } else {
+              const int half = L >> 1;
+              const bool up = (l & half) != 0;
+              const longlong2 out = up ? wait : t;
+              longlong2 keep = up ? t : wait;
+              keep.x += __shfl_xor_sync(FULL, out.x, half);
+              keep.y += __shfl_xor_sync(FULL, out.y, half);
+              for (int off = half >> 1; off > 0; off >>= 1) {
+                keep.x += __shfl_xor_sync(FULL, keep.x, off);
+                keep.y += __shfl_xor_sync(FULL, keep.y, off);
+              }
+              if ((l & (half - 1)) == 0) row[(up ? op.k : wait_k) - 1] = active ? keep : make_longlong2(0, 0);
+              wait_k = 0;
             }
-            if (l == 0) row[op.k - 1] = active ? t : make_longlong2(0, 0);
           }
+          __syncwarp();
+        }
+        if (wait_k != 0) {  // uniform over the warp
+          for (int off = L >> 1; off > 0; off >>= 1) {
+            wait.x += __shfl_xor_sync(FULL, wait.x, off);
+            wait.y += __shfl_xor_sync(FULL, wait.y, off);
+          }
+          if (l == 0) row[wait_k - 1] = active ? wait : make_longlong2(0, 0);
           __syncwarp();
         }
         staged += G;
