@@ -70,31 +70,54 @@ __global__ void enumerate_kernel(int m, int n, int64_t first, int64_t count,
   }
 }
 
-// Inclusive prefix sum of count doubles in a fixed order (one block): thread
-// t sums its contiguous chunk, the chunk totals are scanned by thread 0, and
-// each thread rescans its chunk from its offset. Deterministic.
-__global__ void prefix_kernel(const double* __restrict__ p, int64_t count, double* __restrict__ cum) {
-  __shared__ double tot[1024];
-  const int T = blockDim.x;
-  const int64_t chunk = (count + T - 1) / T;
-  const int64_t lo = threadIdx.x * chunk, hi = min(count, lo + chunk);
-  double s = 0.0;
-  for (int64_t i = lo; i < hi; ++i) s += p[i];
-  tot[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double run = 0.0;
-    for (int i = 0; i < T; ++i) {
-      const double v = tot[i];
-      tot[i] = run;
-      run += v;
+// Inclusive prefix sum of count doubles in a fixed order (one block), in tiles
+// of 8 consecutive values a thread: a thread's own running sums, the threads'
+// totals by a scan over the warp and over the warps, and the running total of
+// the tiles before. Deterministic. (Thread 0 joining 1024 totals one by one
+// took 60 us at 3876 values, three quarters of it that loop; this takes a
+// fixed number of steps per 8192 values.)
+constexpr int kScanPer = 8;
+__global__ void __launch_bounds__(1024) prefix_kernel(const double* __restrict__ p, int64_t count,
+                                                      double* __restrict__ cum) {
+  __shared__ double warp_tot[32];
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  double before = 0.0;
+  for (int64_t base = 0; base < count; base += (int64_t)blockDim.x * kScanPer) {
+    const int64_t lo = base + (int64_t)threadIdx.x * kScanPer;
+    double v[kScanPer];
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < kScanPer; ++i) v[i] = (lo + i < count) ? p[lo + i] : 0.0;
+#pragma unroll
+    for (int i = 0; i < kScanPer; ++i) {
+      s += v[i];
+      v[i] = s;
     }
-  }
-  __syncthreads();
-  double run = tot[threadIdx.x];
-  for (int64_t i = lo; i < hi; ++i) {
-    run += p[i];
-    cum[i] = run;
+    double inc = s;
+    for (int off = 1; off < 32; off <<= 1) {
+      const double t = __shfl_up_sync(FULL, inc, off);
+      if (lane >= off) inc += t;
+    }
+    if (lane == 31) warp_tot[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      double t = (lane < nw) ? warp_tot[lane] : 0.0;
+      for (int off = 1; off < 32; off <<= 1) {
+        const double x = __shfl_up_sync(FULL, t, off);
+        if (lane >= off) t += x;
+      }
+      warp_tot[lane] = t;
+    }
+    __syncthreads();
+    double run = __shfl_up_sync(FULL, inc, 1);
+    if (lane == 0) run = 0.0;
+    run += before + (warp > 0 ? warp_tot[warp - 1] : 0.0);
+#pragma unroll
+    for (int i = 0; i < kScanPer; ++i)
+      if (lo + i < count) cum[lo + i] = run + v[i];
+    before += warp_tot[nw - 1];
+    __syncthreads();
   }
 }
 
