@@ -368,9 +368,11 @@ __global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, Subse
 //   sum_T w(T) c_k(|T| + 1) |sum_i b_i h_i|^2 = b* M b,
 //   M_ij = sum_{T holds i, j} w(T) c_k(|T| + 1) conj(h_i) h_j,
 // and M serves every candidate of the sample: k^2 / 2 products a candidate
-// instead of up to k 2^(k-2). The at most k - 1 modes that are in the prefix
-// have other weights (one copy more) and get their sums one by one, as all
-// candidates do on the last steps, where the sets are few. The sets without
+// instead of up to k 2^(k-2). A mode in the prefix has one copy more, and with
+// it a larger weight on the sets that do not hold all its positions: what it
+// has more there (every term positive) is summed apart, for at most k - 1
+// modes. On the last step, with one set, all candidates are summed one by one.
+// The sets without
 // the new photon count 1 + (multiplicity of l in the prefix) times:
 // (a+1)! C(m+1, a+1) = (m+1) a! C(m, a). 64 samples of 16 photons over 256
 // modes: 9.56 ms (every candidate's table and sums over subsets) -> 0.80 ms.
@@ -380,6 +382,7 @@ struct ChainStep {
   SubsetClasses rho;         // sets of the prefix that count (even)
   SubsetClasses odd;         // sets T of the prefix with c_k(|T| + 1) in range
   SubsetClasses pair, diag;  // T without two (one) of its positions, over the other kp - 2 (kp - 1)
+  SubsetClasses miss;        // sets T that do not hold one given position, over the other kp - 1
   SubsetClasses grow;        // odd sets whose union with the new photon a later step reads
   int n_pair, c_pair, c_own, c_rho;  // position pairs i <= j; warps of each, of a prefix mode, of the rho sum
   int tasks;                 // warps per sample
@@ -394,9 +397,11 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// One warp per task of sample blockIdx.y: a chunk of M_ij, of the sum of one
-// prefix mode (that of position t, by its first position; 0 for others) or of
-// the sum over rho. part[sample * tasks + task].
+// One warp per task of sample blockIdx.y: a chunk of M_ij, of what one prefix
+// mode has more (that of position t, by its first position; 0 for others) or
+// of the sum over rho. part[sample * tasks + task]. A mode held once (the
+// common case) has weight 2 instead of 1 on the sets without its position, so
+// half the sets are enough for it; a repeated one goes through all of them.
 __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, const double2* __restrict__ cache,
                                                                   int64_t cstride, const double2* __restrict__ B,
                                                                   const int* __restrict__ x,
@@ -453,12 +458,16 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
       for (int i = 0; i < R.n; ++i)
         if (R.mode[i] == v) extra = i;
       const double2* row = B + (int64_t)v * S.m;
-      const int end = (int)min(S.odd.total(), (int64_t)c0 + kOwnChunk);
+      const int end = (int)min(extra < 0 ? S.miss.total() : S.odd.total(), (int64_t)c0 + kOwnChunk);
       for (int r = c0 + lane; r < end; r += 32) {
-        const int T = subset_of(S.odd, r, binom);
+        const int T = extra < 0 ? open_bit(subset_of(S.miss, r, binom), p) : subset_of(S.odd, r, binom);
+        double w = weight(T, __popc(T) + 1);
+        if (extra >= 0) {  // (m + 1) / (m + 1 - alpha) times as much, alpha of m copies outside T
+          const int mv = R.mult[extra], al = mv - __popc(T & R.mask[extra]);
+          if (al == 0) continue;
+          w = weight(T, __popc(T) + 1, extra) - w;
+        }
         const double2 h = expand(H, T, [&](int i) { return __ldg(row + xs[i]); });
-        double w = weight(T, __popc(T) + 1, extra);
-        if (extra < 0 && !(T >> p & 1)) w *= 2.0;  // held once: C(2, 1)
         re = fma(w, h.x * h.x + h.y * h.y, re);
       }
     }
@@ -536,9 +545,8 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
       if (mult == 1 && !(T >> first & 1)) w *= 2.0;
       s = fma(w, h.x * h.x + h.y * h.y, s);
     }
-  } else if (mult > 0) {
-    s = own[first];
   } else {
+    if (mult > 0) s = own[first];
     for (int i = 0; i < S.kp; ++i) {
       const double2 bi = b[i][threadIdx.x];
       double2 y = make_double2(0.0, 0.0);  // sum_{j > i} M_ij b_j
@@ -633,6 +641,7 @@ ChainStep chain_step(int k, int n, int m, unsigned later) {
   S.odd = subset_classes(S.kp, sizes, 1);
   S.pair = subset_classes(std::max(S.kp - 2, 0), S.kp >= 2 ? sizes : 0, 3);
   S.diag = subset_classes(std::max(S.kp - 1, 0), S.kp >= 1 ? sizes : 0, 2);
+  S.miss = S.kp >= 1 ? subset_classes(S.kp - 1, sizes, 1) : SubsetClasses();
   S.grow = subset_classes(S.kp, later, 1);
   // a candidate costs kp products per set one by one and kp / 2 per position by
   // the form (at k = n there is one set; at k = n - 1 of 16, 14 sets one by one
@@ -851,7 +860,7 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
       chain_weight_kernel<<<dim3((m + kWeightThreads - 1) / kWeightThreads, S), kWeightThreads, 0, st>>>(
           C, d_cache, cstride, B, d_x, d_c, d_part, d_q);
       // the draws, then the chosen modes' new sub-Hafnians into the caches
-      const int nb = kk < n ? (int)std::max<int64_t>(1, std::min<int64_t>(64, (C.grow.total() + 511) / 512)) : 1;
+      const int nb = kk < n ? (int)std::max<int64_t>(1, std::min<int64_t>(64, (C.grow.total() + 255) / 256)) : 1;
       chain_pick_kernel<<<dim3(nb, S), kMargThreads, 0, st>>>(C, d_q, d_u, d_x, d_cache, cstride, B);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) {
