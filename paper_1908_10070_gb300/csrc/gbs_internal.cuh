@@ -8,6 +8,39 @@
 
 namespace gbs {
 
+// Dependent launches: a kernel launched by launch_dependent may be set up, and
+// run up to dependency_wait(), while the blocks of the kernel before it in the
+// stream leave; the wait ends when that one has finished (each waits for its
+// own predecessor, so for all before it). Kernels call dependency_wait()
+// before they read or write anything another kernel touches; tables in
+// constant initialised memory may be copied earlier. It returns at once after
+// an ordinary launch. In calls of many short kernels this takes 2 us off a
+// launch: 64 chain samples of 16 photons (50 launches) 716 -> 616 us, 301
+// matrices of n <= 22 (16) 154 -> 127, one 16-photon pattern 141 -> 126. No
+// kernel asks for its successor early: blocks that wait then hold shared
+// memory which the running kernels need (4096 patterns of n = 16: 4.46 ms
+// instead of 2.85).
+__device__ __forceinline__ void dependency_wait() {
+#if defined(__CUDA_ARCH__)
+  cudaGridDependencySynchronize();
+#endif
+}
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                    const A&... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // One matrix of a batch: the n x n matrix whose (i, j) entry is
 // src[src_off + row(i) * ld + row(j)], row(i) = idx[idx_off + i] (or i when
 // idx_off < 0). For probabilities src is B and the rows are the pattern's mode

@@ -981,6 +981,7 @@ constexpr int kFinWarps = 16;  // most warps in a finalisation block
 __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const FinalizeLaunch F) {
   __shared__ double sv[6][kFinWarps];  // re hi/lo, im hi/lo, sum |f|, prod s_j!
   __shared__ int sbad[kFinWarps];     // status flag of the pattern
+  dependency_wait();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wpb = blockDim.x >> 5;
@@ -1432,6 +1433,7 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
   extern __shared__ __align__(16) unsigned char rep_smem[];
   RepWarp* ws = reinterpret_cast<RepWarp*>(rep_smem);
   __shared__ int binom[kMaxN + 1][kMaxN + 1];
+  dependency_wait();
   // the grid covers the reservation; with no item (no bunched pattern) every
   // block leaves before building its table (uniform over the block)
   const int n_items = min(*R.n_items_dev, R.n_items);
@@ -1533,6 +1535,7 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
 // last block to finish assigns each repeated-row pattern its partial range in
 // pattern order (a block-wide prefix sum over tiles of the batch).
 __global__ void __launch_bounds__(256) route_plan_kernel(const RoutePlan R) {
+  dependency_wait();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   for (int b = blockIdx.x * wpb + warp; b < R.batch; b += gridDim.x * wpb) {
@@ -1643,8 +1646,7 @@ cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st) {
   int blocks = (R.n_items + 3) / 4;
   const int cap = (sms > 0 ? sms : 1) * (int)std::min<size_t>(8, (size_t)220 * 1024 / smem);
   if (blocks > cap) blocks = cap;
-  haf_repeated_kernel<<<blocks, 128, smem, st>>>(R);
-  return cudaGetLastError();
+  return launch_dependent(haf_repeated_kernel, dim3(blocks), 128, smem, st, R);
 }
 
 cudaError_t launch_pairing_select(const PairingSelect& S, cudaStream_t st) {
@@ -1681,11 +1683,14 @@ cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, 
     done[dev].store(1, std::memory_order_release);
   }
   const int h = T.stage_h, chunks = (h * (h + 1) / 2 + kSumBlocks - 1) / kSumBlocks;
-  terms_prep_kernel<<<T.batch, 256, 0, st>>>(T);
-  if (h >= 3) terms_sums_kernel<<<(unsigned)((int64_t)T.batch * chunks), 256, 0, st>>>(T);
-  haf_terms_kernel<<<blocks, warps_per_block * 32, (size_t)warps_per_block * T.warp_bytes, st>>>(T);
-  terms_check_kernel<<<std::min((T.batch + 7) / 8, 1024), 256, 0, st>>>(T);
-  return cudaGetLastError();
+  e = launch_dependent(terms_prep_kernel, dim3(T.batch), 256, 0, st, T);
+  if (e == cudaSuccess && h >= 3)
+    e = launch_dependent(terms_sums_kernel, dim3((unsigned)((int64_t)T.batch * chunks)), 256, 0, st, T);
+  if (e == cudaSuccess)
+    e = launch_dependent(haf_terms_kernel, dim3(blocks), warps_per_block * 32, (size_t)warps_per_block * T.warp_bytes, st,
+                         T);
+  if (e == cudaSuccess) e = launch_dependent(terms_check_kernel, dim3(std::min((T.batch + 7) / 8, 1024)), 256, 0, st, T);
+  return e;
 }
 
 // Raise the kernel's dynamic shared-memory limit to the device maximum once
@@ -1774,8 +1779,7 @@ cudaError_t launch_finalize(const FinalizeLaunch& F, cudaStream_t st) {
   const int threads = kFinWarps * 32;  // one warp per pattern
   int blocks = (F.batch + kFinWarps - 1) / kFinWarps;
   if (blocks > 8192) blocks = 8192;
-  finalize_kernel<<<blocks, threads, 0, st>>>(F);
-  return cudaGetLastError();
+  return launch_dependent(finalize_kernel, dim3(blocks), threads, 0, st, F);
 }
 
 }  // namespace gbs

@@ -100,6 +100,7 @@ __device__ __forceinline__ int blk_index(int r, int c, int s) {
 __global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P) {
   __shared__ float2 A[kMaxN * kMaxN], R[kMaxN * kMaxN];
   __shared__ int rows[kMaxN], s_max[kMaxN / 2 + 1], s_lo, s_bad;
+  dependency_wait();
   const int b = blockIdx.x;
   const PatDesc d = P.pats[b];
   const int n = d.n, h = n >> 1;
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P) {
 // the low and of the high pairs.
 __global__ void __launch_bounds__(256) terms_sums_kernel(const TermsLaunch P) {
   __shared__ int4 Q[kSumBlocks * 4 * kMaxH];
+  dependency_wait();
   const int hm = P.stage_h, chunks = (hm * (hm + 1) / 2 + kSumBlocks - 1) / kSumBlocks;
   const int b = blockIdx.x / chunks, b0 = (blockIdx.x - b * chunks) * kSumBlocks;
   const int n = P.pats[b].n, h = n >> 1, nb = h * (h + 1) / 2;
@@ -390,6 +392,7 @@ __global__ void __launch_bounds__(kTermsWarps * 32, 1) haf_terms_kernel(const Te
     tab.inv2k[a] = (a == 0) ? 0.0 : 1.0 / (2.0 * a);
     for (int r = 0; r < a && a < kMaxH; ++r) rc[a * (a - 1) / 2 + r] = (unsigned short)(r | (a << 8));
   }
+  dependency_wait();
   __syncthreads();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -627,6 +630,7 @@ __global__ void __launch_bounds__(kTermsWarps * 32, 1) haf_terms_kernel(const Te
 // or whose rounding bound is above 2^-33 of the sum, goes to the FP64 kernel,
 // whose item count the last block sets (0 where no matrix does).
 __global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P) {
+  dependency_wait();
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
   bool redo = false;
   for (int b = blockIdx.x * wpb + (threadIdx.x >> 5); b < P.batch; b += gridDim.x * wpb) {

@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, con
   __shared__ double red[kMargThreads];
   double2* H = reinterpret_cast<double2*>(smem);
   load_binom(binom, kMaxK);
+  dependency_wait();
   if (threadIdx.x < k) xs[threadIdx.x] = x[(int64_t)blockIdx.x * k + threadIdx.x];
   if (threadIdx.x == 0) H[0] = make_double2(1.0, 0.0);
   __syncthreads();
@@ -413,6 +414,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
   __shared__ double coef[kCoefs];
   const int smp = blockIdx.y, lane = threadIdx.x & 31;
   load_binom(binom, kMaxK);
+  dependency_wait();
   if (threadIdx.x < S.kp) xs[threadIdx.x] = x[(int64_t)smp * kMaxK + threadIdx.x];
   if (threadIdx.x < kCoefs) coef[threadIdx.x] = 2 * threadIdx.x <= S.k ? coefs[(int64_t)S.k * kCoefs + threadIdx.x] : 0.0;
   __syncthreads();
@@ -501,8 +503,9 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
   __shared__ double coef[kCoefs];
   const int smp = blockIdx.y, l = blockIdx.x * kWeightThreads + threadIdx.x;
   const double2* ps = part + (int64_t)smp * S.tasks;
+  if (S.direct) load_binom(binom, kMaxK);
+  dependency_wait();
   if (S.direct) {
-    load_binom(binom, kMaxK);
     if (threadIdx.x < kCoefs) coef[threadIdx.x] = 2 * threadIdx.x <= S.k ? coefs[(int64_t)S.k * kCoefs + threadIdx.x] : 0.0;
   }
   if (threadIdx.x < S.kp) xs[threadIdx.x] = x[(int64_t)smp * kMaxK + threadIdx.x];
@@ -572,18 +575,26 @@ __global__ void chain_init_kernel(double2* __restrict__ cache, int64_t cstride, 
 // exceeds u_k times the total (m - 1 if there is none); block 0 writes it. The
 // update: the sets of x_k with the odd T' that later steps read.
 //   u: n uniforms per sample; x: kMaxK sampled modes per sample.
+constexpr int kPickModes = 2048;
 __global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, const double* __restrict__ q,
                                                                   const double* __restrict__ u, int* __restrict__ x,
                                                                   double2* __restrict__ cache, int64_t cstride,
                                                                   const double2* __restrict__ B) {
   __shared__ int s_pick;
   __shared__ int binom[kMaxK + 1][kMaxK + 1], xs[kMaxK];
+  __shared__ double s_q[kPickModes];  // the weights, where they fit
   const int smp = blockIdx.y, m = S.m;
   if (S.k < S.n) load_binom(binom, kMaxK);
+  dependency_wait();
   if (threadIdx.x < S.kp) xs[threadIdx.x] = x[(int64_t)smp * kMaxK + threadIdx.x];
+  const bool fits = m <= kPickModes;
+  if (fits) {
+    for (int l = threadIdx.x; l < m; l += blockDim.x) s_q[l] = q[(int64_t)smp * m + l];
+    __syncthreads();
+  }
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
-    const double* qs = q + (int64_t)smp * m;
+    const double* qs = fits ? s_q : q + (int64_t)smp * m;
     const int per = (m + 31) / 32, lo = min(m, lane * per), hi = min(m, lo + per);
     double part = 0.0;
     for (int l = lo; l < hi; ++l) part += qs[l];
@@ -725,8 +736,9 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
     coef_kernel<<<1, kMargThreads, 0, st>>>(kk, n, k->m, size_scale(k->t_uniform), d_c);
     double* qd = q_dev ? q_out : d_q;
     if (small) {
-      marginal_small_kernel<<<batch, kMargThreads, 16 * ((size_t)1 << std::max(kk - 1, 0)), st>>>(kk, B, k->m, d_x, sizes,
-                                                                                                 coef, qd);
+      e = launch_dependent(marginal_small_kernel, dim3(batch), kMargThreads, 16 * ((size_t)1 << std::max(kk - 1, 0)), st, kk,
+                           B, k->m, d_x, sizes, coef, qd);
+      if (e != cudaSuccess) { ret = cuda_fail(e, "marginal kernel"); break; }
     } else {
       std::vector<int> idx, nv;
       std::vector<int64_t> offs;
@@ -855,15 +867,18 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
     for (int kk = 1; kk <= n; ++kk) {
       const ChainStep& C = steps[kk];
       constexpr int wpb = kMargThreads / 32;
-      chain_gram_kernel<<<dim3((C.tasks + wpb - 1) / wpb, S), kMargThreads, 0, st>>>(C, d_cache, cstride, B, d_x, d_c,
-                                                                                     d_part);
-      chain_weight_kernel<<<dim3((m + kWeightThreads - 1) / kWeightThreads, S), kWeightThreads, 0, st>>>(
-          C, d_cache, cstride, B, d_x, d_c, d_part, d_q);
+      e = launch_dependent(chain_gram_kernel, dim3((C.tasks + wpb - 1) / wpb, S), kMargThreads, 0, st, C, d_cache, cstride,
+                           B, d_x, d_c, d_part);
+      if (e == cudaSuccess)
+        e = launch_dependent(chain_weight_kernel, dim3((m + kWeightThreads - 1) / kWeightThreads, S), kWeightThreads, 0, st,
+                             C, d_cache, cstride, B, d_x, d_c, d_part, d_q);
       // the draws, then the chosen modes' new sub-Hafnians into the caches
       const int nb = kk < n ? (int)std::max<int64_t>(1, std::min<int64_t>(64, (C.grow.total() + 255) / 256)) : 1;
-      chain_pick_kernel<<<dim3(nb, S), kMargThreads, 0, st>>>(C, d_q, d_u, d_x, d_cache, cstride, B);
+      if (e == cudaSuccess)
+        e = launch_dependent(chain_pick_kernel, dim3(nb, S), kMargThreads, 0, st, C, d_q, d_u, d_x, d_cache, cstride, B);
+      if (e != cudaSuccess) break;
     }
-    if ((e = cudaGetLastError()) != cudaSuccess) {
+    if (e != cudaSuccess) {
       ret = cuda_fail(e, "chain kernels");
       break;
     }

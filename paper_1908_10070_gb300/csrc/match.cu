@@ -181,6 +181,7 @@ __global__ void __launch_bounds__(kMatchThreads) match_small_kernel(const MatchL
   const int n = T.n, lp = T.lp, P = 1 << lp;
   if (threadIdx.x == 0) s_any = (L.skip == nullptr);
   load_binom(bin);
+  dependency_wait();
   __syncthreads();
   layer_bases(bin, lb, n);
   for (int t = threadIdx.x; t < n << lp; t += blockDim.x) {
@@ -225,6 +226,7 @@ __global__ void __launch_bounds__(kMatchThreads) match_small_kernel(const MatchL
 __global__ void __launch_bounds__(kMatchThreads) match_head_kernel(const MatchLaunch L, const MatchChunk C) {
   __shared__ int rows[kMaxN];
   __shared__ double2 A[kMaxN * (kMaxN - 1) / 2];
+  dependency_wait();
   int g = 0;
   while (g + 1 < C.n_groups && (int)blockIdx.x >= C.g[g + 1].begin) ++g;
   const MatchGroup G = C.g[g];
@@ -268,6 +270,7 @@ __global__ void __launch_bounds__(kMatchThreads) match_head_kernel(const MatchLa
 __global__ void __launch_bounds__(kMatchThreads) match_layer_kernel(const MatchLaunch L, const MatchChunk C, int i) {
   __shared__ int bin[kBinRows * kBinCols];
   load_binom(bin);
+  dependency_wait();
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int nw = gridDim.x * (blockDim.x >> 5);
@@ -313,6 +316,8 @@ __global__ void __launch_bounds__(kMatchThreads) match_tail_kernel(const MatchLa
   __shared__ int bin[kBinRows * kBinCols];
   __shared__ int lb[kMaxN + 1][kMaxN / 2 + 2];
   __shared__ double2 buf[2][1 << (kMatchTail - 1)];
+  load_binom(bin);
+  dependency_wait();
   int g = 0;
   while (g + 1 < C.n_groups && (int)blockIdx.x >= C.g[g + 1].begin) ++g;
   const MatchGroup G = C.g[g];
@@ -322,7 +327,6 @@ __global__ void __launch_bounds__(kMatchThreads) match_tail_kernel(const MatchLa
   const double2* even = A + n * (n - 1) / 2;
   const int i0 = n - kMatchTail;
   const double2* in = (i0 & 1) ? even + G.even : even;
-  load_binom(bin);
   for (int e = threadIdx.x; e < 1 << (kMatchTail - 1); e += blockDim.x) buf[i0 & 1][e] = in[e];
   __syncthreads();
   layer_bases(bin, lb, n);
@@ -372,8 +376,7 @@ cudaError_t launch_match_small(const MatchLaunch& L, int tiles, size_t smem, cud
     if (e != cudaSuccess) return e;
     done[dev].store(1, std::memory_order_release);
   }
-  match_small_kernel<<<tiles, kMatchThreads, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_dependent(match_small_kernel, dim3(tiles), kMatchThreads, smem, st, L);
 }
 
 cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t st) {
@@ -388,7 +391,7 @@ cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t 
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, match_layer_kernel, kMatchThreads, 0);
   if (e != cudaSuccess) return e;
-  match_head_kernel<<<mats, kMatchThreads, 0, st>>>(L, C);
+  if ((e = launch_dependent(match_head_kernel, dim3(mats), kMatchThreads, 0, st, L, C)) != cudaSuccess) return e;
   constexpr int wpb = kMatchThreads / 32;
   for (int i = 2; i < nmax - kMatchTail; ++i) {
     int64_t warps = 0;  // below 2^31: the scratch holds 16 bytes for each of a task's 32 sets
@@ -401,10 +404,10 @@ cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t 
       warps += (int64_t)G.tasks * G.count;
     }
     const int64_t blocks = std::min<int64_t>((warps + wpb - 1) / wpb, (int64_t)sms * resident);
-    match_layer_kernel<<<(unsigned)blocks, kMatchThreads, 0, st>>>(L, C, i);
+    e = launch_dependent(match_layer_kernel, dim3((unsigned)blocks), kMatchThreads, 0, st, L, C, i);
+    if (e != cudaSuccess) return e;
   }
-  match_tail_kernel<<<mats, kMatchThreads, 0, st>>>(L, C);
-  return cudaGetLastError();
+  return launch_dependent(match_tail_kernel, dim3(mats), kMatchThreads, 0, st, L, C);
 }
 
 }  // namespace gbs
