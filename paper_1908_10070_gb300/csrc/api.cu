@@ -327,37 +327,6 @@ bool shape_fits(int precision, int warp_bytes, int maxn) {
   return true;
 }
 
-// Launch shape of the terms kernel: the most warps (one block per SM, up to
-// kTermsWarps) whose shared memory holds every lane group of orders <= n.
-// Measured on 4096 patterns of n = 16 and 80 of n = 28 and 30 (all outputs):
-// 6 / 8 / 10 / 12 warps 4.17 / 3.62 / 3.36 / 3.46 ms at n = 16; at n = 28 no
-// more than 6 fit. Rounds per item 1 / 2 / 4 / 8: 3.57 / 3.41 / 3.36 / 3.36 ms
-// and 77.7 / 62.3 / 54.9 / 52.1 ms (few subsets in an item leave the series,
-// one lane per subset, mostly idle); small batches halve them as needed.
-static TuneCfg terms_cfg(int n) {
-  static const int optin = [] {  // thread-safe one-time initialisation
-    int dev = 0, v = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess || v <= 0) {
-      cudaGetLastError();
-      v = 232448;  // 227 KB, the GB300 opt-in limit
-    }
-    return v;
-  }();
-  TuneCfg c;
-  const int h = std::max(n / 2, 1);
-  c.rounds = 8;
-  for (int w = kTermsWarps; w >= 1; --w) {
-    c.warps_per_block = w;
-    c.warp_bytes = ((optin - 4096) / w) & ~127;
-    bool fits = true;
-    for (int v = 1; v <= h; ++v)
-      for (int s = 1; s <= v; ++s) fits = fits && terms_lanes(s, v, c.warp_bytes, h) != 0;
-    if (fits) break;
-  }
-  return c;
-}
-
 int64_t binom64(int a, int b) {
   if (b < 0 || b > a) return 0;
   int64_t r = 1;
@@ -383,7 +352,7 @@ static int64_t key_cost(int key) {
 }
 
 void Planner::init(const int* n, int batch, int precision, int warp_bytes, const int* rounds_for_n,
-                   int64_t whole_reserve, bool terms) {
+                   int64_t whole_reserve) {
   n_ = n;
   batch_ = batch;
   const int cb = complex_bytes(precision);
@@ -409,7 +378,7 @@ void Planner::init(const int* n, int batch, int precision, int warp_bytes, const
       total_ += nwhole_[v];
     }
     for (int sz = 1; sz <= h; ++sz) {
-      const int G = 32 / (terms ? terms_lanes(sz, h, warp_bytes, stage_h) : lanes_for(2 * sz, h, warp_bytes, stage_h, cb));
+      const int G = 32 / lanes_for(2 * sz, h, warp_bytes, stage_h, cb);
       const int64_t cnt = binom64(h, sz), cap = (int64_t)G * R;
       for (int64_t r0 = 0; r0 < cnt; r0 += cap) {
         ItemTemplate t;
@@ -656,8 +625,7 @@ struct BatchLayout {
   // matching route: the even-order matrices by order (largest first), the
   // tiles of the small ones, and the scratch of the large ones
   bool match = false, terms = false;
-  TuneCfg tcfg;  // terms kernel's launch shape
-  size_t matoff_at = 0, arena_b = 0;
+  size_t arena_b = 0;  // scratch of the terms
   int by_order[kMaxN + 1] = {0}, first_of[kMaxN + 1] = {0}, n_order = 0, n_tiles = 0;
   size_t order_at = 0, tiles_at = 0, tile_smem = 0, match_b = 0;
 };
@@ -708,6 +676,53 @@ static void plan_matching(const int* n, int batch, int sms, BatchLayout& U, std:
       most = match_matrix_bytes(v);
     }
   U.match_b = std::max(most, std::min(large, kMatchBudget));
+}
+
+// Scratch of the terms: chunks of at most this many bytes (one matrix of order
+// 30 takes 12 MB, one of order 16 53 KB).
+constexpr size_t kTermsBudget = (size_t)1 << 30;
+static size_t terms_bytes(const BatchLayout& U) {
+  size_t all = 0, most = 0;
+  for (int v = 2; v <= kMatchMaxN; v += 2)
+    if (U.by_order[v]) {
+      most = 16 * (size_t)terms_matrix_units(v);
+      all += U.by_order[v] * most;
+    }
+  return std::max(most, std::min(all, kTermsBudget));
+}
+static void terms_chunks(const BatchLayout& U, void* scratch, std::vector<TermsChunk>* out) {
+  TermsChunk c;
+  memset(&c, 0, sizeof(c));
+  size_t used = 0;
+  int mats = 0;
+  for (int v = kMatchMaxN; v >= 2; v -= 2) {
+    const size_t one = 16 * (size_t)terms_matrix_units(v);
+    for (int done = 0; done < U.by_order[v];) {
+      const int take = (int)std::min<size_t>(U.by_order[v] - done, (U.arena_b - used) / one);
+      if (take == 0) {
+        c.scratch = scratch;
+        out->push_back(c);
+        memset(&c, 0, sizeof(c));
+        used = 0;
+        mats = 0;
+        continue;
+      }
+      TermsGroup& g = c.g[c.n_groups++];
+      g.n = v;
+      g.first = U.first_of[v] + done;
+      g.count = take;
+      g.begin = mats;
+      g.off = (int64_t)(used / 16);
+      g.stride = (int64_t)(one / 16);
+      used += take * one;
+      mats += take;
+      done += take;
+    }
+  }
+  if (c.n_groups) {
+    c.scratch = scratch;
+    out->push_back(c);
+  }
 }
 
 // The chunks of the larger orders, each within U.match_b bytes of scratch.
@@ -983,16 +998,10 @@ int run_batch(const BatchArgs& a) {
     std::vector<int> order;
     std::vector<MatchTile> tiles;
     if (U.match) plan_matching(a.n, batch, device_sm_count(), U, &order, &tiles);
-    if (U.terms) {
-      U.tcfg = terms_cfg(maxn);
-      for (int v = 0; v <= kMaxN; ++v) rounds_for_n[v] = U.tcfg.rounds;
-    }
+    // (beside the terms: the items of the FP64 kernel behind them)
+    if (U.terms) U.arena_b = terms_bytes(U);
     auto init = [&]() {
-      if (U.terms)
-        plan.init(a.n, batch, a.precision, U.tcfg.warp_bytes, rounds_for_n,
-                  (int64_t)device_sm_count() * U.tcfg.warps_per_block / 2, true);
-      else if (!U.match)
-        plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
+      if (U.terms || !U.match) plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
     };
     init();
     if (!a.cfg_override && (U.terms || !U.match)) {
@@ -1024,7 +1033,7 @@ int run_batch(const BatchArgs& a) {
     }
 
     // plan block: pats | items | (pair-sum offsets) | (probe tables) | (chunk
-    // tables) | (order | tiles of the matchings) | (arena offsets of the terms)
+    // tables) | (order | tiles of the matchings)
     U.pats_b = al(sizeof(PatDesc) * batch);
     U.items_b = al(sizeof(WorkItem) * std::max<int64_t>(U.n_items, 1));
     if (a.precision == GBS_FP64 && !U.match)
@@ -1070,10 +1079,6 @@ int run_batch(const BatchArgs& a) {
       U.tiles_at = U.order_at + al(sizeof(int) * order.size());
       U.up_b = U.tiles_at + al(sizeof(MatchTile) * std::max<size_t>(tiles.size(), 1));
     }
-    if (U.terms) {
-      U.matoff_at = U.up_b;
-      U.up_b += al(2 * sizeof(int64_t) * batch);
-    }
 
     int rc = pinned_acquire(U.up_b + data_b, &host_stage, &slot);
     if (rc) return rc;
@@ -1083,27 +1088,6 @@ int run_batch(const BatchArgs& a) {
     if (U.match) {
       memcpy(hs + U.order_at, order.data(), sizeof(int) * order.size());
       if (!tiles.empty()) memcpy(hs + U.tiles_at, tiles.data(), sizeof(MatchTile) * tiles.size());
-    }
-    if (U.terms) {
-      // every even-order matrix's blocks, and its pair sums while they fit the
-      // budget (later matrices form A_S X A_S by the product)
-      int64_t* mat_off = (int64_t*)(hs + U.matoff_at);
-      int64_t* sum_off = mat_off + batch;
-      int64_t at = 0, sums = 0;
-      for (int b = 0; b < batch; ++b) {
-        const int v = a.n[b], h = v / 2, nb = h * (h + 1) / 2;
-        mat_off[b] = sum_off[b] = -1;
-        if (v < 2 || (v & 1)) continue;
-        mat_off[b] = at;
-        at += 4 * nb;
-        const int64_t q = v >= 6 ? 4ll * nb * pair_sums_width(h) : 0;
-        if (q > 0 && 16 * (sums + q) <= kPairTermBudget) {
-          sum_off[b] = at;
-          at += q;
-          sums += q;
-        }
-      }
-      U.arena_b = al(16 * (size_t)at);
     }
     for (int b = 0; b < batch; ++b) {
       PatDesc& d = h_pats[b];
@@ -1189,10 +1173,9 @@ int run_batch(const BatchArgs& a) {
   const size_t status_b = al(sizeof(int) * batch);
   const size_t pstatus_b = n_sel ? al(sizeof(int) * n_probe) : 0;  // zeroed with ctr and status
   const size_t ok_b = U.terms ? al(sizeof(int) * batch) : 0;       // zeroed too
-  // matchings: a partial per matrix | scratch; terms: exponents | item sums | matrix sums | arena
+  // matchings: a partial per matrix | scratch; terms: exponents | matrix sums | scratch
   const size_t mparts_b = U.match ? al(sizeof(Partial) * batch) : 0;
   const size_t exps_b = U.terms ? al(sizeof(int) * kExpInts * batch) : 0;
-  const size_t kparts_b = U.terms ? al(16 * std::max<int64_t>(n_items, 1)) : 0;
   const size_t ksum_b = U.terms ? al(8 * (size_t)batch) : 0;
   // outputs in host memory (any of them sends all through device staging)
   bool out_hmem[4];
@@ -1211,7 +1194,7 @@ int run_batch(const BatchArgs& a) {
   // route choice on the device: rep_half | rep_end | repeated-row partials
   const size_t droute_b = dev_rep_cap ? 2 * al(sizeof(int) * batch) + al(sizeof(Partial) * dev_rep_cap) : 0;
   const size_t dev_b = data_b + parts_b + ctr_b + status_b + pstatus_b + outs_b + a32_b + pt_b + pparts_b + chparts_b + mperm_b + droute_b + ok_b +
-                       mparts_b + U.match_b + exps_b + kparts_b + ksum_b + U.arena_b;
+                       mparts_b + U.match_b + exps_b + ksum_b + U.arena_b;
   const size_t own_up_b = pe ? 0 : U.up_b;
 
   void* dmem = nullptr;
@@ -1270,11 +1253,9 @@ int run_batch(const BatchArgs& a) {
   o += U.match_b;
   int* d_exps = (int*)(dv + o);
   o += exps_b;
-  double2* d_kparts = (double2*)(dv + o);
-  o += kparts_b;
   double* d_ksum = (double*)(dv + o);
   o += ksum_b;
-  int4* d_arena = (int4*)(dv + o);
+  void* d_arena = dv + o;
 
   HafLaunch L;
   memset(&L, 0, sizeof(L));
@@ -1355,6 +1336,38 @@ int run_batch(const BatchArgs& a) {
         if (e != cudaSuccess) { ret = cuda_fail(e, "route choice launch"); break; }
         L.skip = d_rephalf;
       }
+      if (U.match) {
+        MatchLaunch M;
+        M.src = L.src;
+        M.idx = L.idx;
+        M.pats = d_pats;
+        M.order = (const int*)(up + U.order_at);
+        M.tiles = (const MatchTile*)(up + U.tiles_at);
+        M.skip = L.skip;
+        M.m_bound = L.m_bound;
+        M.status = d_status;
+        M.parts = d_mparts;
+        // Matchings that leave SMs idle run beside the terms, those of the
+        // large orders in any case (FP64 pipe against integer and FP32), and
+        // few small tiles beside the large orders' layers: one 16-photon
+        // pattern with its estimate 176 -> 141 us, 301 matrices of n <= 22 226 ->
+        // 154, 80 patterns of n = 28 and 30 with it 22.2 -> 20.3 ms. Tiles that
+        // fill the SMs gain nothing there (4096 patterns of n = 16: the terms
+        // wait for room as long as the tiles run).
+        const bool shared = U.terms && n_items > 0;
+        const bool few = U.n_tiles <= device_sm_count();
+        const bool beside = (shared && (U.match_b || few)) || (U.n_tiles && U.match_b);
+        if (beside) side.begin(st);
+        else side.here(st);
+        if (U.n_tiles) e = launch_match_small(M, U.n_tiles, U.tile_smem, side.stream());
+        if (e == cudaSuccess && U.match_b) {
+          std::vector<MatchChunk> chunks;
+          match_chunks(U, d_match, &chunks);
+          for (const MatchChunk& c : chunks)
+            if ((e = launch_match_large(M, c, shared, shared ? side.stream() : st)) != cudaSuccess) break;
+        }
+        if (e != cudaSuccess) { ret = cuda_fail(e, "matching kernel launch"); break; }
+      }
       if (n_sel) {
         // probe launch over the candidate orderings, then the choice per matrix
         HafLaunch Lp = L;
@@ -1396,61 +1409,27 @@ int run_batch(const BatchArgs& a) {
         if (e != cudaSuccess) { ret = cuda_fail(e, "pairing choice launch"); break; }
       }
       if (U.match) {
-        MatchLaunch M;
-        M.src = L.src;
-        M.idx = L.idx;
-        M.pats = d_pats;
-        M.order = (const int*)(up + U.order_at);
-        M.tiles = (const MatchTile*)(up + U.tiles_at);
-        M.skip = L.skip;
-        M.m_bound = L.m_bound;
-        M.status = d_status;
-        M.parts = d_mparts;
-        // the small orders' tiles run beside the large orders' layers and the
-        // terms: for one 16-photon pattern with its estimate they are 46 us on
-        // one SM, for 300 matrices of n <= 22 84 us on 109
-        if (U.n_tiles) {
-          if (U.match_b || U.terms) side.begin(st);
-          else side.here(st);
-          e = launch_match_small(M, U.n_tiles, U.tile_smem, side.stream());
-          if (e != cudaSuccess) { ret = cuda_fail(e, "matching kernel launch"); break; }
-        }
-        if (U.match_b) {
-          std::vector<MatchChunk> chunks;
-          match_chunks(U, d_match, &chunks);
-          for (const MatchChunk& c : chunks)
-            if ((e = launch_match_large(M, c, st)) != cudaSuccess) break;
-        }
-        if (e != cudaSuccess) { ret = cuda_fail(e, "matching kernel launch"); break; }
         if (U.terms && n_items > 0) {
           TermsLaunch T;
           memset(&T, 0, sizeof(T));
           T.src = L.src;
           T.idx = L.idx;
           T.pats = d_pats;
-          T.items = d_items;
+          T.order = (const int*)(up + U.order_at);
           T.n_items = (int)n_items;
-          T.batch = batch;
           T.m_bound = L.m_bound;
           T.perm = L.perm;
           T.perm_off = L.perm_off;
           T.skip = L.skip;
-          T.counter = d_ctr + 40;
           T.status = d_status;
-          T.warp_bytes = U.tcfg.warp_bytes;
-          T.stage_h = maxn / 2;
-          T.mat = d_arena;
-          T.mat_off = (const int64_t*)(up + U.matoff_at);
-          T.sum_off = T.mat_off + batch;
           T.exps = d_exps;
           T.ok = d_ok;
-          T.kparts = d_kparts;
           T.ksum = d_ksum;
-          T.n_redo = d_ctr + 41;
-          T.blocks_done = (unsigned*)(d_ctr + 42);
           T.fp64_items = d_ctr + 43;
-          const int tw = U.tcfg.warps_per_block;
-          e = launch_terms(T, (int)std::min<int64_t>(device_sm_count(), (n_items + tw - 1) / tw), tw, st);
+          std::vector<TermsChunk> chunks;
+          terms_chunks(U, d_arena, &chunks);
+          for (const TermsChunk& c : chunks)
+            if ((e = launch_terms(T, c, st)) != cudaSuccess) break;
           if (e != cudaSuccess) { ret = cuda_fail(e, "terms kernel launch"); break; }
           // the matrices the fixed-point terms gave back (normally none)
           HafLaunch L2 = L;

@@ -86,10 +86,8 @@ class Planner {
   // covers all their subsets (sizes staged and reduced together); the
   // remaining ones keep one item per size and rank range, which fill the tail
   // of the schedule (whole items go first, as the largest).
-  // terms: lane groups of the fixed-point terms kernel instead of the subset
-  // kernel's.
   void init(const int* n, int batch, int precision, int warp_bytes, const int* rounds_for_n,
-            int64_t whole_reserve = 0, bool terms = false);
+            int64_t whole_reserve = 0);
   void fill(PatDesc* pats, WorkItem* items);
   int64_t total() const { return total_; }
   // work items of one matrix of order v (0 for odd v or v < 2)

@@ -185,55 +185,48 @@ __host__ __device__ inline bool spare_tile(int N, int h, int warp_bytes, int sta
   return (32 / L) * group_bytes(N, h, cbytes, true) <= avail;
 }
 
-// ---- fixed-point terms (haf_terms.cuh): lane groups of 2 x 2 blocks ----
-__host__ __device__ inline int terms_stage_bytes(int stage_h) {
-  return stage_slots(stage_h) * stage_stride(stage_h) * 16;
+// ---- the subset sum's terms for the error estimate (haf_terms.cuh) ----
+constexpr int kExpInts = 20;        // exponents kept per matrix
+constexpr int kDeltaThreads = 256;  // threads of a block of the delta kernel
+// Lanes per subset of s pairs: one per row of the others, 6 at least (the few
+// small subsets would otherwise set a warp's shared memory).
+__host__ __device__ inline int terms_lanes(int s) { return s > 3 ? 2 * (s - 1) : 6; }
+// Shared memory of one subset of s of h pairs: two columns' vectors, 3 h sums,
+// the pair numbers.
+__host__ __device__ inline int terms_group_bytes(int s, int h) {
+  return (((h - 1) / 2 + 1) * 4 * (s - 1) + 3 * h + ((s + 3) >> 2)) * 16;
 }
-// One lane group's region for subsets of s pairs of a matrix of h pairs: the
-// schedule row's matrices (s (s + 1) / 2 blocks of 64 bytes each) and the pair
-// numbers, padded so that the 8 lanes of a 16-byte access that lie in
-// different groups of fewer than 8 lanes start in different banks.
-__host__ __device__ inline int terms_group_bytes(int s, int h, int L) {
-  int units = sched_nbuf(h) * 2 * s * (s + 1) + ((s + 3) >> 2);
-  if (L < 8)
-    while ((units & 7) != L) ++units;
-  return units * 16;
-}
-// Lanes per subset of s pairs: the fewest (a power of two) whose 32 / L groups
-// fit the warp's bytes and the staging slots and are not mostly idle on the
-// C(h, s) subsets of that size; 0 if none fits.
-__host__ __device__ inline int terms_lanes(int s, int h, int warp_bytes, int stage_h) {
-  const int avail = warp_bytes - 512 - terms_stage_bytes(stage_h);
-  int c = 1;
-  for (int i = 1; i <= s; ++i) c = c * (h - s + i) / i;
-  for (int L = 32 / stage_slots(stage_h); L <= 32; L <<= 1)
-    if (32 / L < 2 * c && (32 / L) * terms_group_bytes(s, h, L) <= avail) return L;
-  return 0;
-}
-constexpr int kTermsWarps = 10;  // most warps in a block (one block per SM); 204 registers a thread
+// The matrices of one order in a chunk. Per matrix the scratch holds n^2 limbs,
+// 2^h h series coefficients D, 2^(h-1) h of G, and the sums' parts.
+struct TermsGroup {
+  int n, first, count;     // matrices order[first, first + count)
+  int begin;               // the group's first matrix in the chunk
+  int block, parts;        // delta kernel: first block, blocks per matrix
+  int region;              // delta kernel: shared bytes per warp
+  int64_t off, stride;     // in units of 16 bytes: the group's first matrix, and per matrix
+};
+struct TermsChunk {
+  int n_groups;
+  void* scratch;
+  TermsGroup g[kMaxN / 2];
+};
 struct TermsLaunch {
   const double* src;       // as in HafLaunch
   const int* idx;
   const PatDesc* pats;
-  const WorkItem* items;
-  int n_items, batch, m_bound;
+  const int* order;        // even-order matrices, by order
+  int n_items, m_bound;
   const int* perm;
   const int* perm_off;
   const int* skip;         // as in HafLaunch: the repeated-row sum gives the estimate
-  int* counter;            // work-queue head, zero before launch
   int* status;
-  int warp_bytes, stage_h;
-  int4* mat;               // limbs: per matrix its entries, and its pair sums
-  const int64_t* mat_off;  // per matrix, in int4 (-1: odd orders)
-  const int64_t* sum_off;  // -1: R_2 by the product
-  int* exps;               // kExpStride exponents per matrix
+  int* exps;               // kExpInts per matrix
   int* ok;                 // zero before launch; in the end 1 where the FP64 kernel has nothing to do
-  double2* kparts;         // per item: sum |f|_1 and the rounding bound
   double* ksum;            // per matrix: sum |f|_1
-  int* n_redo;             // zero before launch
-  unsigned* blocks_done;   // zero before launch
-  int* fp64_items;         // out: items the FP64 kernel is to look at (0 or n_items)
+  int* fp64_items;         // zero before launch; n_items where the FP64 kernel has work
 };
+// 16-byte units of scratch of one matrix.
+int64_t terms_matrix_units(int n);
 
 struct HafLaunch {
   const double* src;       // interleaved complex source matrices
@@ -427,13 +420,13 @@ void match_sizes(int n, int* even, int* odd, double* macs);
 // Device scratch of one matrix of a larger order.
 size_t match_matrix_bytes(int n);
 cudaError_t launch_match_small(const MatchLaunch& L, int tiles, size_t smem, cudaStream_t st);
-cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t st);
+// `shared`: other kernels run beside these and are to find room on the SMs.
+cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, bool shared, cudaStream_t st);
 
 // Defined in haf_subsets.cu
 cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st);
-// The fixed-point terms: prep and pair sums, the terms, and the check.
-cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, cudaStream_t st);
-constexpr int kExpInts = 20;  // ints of TermsLaunch::exps per matrix
+// The terms of a chunk's matrices, and the check.
+cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st);
 cudaError_t launch_route_plan(const RoutePlan& R, cudaStream_t st);
 cudaError_t launch_haf_subsets(const HafLaunch& L, int precision, int blocks, int warps_per_block,
                                cudaStream_t st);

@@ -1662,34 +1662,69 @@ cudaError_t launch_pair_terms(const HafLaunch& L, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_terms(const TermsLaunch& T, int blocks, int warps_per_block, cudaStream_t st) {
-  static_assert(kExpInts == kExpStride, "exponent stride");
-  if (warps_per_block < 1 || warps_per_block > kTermsWarps) return cudaErrorInvalidValue;
-  static std::atomic<int> done[64];
-  int dev = 0;
+int64_t terms_matrix_units(int n) {
+  const int h = n / 2;
+  return (int64_t)n * n + ((int64_t)h << h) + ((int64_t)h << (h - 1)) + (h > 8 ? 1 << (h - 8) : 1);
+}
+
+cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st) {
+  if (C.n_groups <= 0) return cudaSuccess;
+  int dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  static std::atomic<int> done[64];
+  constexpr int most = 160 * 1024;
   if (!done[dev].load(std::memory_order_acquire)) {
-    cudaFuncAttributes fa;
-    e = cudaFuncGetAttributes(&fa, (const void*)haf_terms_kernel);
-    if (e != cudaSuccess) return e;
-    int optin = 0;
-    e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(haf_terms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             optin - (int)fa.sharedSizeBytes);
+    e = cudaFuncSetAttribute(terms_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     done[dev].store(1, std::memory_order_release);
   }
-  const int h = T.stage_h, chunks = (h * (h + 1) / 2 + kSumBlocks - 1) / kSumBlocks;
-  e = launch_dependent(terms_prep_kernel, dim3(T.batch), 256, 0, st, T);
-  if (e == cudaSuccess && h >= 3)
-    e = launch_dependent(terms_sums_kernel, dim3((unsigned)((int64_t)T.batch * chunks)), 256, 0, st, T);
-  if (e == cudaSuccess)
-    e = launch_dependent(haf_terms_kernel, dim3(blocks), warps_per_block * 32, (size_t)warps_per_block * T.warp_bytes, st,
-                         T);
-  if (e == cudaSuccess) e = launch_dependent(terms_check_kernel, dim3(std::min((T.batch + 7) / 8, 1024)), 256, 0, st, T);
+  constexpr int nw = kDeltaThreads / 32;
+  // rounds of each order, and parts of a matrix: as few (a matrix copy each)
+  // as still give the SMs several blocks
+  int64_t rounds[kMaxH + 1] = {0};
+  for (int h = 1; h <= kMaxH; ++h) {
+    int64_t c = 1;
+    for (int s = 1; s <= h; ++s) {
+      c = c * (h - s + 1) / s;
+      const int gpw = 32 / terms_lanes(s);
+      rounds[h] += (c + gpw - 1) / gpw;
+    }
+  }
+  int per = 16;  // rounds per warp
+  for (; per > 1; per /= 2) {
+    int64_t blocks = 0;
+    for (int g = 0; g < C.n_groups; ++g)
+      blocks += C.g[g].count * ((rounds[C.g[g].n / 2] + per * nw - 1) / (per * nw));
+    if (blocks >= 16 * sms) break;
+  }
+  int blocks = 0, mats = 0, hmax = 0;
+  size_t smem = 0;
+  for (int g = 0; g < C.n_groups; ++g) {
+    TermsGroup& G = C.g[g];
+    const int h = G.n / 2;
+    G.parts = (int)((rounds[h] + per * nw - 1) / (per * nw));
+    G.block = blocks;
+    blocks += G.count * G.parts;
+    mats = G.begin + G.count;
+    hmax = std::max(hmax, h);
+    G.region = 0;
+    for (int s = 1; s <= h; ++s) G.region = std::max(G.region, (32 / terms_lanes(s)) * terms_group_bytes(s, h));
+    smem = std::max(smem, (size_t)G.n * (G.n + 1) * 16 + (size_t)nw * G.region);
+  }
+  if (smem > (size_t)most) return cudaErrorInvalidValue;
+  e = launch_dependent(terms_prep_kernel, dim3(mats), 256, 0, st, T, C);
+  if (e == cudaSuccess) e = launch_dependent(terms_delta_kernel, dim3(blocks), kDeltaThreads, smem, st, T, C);
+  if (e == cudaSuccess) e = launch_dependent(terms_series_kernel, dim3(mats), 256, 0, st, T, C, -1);
+  for (int level = 8; level < hmax && e == cudaSuccess; ++level) {
+    int64_t grid = 0;
+    for (int g = 0; g < C.n_groups; ++g)
+      if (C.g[g].n / 2 > level) grid += (int64_t)C.g[g].count << (level - 8);
+    e = launch_dependent(terms_series_kernel, dim3((unsigned)grid), 256, 0, st, T, C, level);
+  }
+  if (e == cudaSuccess) e = launch_dependent(terms_check_kernel, dim3(std::min((mats + 7) / 8, 1024)), 256, 0, st, T, C);
   return e;
 }
 

@@ -1,50 +1,71 @@
-// sum_S |f(X A_S)|_1 of the subset sum, in fixed point (included by
-// haf_subsets.cu, inside its anonymous namespace).
+// sum_S |f(X A_S)|_1 of the subset sum (included by haf_subsets.cu, inside its
+// anonymous namespace).
 //
-// The estimate of a result's error needs the moduli of the subset sum's terms;
-// the Hafnian itself comes from the matchings (match.cu). The terms' power
-// traces are the FP64 kernel's, but a product entry here is fixed point: an
-// entry of R_k = A (X A)^{k-1} is (hi + lo) 2^{E_k - 27}, hi a whole number of
-// at most 2^27, lo a float of at most a half, with one exponent E_k per matrix
-// and power. A complex multiply-add is then 4 IMAD.WIDE (hi hi, summed exactly
-// in 64 bits) and 8 FFMA (hi lo and lo hi, which need 24 bits only), instead of
-// 4 DFMA: 32 clocks of a warp and SM quarter instead of 256 on this part (DFMA
-// 2 a clock and SM; IMAD.WIDE 32; FFMA 128). All four products as IMAD.WIDE,
-// with lo an integer too, took 52.
+// The estimate of a result's error needs the moduli of the subset sum's terms
+// f(X A_S) = [x^h] det(I - x X A_S)^{-1/2}; the Hafnian itself comes from the
+// matchings (match.cu). For p the last pair of S and S' = S \ {p}, the Schur
+// complement of the pairs of S' leaves a 2 x 2 determinant:
+//     det(I - x X A_S) = det(I - x X A_S') D_S,   D_S = (1 - b)^2 - a c,
+// a, b, c the power series of the walks from p to p whose inside lies in S',
+//     b = x A(2p, 2p+1) + sum_k x^{k+2} u^T X (A_S' X)^k v   (a: u u, c: v v),
+// u, v the columns 2p and 2p+1 of A on the rows of S'. A term then costs the
+// Krylov vectors u_j = (A_S' X)^j u, j <= (h-1)/2, of two columns (walks of
+// length i + j from u_i and u_j), about h/2 steps of (2|S'|)^2 products each,
+// and three series products, instead of the powers of a 2|S| matrix: 450
+// complex multiply-adds against 1500 at n = 16, 3300 against 14,000 at n = 30.
+// A and its subsets share one copy in shared memory; a subset keeps vectors
+// only, so enough warps are resident to hide latency.
+//   terms_delta_kernel   D_S of every subset,
+//   terms_series_kernel  f_S = [x^h] prod over the pairs of S of D^{-1/2},
+//                        by the last pair: G_S = G_S' D_S^{-1/2}.
+// 4096 patterns of n = 16: 0.91 and 0.31 ms (powers in the same arithmetic:
+// 2.35 ms and 0.16 for pair sums); 64 of n = 28 with 16 of n = 30: 11.9 and 1.4
+// ms (40). The first kernel keeps the multipliers 55 % busy at n = 28; two
+// thirds of its lanes have a row.
+//
+// Arithmetic. A vector entry is fixed point, (hi + lo) 2^{E_k - 27}, hi a whole
+// number of at most 2^27, lo a float of at most a half, with one exponent E_k
+// per matrix and power. A complex multiply-add is then 4 IMAD.WIDE (hi hi,
+// summed exactly in 64 bits) and 8 FFMA (hi lo and lo hi, which need 24 bits
+// only), instead of 4 DFMA: 32 clocks of a warp and SM quarter instead of 256
+// on this part (DFMA 2 a clock and SM; IMAD.WIDE 32; FFMA 128). All four
+// products as IMAD.WIDE, with lo an integer too, took 52. The series run in
+// pairs of floats (48 FP32 operations a multiply-add), coefficient k in units
+// of 2^{e k}, e a mean growth of the E_k.
 //
 // E_k is fixed per matrix from its full powers (in float, prep kernel) with a
 // factor 4..8 of room; an entry is then rounded at 2^-49 of the range. What
 // that cannot promise is checked: a value past the range, inputs that are not
-// finite, exponents too far apart, or a bound on the rounding carried along
-// with the series that comes out above 2^-33 of the sum, send the matrix to
-// the FP64 kernel (launched after; it returns at once when no matrix is left
-// to it).
+// finite, exponents too far apart, or an estimate of the rounding carried along
+// with the series (several times what is met, and added over the subsets
+// without regard to sign) that comes out above 2^-33 of the sum, send the
+// matrix to the FP64 subset kernel (launched after; it returns at once when no matrix is
+// left to it).
 
 constexpr int kFxBits = 27;      // |hi| <= 2^27
 constexpr int kFxRoom = 2;       // exponents added to the float estimate of a power's largest entry
-constexpr int kTermsHeader = 512;  // per warp: scales, rounding bounds, exponents
-constexpr int kExpStride = 20;   // exponents kept per matrix
-constexpr int kSumBlocks = 8;    // 2 x 2 blocks of pair sums per thread block
+constexpr int kExpStride = kExpInts;  // per matrix: E_1, E_2, .. at 1, 2, ..; e at kExpUnit
+constexpr int kExpUnit = 18;
 
 // A stored complex entry: x, y = hi (re, im), z, w = lo (float bits). In
-// registers hi comes as a float too, hi 2^-6 cut to a whole number (the
-// products with lo need no more), by adding and taking off 1.5 2^23.
+// registers hi comes as a float too, for the products with lo. (Cut to its top
+// 22 bits, which an addition converts, it cost the estimate of one 16-photon
+// pattern four bits.)
 struct FxOp {
   int hr, hi;
   float lr, li, fr, fi;
 };
-__device__ __forceinline__ float fx_float(int h) { return __int_as_float((h >> 6) + 0x4B400000) - 12582912.0f; }
 __device__ __forceinline__ FxOp fx_load(const int4& v) {
   FxOp o;
   o.hr = v.x;
   o.hi = v.y;
   o.lr = __int_as_float(v.z);
   o.li = __int_as_float(v.w);
-  o.fr = fx_float(v.x);
-  o.fi = fx_float(v.y);
+  o.fr = (float)v.x;
+  o.fi = (float)v.y;
   return o;
 }
-struct Fx {  // one complex sum: h + 64 m
+struct Fx {  // one complex sum: h + m
   long long rh, ih;
   float rm, im;
 };
@@ -71,12 +92,12 @@ __device__ __forceinline__ int2 fx_pack(int hi, float lo, bool& over) {
   over |= (unsigned)(hi + (1 << kFxBits)) > (2u << kFxBits);
   return make_int2(hi, __float_as_int(lo - (q - 12582912.0f)));
 }
-// (h + 64 m) 2^-sh, 18 <= sh <= 31 (so h 2^-sh is below 2^44).
+// (h + m) 2^-sh, 18 <= sh <= 31 (so h 2^-sh is below 2^44).
 __device__ __forceinline__ int2 fx_round(long long h, float m, int sh, bool& over) {
   const long long top = h >> sh;
-  over |= (unsigned)((int)(top >> 28) + 1) > 1u || !(fabsf(m) < 0x1p30f);
+  over |= (unsigned)((int)(top >> 28) + 1) > 1u || !(fabsf(m) < 0x1p36f);
   const float unit = __int_as_float((127 - sh) << 23);
-  const float lo = (float)((unsigned)h & ((1u << sh) - 1)) * unit + m * (64.0f * unit);
+  const float lo = (float)((unsigned)h & ((1u << sh) - 1)) * unit + m * unit;
   return fx_pack((int)top, lo, over);
 }
 __device__ __forceinline__ int4 fx_entry(const Fx& c, int sh, bool& over) {
@@ -85,26 +106,22 @@ __device__ __forceinline__ int4 fx_entry(const Fx& c, int sh, bool& over) {
 }
 __device__ __forceinline__ bool fx_shift_ok(int sh) { return sh >= 18 && sh <= 31; }
 
-// A symmetric matrix of s pairs as 2 x 2 blocks of its upper block triangle:
-// block (r, c), r < c, is number c(c-1)/2 + r, block (r, r) number
-// s(s-1)/2 + r; element 2 i + j of a block is entry (2r + i, 2c + j).
-__device__ __forceinline__ int blk_index(int r, int c, int s) {
-  const int lo = min(r, c), hi = max(r, c);
-  return lo == hi ? s * (s - 1) / 2 + lo : hi * (hi - 1) / 2 + lo;
-}
 
-// Per matrix: the exponents, the entries' limbs (block layout of all h pairs,
-// elements innermost), and whether it can be done in fixed point at all. One
-// block per matrix. The powers of the whole matrix, scaled to entries below 1,
-// are formed in float only for the size of their largest entry.
-__global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P) {
+// Per matrix: the exponents, the entries' limbs (rows and columns in the
+// subset sum's order, zero diagonal), and whether it can be done in fixed
+// point at all. One block per matrix. The powers of the whole matrix, scaled
+// to entries below 1, are formed in float only for the size of their largest
+// entry.
+__global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P, const TermsChunk C) {
   __shared__ float2 A[kMaxN * kMaxN], R[kMaxN * kMaxN];
   __shared__ int rows[kMaxN], s_max[kMaxN / 2 + 1], s_lo, s_bad;
   dependency_wait();
-  const int b = blockIdx.x;
+  int g = 0;
+  while (g + 1 < C.n_groups && (int)blockIdx.x >= C.g[g + 1].begin) ++g;
+  const TermsGroup G = C.g[g];
+  const int q = blockIdx.x - G.begin, b = P.order[G.first + q];
   const PatDesc d = P.pats[b];
-  const int n = d.n, h = n >> 1;
-  if (n < 2 || (n & 1) || P.mat_off[b] < 0) return;
+  const int n = G.n, h = n >> 1;
   if (P.skip != nullptr && P.skip[b] != 0) return;
   if (threadIdx.x < n) {
     int pos = default_pos(threadIdx.x, h);
@@ -146,27 +163,24 @@ __global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P) {
   if (e1 > 900 || e1 < -900 || s_max[0] - s_lo > 20) return;  // ok stays 0 (uniform)
   const double up = __hiloint2double((kFxBits - e1 + 1023) << 20, 0);
   const double unit = __hiloint2double((1023 - e1) << 20, 0);
-  int4* out = P.mat + P.mat_off[b];
+  int4* out = reinterpret_cast<int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int r = e / n, c = e - r * n;
     double2 v = make_double2(0.0, 0.0);
     if (r != c) v = __ldg(src2 + (int64_t)rows[min(r, c)] * d.ld + rows[max(r, c)]);
     A[e] = R[e] = make_float2((float)(v.x * unit), (float)(v.y * unit));
-    if ((r >> 1) <= (c >> 1)) {
-      const double x = v.x * up, y = v.y * up;
-      const int hx = __double2int_rn(x), hy = __double2int_rn(y);
-      out[4 * blk_index(r >> 1, c >> 1, h) + 2 * (r & 1) + (c & 1)] =
-          make_int4(hx, hy, __float_as_int((float)(x - hx)), __float_as_int((float)(y - hy)));
-    }
+    const double x = v.x * up, y = v.y * up;
+    const int hx = __double2int_rn(x), hy = __double2int_rn(y);
+    out[e] = make_int4(hx, hy, __float_as_int((float)(x - hx)), __float_as_int((float)(y - hy)));
   }
   __syncthreads();
-  // largest entries of the powers the schedule keeps, as float bits
-  const int top = (int)((0x8877665645332211ull >> (4 * (h - 1))) & 15u);
+  // largest entries of the powers that vectors reach, as float bits
+  const int top = (h + 1) / 2;
   for (int k = 2; k <= top; ++k) {
     float2 acc[4];
     float big = 0.0f;
-    int q = 0;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x, ++q) {
+    int i = 0;
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x, ++i) {
       const int r = e / n, c = e - r * n;
       float2 s = make_float2(0.f, 0.f);
       for (int t = 0; t < n; ++t) {
@@ -176,493 +190,385 @@ __global__ void __launch_bounds__(256) terms_prep_kernel(const TermsLaunch P) {
         s.y = fmaf(x.x, y.y, s.y);
         s.y = fmaf(x.y, y.x, s.y);
       }
-      acc[q] = s;
+      acc[i] = s;
       big = fmaxf(big, fmaxf(fabsf(s.x), fabsf(s.y)));
     }
     atomicMax(&s_max[k], __float_as_int(big));
     __syncthreads();
-    q = 0;
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x, ++q) R[e] = acc[q];
+    i = 0;
+    for (int e = threadIdx.x; e < n * n; e += blockDim.x, ++i) R[e] = acc[i];
     __syncthreads();
   }
-  if (threadIdx.x < kExpStride) {
+  int* ex = P.exps + (int64_t)b * kExpStride;
+  if (threadIdx.x >= 1 && (int)threadIdx.x <= top) {
     const int k = threadIdx.x;
-    int ek = 0;
-    if (k == 1) ek = e1;
-    if (k >= 2 && k <= top) {
+    int ek = e1;
+    if (k >= 2) {
       const int f = (s_max[k] >> 23) & 255;
       if (f < 20 || f > 250) s_bad = 1;  // zero, vanishing or not finite
       ek = k * e1 + f - 126 + kFxRoom;
     }
-    P.exps[(int64_t)b * kExpStride + k] = ek;
+    ex[k] = ek;
+    if (k == top) ex[kExpUnit] = __float2int_rn((float)ek / (float)top);
   }
   __syncthreads();
   if (threadIdx.x == 0 && !s_bad) P.ok[b] = 1;
 }
 
-// Pair sums (see pair_terms_elems) of kSumBlocks blocks of one matrix: Q_p of
-// each entry by two fixed-point products, then the sums over the subsets of
-// the low and of the high pairs.
-__global__ void __launch_bounds__(256) terms_sums_kernel(const TermsLaunch P) {
-  __shared__ int4 Q[kSumBlocks * 4 * kMaxH];
-  dependency_wait();
-  const int hm = P.stage_h, chunks = (hm * (hm + 1) / 2 + kSumBlocks - 1) / kSumBlocks;
-  const int b = blockIdx.x / chunks, b0 = (blockIdx.x - b * chunks) * kSumBlocks;
-  const int n = P.pats[b].n, h = n >> 1, nb = h * (h + 1) / 2;
-  if (n < 6 || (n & 1) || b0 >= nb || P.sum_off[b] < 0 || P.ok[b] == 0) return;  // uniform
-  const int* ex = P.exps + (int64_t)b * kExpStride;
-  const int sh = 27 + ex[2] - 2 * ex[1];
-  if (!fx_shift_ok(sh)) {
-    if (threadIdx.x == 0) P.ok[b] = 0;
-    return;
-  }
-  const int4* mat = P.mat + P.mat_off[b];
-  const int cnt = min(kSumBlocks, nb - b0);
-  bool over = false;
-  auto entry = [&](int i, int j) -> int4 {  // A(i, j)
-    const int r = i >> 1, c = j >> 1;
-    const int el = (r <= c) ? 2 * (i & 1) + (j & 1) : 2 * (j & 1) + (i & 1);
-    return __ldg(mat + 4 * blk_index(r, c, h) + el);
-  };
-  for (int t = threadIdx.x; t < cnt * 4 * h; t += blockDim.x) {
-    const int p = t % h, el = (t / h) & 3, k = b0 + t / (4 * h);
-    int r, c;
-    if (k >= h * (h - 1) / 2) {
-      r = c = k - h * (h - 1) / 2;
-    } else {
-      c = 1;
-      while (c * (c + 1) / 2 <= k) ++c;
-      r = k - c * (c - 1) / 2;
-    }
-    const int i = 2 * r + (el >> 1), j = 2 * c + (el & 1);
-    Fx q = fx_zero();
-    const FxOp a0 = fx_load(entry(i, 2 * p)), a1 = fx_load(entry(i, 2 * p + 1));
-    fx_mac(q, a0, -a0.hi, fx_load(entry(2 * p + 1, j)));
-    fx_mac(q, a1, -a1.hi, fx_load(entry(2 * p, j)));
-    Q[t] = fx_entry(q, sh, over);
-  }
-  __syncthreads();
-  const int hl = pair_split_lo(h), W = pair_sums_width(h);
-  int4* out = P.mat + P.sum_off[b] + (int64_t)b0 * W * 4;
-  for (int t = threadIdx.x; t < cnt * W * 4; t += blockDim.x) {
-    const int el = t & 3, w = (t >> 2) % W, k = (t >> 2) / W;
-    const bool low = w < (1 << hl);
-    unsigned m = low ? (unsigned)w : (unsigned)(w - (1 << hl)) << hl;
-    int hr = 0, hi = 0;
-    float lr = 0.0f, li = 0.0f;
-    for (; m; m &= m - 1) {
-      const int4 v = Q[(k * 4 + el) * h + __ffs(m) - 1];
-      hr += v.x;
-      hi += v.y;
-      lr += __int_as_float(v.z);
-      li += __int_as_float(v.w);
-    }
-    const int2 x = fx_pack(hr, lr, over), y = fx_pack(hi, li, over);
-    out[t] = make_int4(x.x, y.x, x.y, y.y);
-  }
-  if (over) P.ok[b] = 0;
+// ---- pairs of floats ------------------------------------------------------
+// A complex number: x, y = high parts (re, im), z, w = low parts.
+// s += a b of one component; the low sum gathers every rounding error but its
+// own (Dekker and Knuth; no contraction between the steps).
+__device__ __forceinline__ void df_mac(float& sh, float& sl, float ah, float al, float bh, float bl) {
+  const float p = __fmul_rn(ah, bh);
+  float e = __fmaf_rn(ah, bh, -p);
+  e = __fmaf_rn(ah, bl, e);
+  e = __fmaf_rn(al, bh, e);
+  const float s = __fadd_rn(sh, p), z = __fsub_rn(s, sh);
+  const float w = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, z)), __fsub_rn(p, z));
+  sh = s;
+  sl = __fadd_rn(sl, __fadd_rn(w, e));
 }
+__device__ __forceinline__ void dfc_mac(float4& c, const float4& a, const float4& b) {
+  df_mac(c.x, c.z, a.x, a.z, b.x, b.z);
+  df_mac(c.y, c.w, a.x, a.z, b.y, b.w);
+  df_mac(c.x, c.z, -a.y, -a.w, b.y, b.w);
+  df_mac(c.y, c.w, a.y, a.w, b.x, b.z);
+}
+__device__ __forceinline__ float4 dfc_norm(const float4& c) {
+  const float h = __fadd_rn(c.x, c.z), i = __fadd_rn(c.y, c.w);
+  return make_float4(h, i, __fsub_rn(c.z, __fsub_rn(h, c.x)), __fsub_rn(c.w, __fsub_rn(i, c.y)));
+}
+// a times a float (exactly rounded at the low part).
+__device__ __forceinline__ float4 dfc_scale(const float4& a, float f) {
+  const float x = __fmul_rn(a.x, f), y = __fmul_rn(a.y, f);
+  return make_float4(x, y, __fmaf_rn(a.z, f, __fmaf_rn(a.x, f, -x)), __fmaf_rn(a.w, f, __fmaf_rn(a.y, f, -y)));
+}
+__device__ __forceinline__ float dfc_abs1(const float4& a) { return fabsf(a.x) + fabsf(a.y); }
+// (h + m) unit as a pair of floats.
+__device__ __forceinline__ float2 df_from(long long h, float m, float unit) {
+  const float hi = __ll2float_rn(h);
+  const float lo = __fadd_rn(__ll2float_rn(h - __float2ll_rn(hi)), m);
+  const float s = __fadd_rn(hi, lo);
+  return make_float2(s * unit, __fsub_rn(lo, __fsub_rn(s, hi)) * unit);
+}
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }  // -126 <= e <= 127
 
-// R_c = R_a X R_b in 2 x 2 blocks: block (r, c) sums over the pairs t the
-// products of block (r, t) of R_a with block (t, c) of R_b, rows swapped; per
-// step eight 16-byte loads feed eight multiply-adds. A block
-// below the diagonal is its mirror with elements 1 and 2 exchanged. Lanes take
-// consecutive blocks (one column, consecutive rows): R_b's loads are then
-// broadcasts and R_a's fall into different banks (their numbers step by 1 or
-// run through the triangular numbers, which differ mod 8).
-__device__ __forceinline__ void fx_prod(int4* __restrict__ dst, const int4* __restrict__ Ra,
-                                        const int4* __restrict__ Rb, const unsigned short* __restrict__ rc, int s,
-                                        int E, int sh, int l, int L, bool& over) {
-  const int D = s * (s - 1) / 2;
-  for (int e0 = 0; e0 < E; e0 += L) {
-    const int e = min(e0 + l, E - 1);
-    int r, c;
-    if (e >= D) {
-      r = c = e - D;
-    } else {
-      const int v = rc[e];
-      r = v & 255;
-      c = v >> 8;
-    }
-    Fx c00 = fx_zero(), c01 = c00, c10 = c00, c11 = c00;
-    const int rr = r * (r - 1) / 2, cc = c * (c - 1) / 2;
-    int tt = 0;  // t (t - 1) / 2
-#pragma unroll 1
-    for (int t = 0; t < s; ++t) {
-      const int ia = (t > r) ? tt + r : (t == r) ? D + r : rr + t;
-      const int ib = (t > c) ? tt + c : (t == c) ? D + c : cc + t;
-      const int a1 = (t < r) ? 2 * E : E, b1 = (t > c) ? 2 * E : E;
-      const int4* pa = Ra + ia;
-      const int4* pb = Rb + ib;
-      const FxOp y10 = fx_load(pb[3 * E - b1]), y00 = fx_load(pb[0]), y11 = fx_load(pb[3 * E]), y01 = fx_load(pb[b1]);
-      {
-        const FxOp x0 = fx_load(pa[0]), x1 = fx_load(pa[a1]);
-        const int n0 = -x0.hi, n1 = -x1.hi;
-        fx_mac(c00, x0, n0, y10);
-        fx_mac(c01, x0, n0, y11);
-        fx_mac(c00, x1, n1, y00);
-        fx_mac(c01, x1, n1, y01);
-      }
-      {
-        const FxOp x0 = fx_load(pa[3 * E - a1]), x1 = fx_load(pa[3 * E]);
-        const int n0 = -x0.hi, n1 = -x1.hi;
-        fx_mac(c10, x0, n0, y10);
-        fx_mac(c11, x0, n0, y11);
-        fx_mac(c10, x1, n1, y00);
-        fx_mac(c11, x1, n1, y01);
-      }
-      tt += t;
-    }
-    if (e0 + l < E) {
-      dst[e] = fx_entry(c00, sh, over);
-      dst[E + e] = fx_entry(c01, sh, over);
-      dst[2 * E + e] = fx_entry(c10, sh, over);
-      dst[3 * E + e] = fx_entry(c11, sh, over);
-    }
-  }
-}
-
-// Traces, this lane's share, as 64-bit integers (tr X R_a X R_b: in
-// 2^{E_a + E_b - 54}, tr X R_a: in 2^{E_a - 47}). Blocks above the diagonal stand for their
-// mirrors too: they come first, and the sum is doubled before the diagonal
-// ones; within a block the square's terms pair up as well.
-__device__ __forceinline__ longlong2 fx_tr2(const int4* __restrict__ Ra, const int4* __restrict__ Rb, int s, int E,
-                                            int l, int L) {
-  const int D = s * (s - 1) / 2;
-  const bool square = Ra == Rb;
-  Fx c = fx_zero();
-  bool twice = false;
-  for (int e = l; e < E; e += L) {
-    if (e >= D && !twice) {
-      c.rh <<= 1;
-      c.ih <<= 1;
-      c.rm *= 2.0f;
-      c.im *= 2.0f;
-      twice = true;
-    }
-    const FxOp x00 = fx_load(Ra[e]), x01 = fx_load(Ra[E + e]);
-    fx_mac(c, x00, -x00.hi, fx_load(Rb[3 * E + e]));
-    fx_mac(c, x01, -x01.hi, fx_load(Rb[2 * E + e]));
-    if (!square) {
-      const FxOp x10 = fx_load(Ra[2 * E + e]), x11 = fx_load(Ra[3 * E + e]);
-      fx_mac(c, x10, -x10.hi, fx_load(Rb[E + e]));
-      fx_mac(c, x11, -x11.hi, fx_load(Rb[e]));
-    }
-  }
-  longlong2 w;
-  w.x = c.rh + __float2ll_rn(64.0f * c.rm);
-  w.y = c.ih + __float2ll_rn(64.0f * c.im);
-  const int up = (twice ? 0 : 1) + (square ? 1 : 0);
-  w.x <<= up;
-  w.y <<= up;
-  return w;
-}
-__device__ __forceinline__ longlong2 fx_tr1(const int4* __restrict__ Ra, int s, int E, int l, int L) {
-  longlong2 w = make_longlong2(0, 0);
-  for (int r = l; r < s; r += L) {
-    const int4 v = Ra[E + s * (s - 1) / 2 + r];
-    w.x += ((long long)v.x << 20) + __float2int_rn(__int_as_float(v.z) * 0x1p20f);
-    w.y += ((long long)v.y << 20) + __float2int_rn(__int_as_float(v.w) * 0x1p20f);
-  }
-  w.x <<= 1;
-  w.y <<= 1;
-  return w;
-}
-
-// Persistent warps over work items (as haf_subsets_kernel): a warp takes
-// 32 / L subsets of one size at a time, L lanes each. Six to ten warps an SM
-// (shared memory sets the number) leave latency in sight, so loads are issued
-// ahead of their use and sums run two at a time. 4096 patterns of n = 16: this
-// kernel 2.66 -> 2.35 ms (with one load in flight, each trace summed alone);
-// with every part timed by leaving it out, products take 1.1 ms of it, their
-// rounding a third of that, traces and loads 0.6, the series 0.3, the sums over
-// lanes 0.3 (before the pairing). 80 patterns of n = 28 and 30: products 22 of
-// 40 ms, at six warps an SM.
-__global__ void __launch_bounds__(kTermsWarps * 32, 1) haf_terms_kernel(const TermsLaunch P) {
+// D_S of every subset: a warp takes rounds of 32 / L subsets of one size, L
+// lanes each (lane = row of S'; then one of the 3 (h - 1) sums; then one
+// coefficient). Round r of a matrix: the sizes in order, the subsets of a size
+// in colex order, consecutive ones side by side. Block (matrix, part) has
+// rounds part, part + parts, ..
+__global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsLaunch P, const TermsChunk C) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ Tables tab;
-  __shared__ unsigned short rc[kMaxH * (kMaxH - 1) / 2];
+  __shared__ int binom[kMaxH + 1][kMaxH + 1], ex[kExpStride], s_bad;
+  __shared__ float unit[kMaxH + 1];  // of the coefficient x^k, k >= 2
   if (threadIdx.x <= kMaxH) {
     const int a = threadIdx.x;
     int c = 1;
     for (int b = 0; b <= kMaxH; ++b) {  // C(a, b) = C(a, b-1) (a-b+1) / b
-      tab.binom[a][b] = (b <= a) ? c : 0;
+      binom[a][b] = (b <= a) ? c : 0;
       if (b < a) c = c * (a - b) / (b + 1);
     }
-    tab.inv2k[a] = (a == 0) ? 0.0 : 1.0 / (2.0 * a);
-    for (int r = 0; r < a && a < kMaxH; ++r) rc[a * (a - 1) / 2 + r] = (unsigned short)(r | (a << 8));
   }
+  if (threadIdx.x == 0) s_bad = 0;
   dependency_wait();
+  int g = 0;
+  while (g + 1 < C.n_groups && (int)blockIdx.x >= C.g[g + 1].block) ++g;
+  const TermsGroup G = C.g[g];
+  const int n = G.n, h = n >> 1, q = (blockIdx.x - G.block) / G.parts, part = (blockIdx.x - G.block) - q * G.parts;
+  const int b = P.order[G.first + q];
+  if (P.ok[b] == 0) return;  // uniform: not in fixed point, or the repeated-row sum's
+  const int4* mat = reinterpret_cast<const int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
+  float4* delta = reinterpret_cast<float4*>(const_cast<int4*>(mat) + n * n);
+  int4* M = reinterpret_cast<int4*>(smem);
+  const int ld = n + 1;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int r = e / n;
+    M[r * ld + e - r * n] = __ldg(mat + e);
+  }
+  if (threadIdx.x < kExpStride) ex[threadIdx.x] = P.exps[(int64_t)b * kExpStride + threadIdx.x];
   __syncthreads();
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* wbase = smem + (size_t)warp * P.warp_bytes;
-  double* sc = reinterpret_cast<double*>(wbase);      // trace k's unit, k = 1..16 at k - 1
-  double* cn = sc + kMaxH;                            // bound on its rounding over 2k
-  int* ex = reinterpret_cast<int*>(cn + kMaxH);       // E_k
-  longlong2* stage = reinterpret_cast<longlong2*>(wbase + kTermsHeader);
-  const int sts = stage_stride(P.stage_h), slots = stage_slots(P.stage_h);
-  unsigned char* gbase = wbase + kTermsHeader + terms_stage_bytes(P.stage_h);
-
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(P.counter, 1);
-    it = __shfl_sync(FULL, it, 0);
-    if (it >= P.n_items) break;
-    const WorkItem w = P.items[it];
-    if ((P.skip != nullptr && P.skip[w.pat] != 0) || P.ok[w.pat] == 0) {
-      if (lane == 0) P.kparts[w.part] = make_double2(0.0, 0.0);
-      continue;
+  const int steps = (h - 1) / 2;  // vectors u_0 .. u_steps
+  if (threadIdx.x >= 1 && (int)threadIdx.x <= steps) {
+    const int k = threadIdx.x;
+    if (!fx_shift_ok(27 + ex[k + 1] - ex[k] - ex[1])) s_bad = 1;
+  }
+  if (threadIdx.x >= 1 && (int)threadIdx.x <= h) {
+    const int k = threadIdx.x, i = (k - 2) >> 1;
+    // x^1: the entry itself; x^k: u_i and u_j, i + j = k - 2, exponents E_{i+1}, E_{j+1}
+    const int e = (k == 1) ? ex[1] - 27 - ex[kExpUnit] : ex[i + 1] + ex[k - 2 - i + 1] - 54 - k * ex[kExpUnit];
+    if (e < -120 || e > 0) s_bad = 1;
+    unit[k] = pow2f(max(min(e, 120), -120));
+  }
+  __syncthreads();
+  if (s_bad) {
+    if (threadIdx.x == 0) P.ok[b] = 0;
+    return;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  unsigned char* wbase = smem + (size_t)n * ld * 16 + (size_t)warp * G.region;
+  bool over = false;
+  int s = 1, done = 0;  // rounds of the sizes below s
+  for (int r = part * nw + warp;; r += G.parts * nw) {
+    int L = terms_lanes(s), rounds = (binom[h][s] + 32 / L - 1) / (32 / L);
+    while (r - done >= rounds) {
+      done += rounds;
+      if (++s > h) break;
+      L = terms_lanes(s);
+      rounds = (binom[h][s] + 32 / L - 1) / (32 / L);
     }
-    const int n = P.pats[w.pat].n, h = n >> 1;
-    const bool whole = w.s_last > w.s;
-    const int s_first = w.s, s_last = whole ? w.s_last : w.s;
-    const int4* mat = P.mat + P.mat_off[w.pat];
-    const int64_t so = P.sum_off[w.pat];
-    const int4* sums = (so >= 0) ? P.mat + so : nullptr;
-    const int hl = pair_split_lo(h), W = pair_sums_width(h);
-    bool over = false;
-    __syncwarp();
-    if (lane < kExpStride) ex[lane] = P.exps[(int64_t)w.pat * kExpStride + lane];
-    __syncwarp();
-    // units and rounding bounds of the traces, by the schedule's ops (the
-    // power each buffer holds in pw, four bits a buffer)
+    if (s > h) break;
+    const int gpw = 32 / L, gi = min(lane / L, gpw - 1), l = lane - gi * L;  // lanes past the last group: l >= L
+    const int rank = (r - done) * gpw + gi;
+    const bool active = rank < binom[h][s] && l < L;
+    int4* V = reinterpret_cast<int4*>(wbase + (size_t)gi * terms_group_bytes(s, h));
+    const int sp = s - 1, N = 2 * sp;
+    float4* mom = reinterpret_cast<float4*>(V + (steps + 1) * 2 * N);  // a, b, c at 3 (k - 1) + 0, 1, 2
+    int* pairs = reinterpret_cast<int*>(mom + 3 * h);
+    unsigned mask = 0;
     {
-      unsigned pw = 1;
-      for (int o = 0; o < kMaxOps; ++o) {
-        const SchedOp op = c_sched[h][o];
-        if (op.kind == kEnd) break;
-        const int ka = (pw >> (4 * op.a)) & 15, kb = (pw >> (4 * op.b)) & 15;
-        if (op.kind == kProd) {
-          pw = (pw & ~(15u << (4 * op.k))) | (unsigned)(ka + kb) << (4 * op.k);
-          if (!fx_shift_ok(27 + ex[ka + kb] - ex[ka] - ex[kb])) over = true;
-        } else if (lane == 0) {
-          const int u = (op.kind == kTr1) ? ex[ka] - 47 : ex[ka] + ex[kb] - 54;
-          if (u < -1000 || u > 1000) over = true;
-          sc[op.k - 1] = __hiloint2double((max(min(u, 1000), -1000) + 1023) << 20, 0);
-          // n entries off by 2^-49 of their range, against the other factor's largest
-          cn[op.k - 1] = (double)n * sc[op.k - 1] * ((op.kind == kTr1) ? 0.25 : 8.0) * tab.inv2k[op.k];
-        }
+      int rk = min(rank, binom[h][s] - 1), c = h - 1;
+      for (int i = s; i >= 1; --i) {
+        while (binom[c][i] > rk) --c;
+        rk -= binom[c][i];
+        mask |= 1u << c;
+        --c;
       }
-      over = __any_sync(FULL, over);
+    }
+    const int p = 31 - __clz((int)mask);
+    const unsigned rest = mask ^ (1u << p);
+    if (l < sp) {
+      unsigned m = rest;
+      for (int t = 0; t < l; ++t) m &= m - 1;
+      pairs[l] = __ffs((int)m) - 1;
+    }
+    __syncwarp();
+    const bool mine = l < N;
+    const int4* row = M + (mine ? 2 * pairs[l >> 1] + (l & 1) : 0) * ld;
+    if (mine) {
+      V[l] = row[2 * p];
+      V[N + l] = row[2 * p + 1];
+    }
+    __syncwarp();
+    for (int k = 1; k <= steps; ++k) {
+      if (mine) {
+        const int4* U = V + (k - 1) * 2 * N;
+        Fx ca = fx_zero(), cb = ca;
+#pragma unroll 1
+        for (int t = 0; t < sp; ++t) {
+          const int c = 2 * pairs[t];
+          const FxOp x0 = fx_load(row[c]), x1 = fx_load(row[c + 1]);
+          const FxOp a1 = fx_load(U[2 * t + 1]), a0 = fx_load(U[2 * t]);
+          const FxOp b1 = fx_load(U[N + 2 * t + 1]), b0 = fx_load(U[N + 2 * t]);
+          fx_mac(ca, x0, -x0.hi, a1);
+          fx_mac(cb, x0, -x0.hi, b1);
+          fx_mac(ca, x1, -x1.hi, a0);
+          fx_mac(cb, x1, -x1.hi, b0);
+        }
+        const int sh = 27 + ex[k + 1] - ex[k] - ex[1];
+        V[k * 2 * N + l] = fx_entry(ca, sh, over);
+        V[k * 2 * N + N + l] = fx_entry(cb, sh, over);
+      }
       __syncwarp();
     }
-    if (over) {
-      if (lane == 0) {
-        P.ok[w.pat] = 0;
-        P.kparts[w.part] = make_double2(0.0, 0.0);
+    // the walks' sums, one a lane
+    for (int t = l; l < L && t < 3 * h; t += L) {
+      const int k = t / 3 + 1, type = t - 3 * (k - 1);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (k == 1) {
+        if (type == 1) {
+          const int4 e = M[2 * p * ld + 2 * p + 1];
+          const float u = unit[1];
+          const float hr = (float)e.x, hi = (float)e.y;
+          v = dfc_norm(make_float4(hr * u, hi * u, ((float)(e.x - (int)hr) + __int_as_float(e.z)) * u,
+                                   ((float)(e.y - (int)hi) + __int_as_float(e.w)) * u));
+        }
+      } else {
+        const int i = (k - 2) >> 1, j = k - 2 - i;
+        const int4* x = V + i * 2 * N + (type == 2 ? N : 0);
+        const int4* y = V + j * 2 * N + (type == 0 ? 0 : N);
+        Fx c = fx_zero();
+#pragma unroll 2
+        for (int r2 = 0; r2 < N; ++r2) {
+          const FxOp xr = fx_load(x[r2]);
+          fx_mac(c, xr, -xr.hi, fx_load(y[r2 ^ 1]));
+        }
+        const float2 re = df_from(c.rh, c.rm, unit[k]), im = df_from(c.ih, c.im, unit[k]);
+        v = make_float4(re.x, im.x, re.y, im.y);
       }
+      mom[t] = v;
+    }
+    __syncwarp();
+    // coefficient k of D_S = 1 - 2 b + b^2 - a c, one a lane
+    for (int k = l + 1; l < L && k <= h; k += L) {
+      float4 c = dfc_scale(mom[3 * (k - 1) + 1], -2.0f);
+#pragma unroll 1
+      for (int i = 1; i < k; ++i) {
+        const float4 bi = mom[3 * (i - 1) + 1], ai = mom[3 * (i - 1)];
+        dfc_mac(c, bi, mom[3 * (k - i - 1) + 1]);
+        dfc_mac(c, make_float4(-ai.x, -ai.y, -ai.z, -ai.w), mom[3 * (k - i - 1) + 2]);
+      }
+      if (active) delta[(int64_t)mask * h + k - 1] = dfc_norm(c);
+    }
+    __syncwarp();
+  }
+  if (over) P.ok[b] = 0;
+}
+
+// The last pair's factor and the product with the subset before, a thread per
+// subset. Masks below 256 by one block per matrix, level after level (`level`
+// < 0); the masks with last pair `level` >= 8 by 2^level / 256 blocks a matrix.
+// A block's sum |f|_1 and its rounding go to parts[mask >> 8].
+__global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, const TermsChunk C, int level) {
+  __shared__ double red[2][256];
+  __shared__ float cn[kMaxH + 1];
+  dependency_wait();
+  int g = 0, bid = blockIdx.x;
+  const int per = level < 0 ? 1 : 1 << (level - 8);
+  for (; g < C.n_groups; ++g) {
+    const int blocks = (C.g[g].n >> 1) > level ? C.g[g].count * per : 0;
+    if (bid < blocks) break;
+    bid -= blocks;
+  }
+  if (g == C.n_groups) return;
+  const TermsGroup G = C.g[g];
+  const int n = G.n, h = n >> 1, q = bid / per, sub = bid - q * per, b = P.order[G.first + q];
+  if (P.ok[b] == 0) return;
+  int4* base = reinterpret_cast<int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
+  float4* delta = reinterpret_cast<float4*>(base + n * n);
+  float4* Gs = delta + ((int64_t)h << h);  // coefficient k of G_S at [k - 1][S], S without pair h - 1
+  const int64_t gl = (int64_t)1 << (h - 1);
+  double2* parts = reinterpret_cast<double2*>(Gs + gl * h);
+  const int* ex = P.exps + (int64_t)b * kExpStride;
+  if (threadIdx.x >= 1 && (int)threadIdx.x <= h) {
+    // rounding of coefficient k of a, b, c, in its units: up to n products of
+    // entries off by 2^-50 of their range, independently, with entries of a
+    // quarter of theirs at most (the room): sqrt(n) 2^-51 is several times that
+    const int k = threadIdx.x, i = (k - 2) >> 1;
+    const int e = (k == 1) ? ex[1] - 48 - ex[kExpUnit] : ex[i + 1] + ex[k - 2 - i + 1] - 51 - k * ex[kExpUnit];
+    cn[k] = sqrtf((float)n) * pow2f(max(min(e, 100), -120));
+  }
+  __syncthreads();
+  double kap = 0.0, noise = 0.0;
+  // y = D^{-1/2} of subset S in place of its D: k y_k = -sum_i (k - i / 2) d_i y_{k-i}
+  auto root = [&](int S) {
+    float4* d = delta + (int64_t)S * h;
+    float4 dl[kMaxH], y[kMaxH];
+#pragma unroll 1
+    for (int k = 0; k < h; ++k) dl[k] = d[k];
+#pragma unroll 1
+    for (int k = 1; k <= h; ++k) {
+      float4 c = dfc_scale(dl[k - 1], 0.5f * k);  // i = k, y_0 = 1
+#pragma unroll 1
+      for (int i = 1; i < k; ++i) dfc_mac(c, dfc_scale(dl[i - 1], (float)k - 0.5f * i), y[k - i - 1]);
+      // times -1/k as a pair of floats
+      const float r = __frcp_rn((float)k), rl = __fmul_rn(__fmaf_rn(-r, (float)k, 1.0f), r);
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      c = dfc_norm(c);
+      df_mac(o.x, o.z, c.x, c.z, -r, -rl);
+      df_mac(o.y, o.w, c.y, c.w, -r, -rl);
+      y[k - 1] = dfc_norm(o);
+      d[k - 1] = y[k - 1];
+    }
+  };
+  // coefficient k of G_S = G_S' y; at k = h counts f_S and its rounding
+  auto grow = [&](int S, int p, int k) {
+    const int Sp = S ^ (1 << p);
+    const float4* y = delta + (int64_t)S * h;
+    float4 c = y[k - 1];
+    float size = dfc_abs1(c), nz = cn[h];
+    if (Sp != 0) {
+      const float4* gp = Gs + Sp;
+      const float4 t = gp[(k - 1) * gl], one = make_float4(1.f, 0.f, 0.f, 0.f);
+      size += dfc_abs1(t);
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+      for (int i = 1; i < k; ++i) {
+        const float4 g0 = gp[(i - 1) * gl], y0 = y[k - i - 1];
+        dfc_mac(a, g0, y0);
+        size += dfc_abs1(g0) * dfc_abs1(y0);
+        if (k == h) nz += cn[k - i] * dfc_abs1(g0);
+      }
+      dfc_mac(a, one, c);
+      dfc_mac(a, one, t);
+      c = dfc_norm(a);
+    }
+    if (p < h - 1) Gs[(k - 1) * gl + S] = c;
+    if (k == h) {
+      nz += 0x1p-42f * size;  // rounding of the series themselves
+      kap += fabs((double)c.x + (double)c.z) + fabs((double)c.y + (double)c.w);
+      noise += 4.0 * (double)nz;  // the pairs before this one too: up to 14 independent shares
+    }
+  };
+  if (level < 0) {
+    // a thread per subset, then per subset and coefficient of a level
+    const int low = min(h, 8);
+    if (threadIdx.x >= 1 && (int)threadIdx.x < (1 << low)) root(threadIdx.x);
+    for (int p = 0; p < low; ++p) {
+      __syncthreads();
+      if (p < h - 1) {
+        for (int t = threadIdx.x; t < h << p; t += blockDim.x) grow((1 << p) + (t & ((1 << p) - 1)), p, h - (t >> p));
+      } else if ((int)threadIdx.x < (1 << p)) {
+        grow((1 << p) + threadIdx.x, p, h);
+      }
+    }
+  } else {
+    const int S = (1 << level) + sub * 256 + threadIdx.x;
+    root(S);
+    for (int k = (level < h - 1) ? 1 : h; k <= h; ++k) grow(S, level, k);
+  }
+  red[0][threadIdx.x] = kap;
+  red[1][threadIdx.x] = noise;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if (threadIdx.x < o) {
+      red[0][threadIdx.x] += red[0][threadIdx.x + o];
+      red[1][threadIdx.x] += red[1][threadIdx.x + o];
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) parts[level < 0 ? 0 : per + sub] = make_double2(red[0][0], red[1][0]);
+}
+
+// One warp per matrix: the sum over its parts, in its own units again; a matrix
+// that left the range, or whose rounding estimate is above 2^-33 of the sum, goes
+// to the FP64 kernel.
+__global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P, const TermsChunk C) {
+  dependency_wait();
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const TermsGroup& last = C.g[C.n_groups - 1];
+  const int mats = last.begin + last.count;
+  bool redo = false;
+  for (int m = blockIdx.x * wpb + (threadIdx.x >> 5); m < mats; m += gridDim.x * wpb) {
+    int g = 0;
+    while (g + 1 < C.n_groups && m >= C.g[g + 1].begin) ++g;
+    const TermsGroup& G = C.g[g];
+    const int n = G.n, h = n >> 1, q = m - G.begin, b = P.order[G.first + q];
+    if (P.skip != nullptr && P.skip[b] != 0) {
+      if (lane == 0) P.ok[b] = 1;  // nothing for the FP64 kernel either
       continue;
     }
-    double kap = 0.0, noise = 0.0;
-    int staged = 0;
-
-    // the exponential series (as in haf_subsets_kernel) of one staged subset
-    // per lane; d f / d tr_k = e_{h-k} / (2k) carries the traces' rounding
-    auto flush = [&]() {
-      if (lane < staged) {
-        double2 e[kMaxH];
-        longlong2* raw = stage + lane * sts;
-        double2* pq = reinterpret_cast<double2*>(raw);
-#pragma unroll 1
-        for (int k = 0; k < h; ++k) {
-          const longlong2 v = raw[k];
-          pq[k] = make_double2((double)v.x * sc[k], (double)v.y * sc[k]);
-        }
-        double2 f = mk<double>(1.0, 0.0);
-        double nz = cn[h - 1];
-#pragma unroll 1
-        for (int k = 1; k <= h; ++k) {
-          double2 a = pq[k - 1];
-#pragma unroll 1
-          for (int j = 1; j < k; ++j) a = cfma<double>(pq[j - 1], e[k - j], a);
-          const double c = tab.inv2k[k];
-          f = mk<double>(a.x * c, a.y * c);
-          if (k < h) {
-            e[k] = f;
-            nz = fma(cn[h - k - 1], fabs(f.x) + fabs(f.y), nz);
-          }
-        }
-        kap += fabs(f.x) + fabs(f.y);
-        noise += nz;
-      }
-      staged = 0;
-      __syncwarp();
-    };
-
-    for (int s = s_first; s <= s_last; ++s) {
-      const int E = s * (s + 1) / 2, D = s * (s - 1) / 2;
-      const int L = terms_lanes(s, h, P.warp_bytes, P.stage_h);
-      const int G = 32 / L, g = lane / L, l = lane - g * L;
-      int4* buf = reinterpret_cast<int4*>(gbase + (size_t)g * terms_group_bytes(s, h, L));
-      int* pairs = reinterpret_cast<int*>(buf + sched_nbuf(h) * 4 * E);
-      const int count = whole ? tab.binom[h][s] : w.count, rank0 = whole ? 0 : w.rank0;
-      const int rounds = (count + G - 1) / G;
-      unsigned gmask = 0;
-      for (int rd = 0; rd < rounds; ++rd) {
-        if (staged + G > slots) flush();
-        const int js = g * rounds + rd;
-        const bool active = js < count;
-        if (rd == 0) {
-          int r = rank0 + (active ? js : 0), c = h - 1;
-          for (int i = s; i >= 1; --i) {
-            while (tab.binom[c][i] > r) --c;
-            r -= tab.binom[c][i];
-            gmask |= 1u << c;
-            --c;
-          }
-        } else if (active) {  // the next larger mask with s bits
-          const unsigned u = gmask & (0u - gmask), v = gmask + u;
-          gmask = v + (((v ^ gmask) >> 2) >> (__ffs(u) - 1));
-        }
-        {
-          unsigned m = gmask;
-          for (int t = 0; t < s; ++t) {
-            if ((t & (L - 1)) == l) pairs[t] = __ffs(m) - 1;
-            m &= m - 1;
-          }
-        }
-        __syncwarp();
-        // R_1 (and R_2 from the pair sums): the subset's blocks
-        const bool have2 = sums != nullptr && h >= 3;
-        const int klo = (int)(gmask & ((1u << hl) - 1)), khi = (1 << hl) + (int)(gmask >> hl);
-        // (the loads of four entries are issued before the first is used)
-        for (int f0 = l; f0 < 4 * E; f0 += 4 * L) {
-          int4 v[4], x[4], y[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int f = f0 + u * L, e = f >> 2, el = f & 3;
-            if (f < 4 * E) {
-              int r, c;
-              if (e >= D) {
-                r = c = e - D;
-              } else {
-                const int z = rc[e];
-                r = z & 255;
-                c = z >> 8;
-              }
-              const int src = blk_index(pairs[r], pairs[c], h);
-              v[u] = __ldg(mat + 4 * src + el);
-              if (have2) {
-                const int4* q = sums + ((int64_t)src * W) * 4 + el;
-                x[u] = __ldg(q + 4 * klo);
-                y[u] = __ldg(q + 4 * khi);
-              }
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const int f = f0 + u * L, e = f >> 2, el = f & 3;
-            if (f < 4 * E) {
-              buf[el * E + e] = v[u];
-              if (have2) {
-                const int2 re = fx_pack(x[u].x + y[u].x, __int_as_float(x[u].z) + __int_as_float(y[u].z), over);
-                const int2 im = fx_pack(x[u].y + y[u].y, __int_as_float(x[u].w) + __int_as_float(y[u].w), over);
-                buf[4 * E + el * E + e] = make_int4(re.x, im.x, re.y, im.y);
-              }
-            }
-          }
-        }
-        __syncwarp();
-        longlong2* const row = stage + (staged + g) * sts;
-        unsigned pw = 1;
-        longlong2 wait = make_longlong2(0, 0);
-        int wait_k = 0;  // 0: none waiting
-        for (int o = 0; o < kMaxOps; ++o) {
-          const SchedOp op = c_sched[h][o];
-          if (op.kind == kEnd) break;
-          const int ka = (pw >> (4 * op.a)) & 15, kb = (pw >> (4 * op.b)) & 15;
-          const int4* Ra = buf + op.a * 4 * E;
-          const int4* Rb = buf + op.b * 4 * E;
-          if (op.kind == kProd) {
-            if (!(have2 && ka + kb == 2))
-              fx_prod(buf + op.k * 4 * E, Ra, Rb, rc, s, E, 27 + ex[ka + kb] - ex[ka] - ex[kb], l, L, over);
-            pw = (pw & ~(15u << (4 * op.k))) | (unsigned)(ka + kb) << (4 * op.k);
-          } else {
-            // the lanes' shares are summed two traces at a time, as group_sum2
-            // does (half the lanes carry one, half the other); they are whole
-            // numbers, so the order does not matter
-            const longlong2 t = (op.kind == kTr1) ? fx_tr1(Ra, s, E, l, L) : fx_tr2(Ra, Rb, s, E, l, L);
-            if (L == 1) {
-              row[op.k - 1] = active ? t : make_longlong2(0, 0);
-            } else if (wait_k == 0) {
-              wait = t;
-              wait_k = op.k;
-            } else {
-              const int half = L >> 1;
-              const bool up = (l & half) != 0;
-              const longlong2 out = up ? wait : t;
-              longlong2 keep = up ? t : wait;
-              keep.x += __shfl_xor_sync(FULL, out.x, half);
-              keep.y += __shfl_xor_sync(FULL, out.y, half);
-              for (int off = half >> 1; off > 0; off >>= 1) {
-                keep.x += __shfl_xor_sync(FULL, keep.x, off);
-                keep.y += __shfl_xor_sync(FULL, keep.y, off);
-              }
-              if ((l & (half - 1)) == 0) row[(up ? op.k : wait_k) - 1] = active ? keep : make_longlong2(0, 0);
-              wait_k = 0;
-            }
-          }
-          __syncwarp();
-        }
-        if (wait_k != 0) {  // uniform over the warp
-          for (int off = L >> 1; off > 0; off >>= 1) {
-            wait.x += __shfl_xor_sync(FULL, wait.x, off);
-            wait.y += __shfl_xor_sync(FULL, wait.y, off);
-          }
-          if (l == 0) row[wait_k - 1] = active ? wait : make_longlong2(0, 0);
-          __syncwarp();
-        }
-        staged += G;
-        if (staged == slots || (rd == rounds - 1 && s == s_last)) flush();
+    double K = 0.0, noise = 0.0;
+    const bool done = P.ok[b] != 0;
+    if (done) {
+      const int4* base = reinterpret_cast<const int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
+      const double2* parts = reinterpret_cast<const double2*>(base + n * n + ((int64_t)h << h) + ((int64_t)h << (h - 1)));
+      for (int i = lane; i < (h > 8 ? 1 << (h - 8) : 1); i += 32) {
+        K += parts[i].x;
+        noise += parts[i].y;
       }
     }
     for (int off = 16; off > 0; off >>= 1) {
-      kap += __shfl_xor_sync(FULL, kap, off);
-      noise += __shfl_xor_sync(FULL, noise, off);
-    }
-    if (__any_sync(FULL, over) && lane == 0) P.ok[w.pat] = 0;
-    if (lane == 0) P.kparts[w.part] = make_double2(kap, noise);
-  }
-}
-
-// One warp per matrix: the sum over its items; a matrix that left the range,
-// or whose rounding bound is above 2^-33 of the sum, goes to the FP64 kernel,
-// whose item count the last block sets (0 where no matrix does).
-__global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P) {
-  dependency_wait();
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
-  bool redo = false;
-  for (int b = blockIdx.x * wpb + (threadIdx.x >> 5); b < P.batch; b += gridDim.x * wpb) {
-    const PatDesc d = P.pats[b];
-    const bool mine = d.n >= 2 && !(d.n & 1) && !(P.skip != nullptr && P.skip[b] != 0);
-    double K = 0.0, noise = 0.0;
-    bool fine = true;
-    if (mine) {
-      for (int q = d.item_begin + lane; q < d.item_end; q += 32) {
-        const double2 v = P.kparts[q];
-        K += v.x;
-        noise += v.y;
-      }
-      int span = 1;
-      while (span < min(32, d.item_end - d.item_begin)) span <<= 1;
-      for (int off = span >> 1; off > 0; off >>= 1) {
-        K += __shfl_xor_sync(0xffffffffu, K, off);
-        noise += __shfl_xor_sync(0xffffffffu, noise, off);
-      }
-      if (lane == 0) fine = P.ok[b] != 0 && noise <= 0x1p-33 * K && K < INFINITY;
+      K += __shfl_xor_sync(0xffffffffu, K, off);
+      noise += __shfl_xor_sync(0xffffffffu, noise, off);
     }
     if (lane == 0) {
-      P.ksum[b] = K;
+      const bool fine = done && noise <= 0x1p-33 * K && K > 0x1p-90 && K < 0x1p120;
+      P.ksum[b] = fine ? ldexp(K, h * P.exps[(int64_t)b * kExpStride + kExpUnit]) : 0.0;
       P.ok[b] = fine ? 1 : 0;
       redo |= !fine;
     }
   }
-  if (redo) atomicAdd(P.n_redo, 1);
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0 && atomicAdd(P.blocks_done, 1u) == gridDim.x - 1) {
-    __threadfence();
-    *P.fp64_items = __ldcg(P.n_redo) ? P.n_items : 0;
-  }
+  if (redo) *P.fp64_items = P.n_items;  // (zero before the first chunk; every writer writes the same)
 }

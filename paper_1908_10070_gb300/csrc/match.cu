@@ -177,11 +177,11 @@ __global__ void __launch_bounds__(kMatchThreads) match_small_kernel(const MatchL
   __shared__ int rows[32 * kMatchSmallMax];
   __shared__ int64_t s_off[32];
   __shared__ int s_ld[32], s_any;
+  load_binom(bin);
+  dependency_wait();
   const MatchTile T = L.tiles[blockIdx.x];
   const int n = T.n, lp = T.lp, P = 1 << lp;
   if (threadIdx.x == 0) s_any = (L.skip == nullptr);
-  load_binom(bin);
-  dependency_wait();
   __syncthreads();
   layer_bases(bin, lb, n);
   for (int t = threadIdx.x; t < n << lp; t += blockDim.x) {
@@ -379,7 +379,7 @@ cudaError_t launch_match_small(const MatchLaunch& L, int tiles, size_t smem, cud
   return launch_dependent(match_small_kernel, dim3(tiles), kMatchThreads, smem, st, L);
 }
 
-cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t st) {
+cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, bool shared, cudaStream_t st) {
   if (C.n_groups <= 0) return cudaSuccess;
   const MatchGroup& last = C.g[C.n_groups - 1];
   const int mats = last.begin + last.count;
@@ -391,6 +391,7 @@ cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, cudaStream_t 
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, match_layer_kernel, kMatchThreads, 0);
   if (e != cudaSuccess) return e;
+  if (shared) resident = std::min(resident, 3);  // beside the terms' blocks (24 warps keep the FP64 pipe busy)
   if ((e = launch_dependent(match_head_kernel, dim3(mats), kMatchThreads, 0, st, L, C)) != cudaSuccess) return e;
   constexpr int wpb = kMatchThreads / 32;
   for (int i = 2; i < nmax - kMatchTail; ++i) {
