@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void sum_add(Comp<double>& a, double v) {
 // digits: C depends on the pattern only, y and the high share on the high
 // digits only, and x . y splits over the two groups of low modes. So a term
 // forms its Q in three complex additions from tables instead of the d^2 / 2
-// multiply-adds of the quadratic form, and takes 41 FP64 operations at h = 12
+// multiply-adds of the quadratic form, and takes 39 FP64 operations at h = 12
 // where it took 170 (d = 8); the tables add about a quarter. The FP64 pipe
 // bounds it: 512 patterns of n = 24 in 8 modes (2^15 terms each) went from
 // 3.5 to 1.75 ms (whole call). The sum keeps its rounding errors (Knuth's two-sum, once a
@@ -1404,12 +1404,12 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
           br = tr;
         }
       }
-      double f = W.w[l];
+      double f = W.w[l] * wh;
       if (2 * (base + l) + 1 == T) f *= 0.5;
       const double vr = f * pr, vi = f * pi;
-      sum_add(re, wh * vr);
-      sum_add(im, wh * vi);
-      kp = fma(fabs(wh), fabs(vr) + fabs(vi), kp);
+      sum_add(re, vr);
+      sum_add(im, vi);
+      kp += fabs(vr) + fabs(vi);
     }
     __syncwarp();
   }

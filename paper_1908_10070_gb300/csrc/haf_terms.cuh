@@ -245,12 +245,17 @@ __device__ __forceinline__ float4 dfc_scale(const float4& a, float f) {
   return make_float4(x, y, __fmaf_rn(a.z, f, __fmaf_rn(a.x, f, -x)), __fmaf_rn(a.w, f, __fmaf_rn(a.y, f, -y)));
 }
 __device__ __forceinline__ float dfc_abs1(const float4& a) { return fabsf(a.x) + fabsf(a.y); }
-// (h + m) unit as a pair of floats.
+// (h + m) unit as a pair of floats, |h| < 2^61: the top 31 and the low 30 bits,
+// each as a float and what that leaves, by 32-bit conversions (64-bit ones run
+// on the FP64 pipe, which they held a quarter of the time).
 __device__ __forceinline__ float2 df_from(long long h, float m, float unit) {
-  const float hi = __ll2float_rn(h);
-  const float lo = __fadd_rn(__ll2float_rn(h - __float2ll_rn(hi)), m);
-  const float s = __fadd_rn(hi, lo);
-  return make_float2(s * unit, __fsub_rn(lo, __fsub_rn(s, hi)) * unit);
+  const int a = (int)(h >> 30), r = (int)h & 0x3fffffff;
+  const float fa = (float)a, fr = (float)r, hi = fa * 0x1p30f;
+  const float rest = __fadd_rn((float)(a - (int)fa) * 0x1p30f, __fadd_rn((float)(r - (int)fr), m));
+  const float t = __fadd_rn(hi, fr);  // (|hi| >= 2^30 > fr, or hi = 0)
+  const float lo = __fadd_rn(__fsub_rn(fr, __fsub_rn(t, hi)), rest);
+  const float s = __fadd_rn(t, lo);
+  return make_float2(s * unit, __fsub_rn(lo, __fsub_rn(s, t)) * unit);
 }
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }  // -126 <= e <= 127
 
