@@ -16,7 +16,6 @@ from __future__ import annotations
 
 import argparse
 import gc
-import hashlib
 import json
 import os
 import subprocess
@@ -31,27 +30,6 @@ sys.path.insert(0, ROOT)
 
 import workloads as W  # noqa: E402
 
-# DRAM bytes (read + write) per launch of haf_subsets_kernel<double> on the
-# headline workload, from one ncu capture (profiles/haf_subsets_fp64_m64_n16.md).
-# Reported only while the kernel's sources are the ones the capture was taken
-# from; any change to them makes the figure stale and the bench reports null.
-NCU_TRAFFIC = {"sources_sha256": "b3893c0911fdf91c94646019a9ce2a1895d97f49e64da263ebfd6285d53d6635", "bytes_per_launch": 367626240.0,
-               # executed FP64 flops per cycle (DFMA x 2 + DADD + DMUL) over the 608 peak
-               "executed_fp64_frac": 0.881}
-KERNEL_SOURCES = ("paper_1908_10070_gb300/csrc/haf_subsets.cu", "paper_1908_10070_gb300/csrc/gbs_internal.cuh")
-
-
-def capture_current():
-    h = hashlib.sha256()
-    for f in KERNEL_SOURCES:
-        with open(os.path.join(ROOT, f), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest() == NCU_TRAFFIC["sources_sha256"]
-
-
-def measured_traffic():
-    return NCU_TRAFFIC["bytes_per_launch"] if capture_current() else None
-
 WORKLOAD = "batched_m64_n16"
 WORKLOAD_DESC = "M=64 Haar U seed 1, r~U[0.6,1.0], 4096 collision-free n=16 patterns, "
 METRIC = "GBS output probs/sec at n=16/24/30 vs FP64 oracle; p50/p99 request latency"
@@ -59,12 +37,38 @@ UNIT = "probs/s"
 SMS, SM_MHZ_MAX, FP64_FLOP_PER_CLK_SM = 152, 2070.0, 4.0
 
 
-def model_flops(n: int) -> float:
-    """Algorithmic FP64 flops of one Hafnian: sum_s C(h,s) * 8 (2s)^3 = 64 2^{h-3} h^2 (h+3)."""
+def matching_macs(n: int) -> int:
+    """Complex multiply-adds of one Hafnian by matchings of a growing prefix."""
+    from math import comb
+
+    if n % 2 or n < 2:
+        return 0
+    return sum(j * comb(n - i, j) for i in range(1, n + 1) for j in range(i % 2, min(i, n - i) + 1, 2))
+
+
+def term_macs(n: int) -> int:
+    """Complex multiply-adds of one matrix's terms f(X A_S), which the error
+    estimate sums: per subset of s pairs, (h - 1) // 2 steps of two vectors of
+    N = 2 (s - 1) entries, the walks' sums, and the three series products."""
+    from math import comb
+
     h = n // 2
-    if n % 2 or h == 0:
-        return 0.0
-    return 64.0 * 2.0 ** (h - 3) * h * h * (h + 3)
+    if n % 2 or h < 1:
+        return 0
+    return sum(comb(h, s) * ((h - 1) // 2 * 2 * (2 * s - 2) ** 2 + 3 * (h - 1) * (2 * s - 2) + 2 * h * (h - 1))
+               for s in range(1, h + 1))
+
+
+def model_flops(n: int, terms: bool = True) -> float:
+    """Flops of one FP64 result, 8 per complex multiply-add: the matchings (FP64
+    pipe) and, with the error estimate, the terms (whole numbers and FP32)."""
+    return 8.0 * (matching_macs(n) + (term_macs(n) if terms else 0))
+
+
+def fixed_point_peak_tflops() -> float:
+    """Peak of the terms' complex multiply-add, 4 IMAD.WIDE and 8 FFMA: measured
+    at 32 clocks a warp and SM quarter, so one a clock and quarter, 8 flops each."""
+    return SMS * 4 * 8.0 * SM_MHZ_MAX * 1e6 / 1e12
 
 
 def fp64_peak_tflops() -> float:
@@ -75,50 +79,34 @@ def fp64_peak_tflops() -> float:
 
 def chain_sample_flops(n: int, m: int, samples: int) -> float:
     """Algorithmic FP64 flops of `samples` Algorithm 1 samples of n photons over
-    m modes, as the library forms them (8 flops per complex multiply-add): per
-    step k, the Theorem 1 products Haf(W_sigma) Haf(W_{rho \\ sigma}) over the
-    sets rho and sizes |sigma| inside the theorem's ranges (one of each pair
-    G(rho, j) = G(rho, |rho| - j); the sets without the new photon once per
-    sample on steps of at least 2^24 subsets), the row expansions of the new
-    sub-Hafnians of the sizes read (|T'| products each), and the chosen mode's
-    cache update (|T'| products for each odd T' of the prefix)."""
+    m modes, as the library forms them (8 flops per complex multiply-add, 4 per
+    squared modulus): per step k, the Hermitian form over the prefix's k - 1
+    positions (or, where the sets are few, none), what the prefix's modes have
+    more, the sum over the sets without the new photon, the form's value for
+    every mode, and the chosen mode's new sub-Hafnians."""
     from math import comb
 
-    def in_range(k, mu, ja, jb):
+    def sizes(k):
         lo = max(0, 2 * k - n)
-        return ja >= lo and jb >= lo and max(0, 3 * k - ja - jb - n) <= mu <= k - max(ja, jb)
+        return [c for c in range(0, k + 1, 2)
+                if any(ja >= lo and jb >= lo and max(0, 3 * k - ja - jb - n) <= k - c <= k - max(ja, jb)
+                       for ja in range(0, c + 1, 2) for jb in range(0, c + 1, 2))]
 
-    def rho_work(k, c):  # subsets one set rho of size c enumerates
-        w = 0
-        for ja in range(0, c + 1, 2):
-            a, a2 = ja // 2, c // 2 - ja // 2
-            used = any(in_range(k, k - c, ja, jb) for jb in range(0, c + 1, 2))
-            twin = a2 < a and any(in_range(k, k - c, 2 * a2, jb) for jb in range(0, c + 1, 2))
-            if used and not twin:
-                w += comb(c, min(ja, c - ja))
-        return w
-
-    def count(k, c, part):  # sets of size c: all, with position k-1, without it
-        if part == 0:
-            return comb(k, c)
-        if part == 1:
-            return comb(k - 1, c - 1) if c >= 1 else 0
-        return comb(k - 1, c)
-
-    macs = 0
-    items = samples * m
-    for k in range(1, n + 1):
-        work = {p: sum(count(k, c, p) * rho_work(k, c) for c in range(0, k + 1, 2)) for p in (0, 1, 2)}
-        if items * work[0] >= 1 << 24:
-            macs += items * work[1] + samples * work[2]
+    macs, later = 0.0, set()
+    for k in range(n, 0, -1):
+        kp, S = k - 1, [c for c in sizes(k)]
+        odd = [c - 1 for c in S if 1 <= c - 1 <= kp]
+        sets = sum(comb(kp, t) for t in odd)
+        macs += 0.5 * sum(comb(kp, c) for c in S)
+        if 2 * sets <= kp:
+            macs += m * sum(comb(kp, t) * (t + 0.5) for t in odd)
         else:
-            macs += items * work[0]
-        sizes = {s for c in range(0, k + 1, 2) for ja in range(0, c + 1, 2) for jb in range(0, c + 1, 2)
-                 if in_range(k, k - c, ja, jb) for s in (ja, c - ja)}
-        macs += items * sum(comb(k - 1, s - 1) * (s - 1) for s in sizes if s >= 2 and s % 2 == 0)
-        if k < n:
-            macs += samples * sum(comb(k - 1, t) * t for t in range(1, k, 2))
-    return 8.0 * macs
+            macs += sum(kp * (kp - 1) / 2 * (comb(kp - 2, t - 2) if t >= 2 else 0) + kp * comb(kp - 1, t - 1) / 2 for t in odd)
+            macs += kp * sum(comb(kp - 1, t) * (t + 0.5) for t in odd if t <= kp - 1)
+            macs += m * kp * (kp + 1) / 2
+        macs += sum(comb(kp, c - 1) * (c - 1) for c in later if 1 <= c - 1 <= kp)
+        later |= set(S) | {c - 2 for c in S if c >= 2} | {c - 2 for c in later if c >= 2}
+    return 8.0 * macs * samples
 
 
 def fp32_peak_tflops() -> float:
@@ -376,8 +364,11 @@ def main():
     e2e_s = (time.perf_counter() - t0) / e2e_steps
     assert np.array_equal(hh, hf.cpu().numpy()), "host and device paths disagree"
 
-    flops = model_flops(16) * b
-    peak = fp64_peak_tflops() if prec == gbs.FP64 else fp32_peak_tflops()
+    # the FP64 route: its terms set the time (whole numbers and FP32); the
+    # float kernel is counted by one N x N complex product per subset
+    fp64 = prec == gbs.FP64
+    flops = (model_flops(16) if fp64 else 64.0 * 2 ** 5 * 64 * 11) * b
+    peak = fixed_point_peak_tflops() if fp64 else fp32_peak_tflops()
     achieved = flops / (t_kern * 1e-3) / 1e12
     # the FP64 pipe's measured throughput (DFMA microbenchmark in the library),
     # with the clocks it ran at: the second denominator of the fraction
@@ -394,27 +385,26 @@ def main():
                    "autotuned_rounds_per_item": tuned_rounds},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
-                     "traffic": measured_traffic() if prec == gbs.FP64 else None,
-                     # the same capture's executed FP64 rate (the flop model above counts
-                     # one N x N complex product per subset; the route executes more)
-                     "ncu_executed_fp64_frac": (NCU_TRAFFIC["executed_fp64_frac"]
-                                                if prec == gbs.FP64 and capture_current() else None),
+                     "traffic": None,
                      "hafnian_terms_per_s": b * (2 ** 8 - 1) / (t_kern * 1e-3),
-                     "kernel": "haf_subsets_kernel<%s>" % ("double" if prec == gbs.FP64 else "float"),
+                     "kernel": ("terms_delta_kernel, terms_series_kernel, match_small_kernel" if fp64
+                                else "haf_subsets_kernel<float>"),
                      "kernel_ms": t_kern,
                      "flops_per_launch": flops,
-                     "peak_note": ("FP64 from unit counts and clock (152 SM x 4 flop/clk x 2.07 GHz)"
-                                   if prec == gbs.FP64 else
+                     "peak_note": ("one complex multiply-add (4 IMAD.WIDE, 8 FFMA) a clock and SM quarter, "
+                                   "152 SM x 4 x 8 flop x 2.07 GHz" if fp64 else
                                    "FP32 from unit counts and clock (152 SM x 256 flop/clk x 2.07 GHz)"),
                      "measured_fp64_peak": measured_peak,
-                     "frac_of_measured_fp64_peak": (achieved / measured_peak) if prec == gbs.FP64 else None,
+                     "matching_flops_frac_of_measured_fp64_peak":
+                         (8.0 * matching_macs(16) * b / (t_kern * 1e-3) / 1e12 / measured_peak) if fp64 else None,
                      "measured_peak_note": "gbs_measure_fp64_peak (independent DFMA chains on every SM), "
                                            "SM clock %s MHz during it" % pclk_s.get("sm_mhz")},
         "e2e": {"value": world * b / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(idx.nbytes),
                 "d2h_bytes_per_step": int(hp.nbytes + hl.nbytes + hh.nbytes + he.nbytes)},
-        # per step: the route choice, pair terms and repeated-row kernel (FP64
-        # only), the subset kernel, finalisation
-        "gpu_launches": (5 if prec == gbs.FP64 else 2) * args.steps,
+        # per step, FP64: the route choice, the matchings, the terms' preparation,
+        # two kernels and check, the subset kernel behind them, the repeated-row
+        # kernel, finalisation; mixed: the subset kernel, finalisation
+        "gpu_launches": (9 if prec == gbs.FP64 else 2) * args.steps,
         "clocks": clk.summary(),
     }
     if rank == 0 and not args.no_cpu_baseline and world == 1 and prec == gbs.FP64:
@@ -567,12 +557,11 @@ def profile_chain(args, torch, gbs):
 
 def extras(gbs, torch, measured_peak):
     out = {}
-    peak = fp64_peak_tflops()
+    peak = fixed_point_peak_tflops()
 
-    def frac(fl, ms):
+    def frac(fl, ms):  # matchings and terms against the terms' multiply-add rate
         a = fl / (ms * 1e-3) / 1e12
-        return {"achieved_tflops": a, "frac_of_nominal_peak": a / peak,
-                "frac_of_measured_peak": (a / measured_peak) if measured_peak else None}
+        return {"achieved_tflops": a, "frac_of_fixed_point_peak": a / peak}
 
     # mixed path on the headline workload
     U, r, pats = W.workload(WORKLOAD)
@@ -625,8 +614,8 @@ def bunched(gbs, torch, reps=3):
     """M = 8, r = 1, 512 patterns of 24 photons drawn with replacement: host
     index lists take the repeated-row route chosen on the host, device index
     lists the same route chosen on the device (cost prod (c_j + 1) terms); the
-    explicit matrices B_x through gbs_hafnian_batch take the subset sum (cost
-    2^12 subsets). Wall time per batch, the routes' largest relative deviations
+    explicit matrices B_x through gbs_hafnian_batch take the matchings and, for
+    kappa, the terms of the subset sum (2^12 subsets). Wall time per batch, the routes' largest relative deviations
     and each route's largest error estimate (the subset sum cancels far more on
     bunched patterns)."""
     U, r, pats = W.workload("bunched_m8")

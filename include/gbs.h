@@ -13,12 +13,17 @@
  * s_j times (Sec. 2.3, Eq. W_s_example); equivalently B_x(i, j) = B(x_i, x_j)
  * for the index list x of the pattern (Sec. 3.2, "Step 2: change of basis").
  *
- * Haf is computed by the 2^{n/2}-subset sum whose O(n^3 2^{n/2}) cost Sec. 2.3
- * cites (Bjorklund, Gupt, Quesada): with n = 2h and pairs {2i, 2i+1},
+ * Haf is computed in one of two ways. The 2^{n/2}-subset sum whose
+ * O(n^3 2^{n/2}) cost Sec. 2.3 cites (Bjorklund, Gupt, Quesada): with n = 2h and
+ * pairs {2i, 2i+1},
  *     Haf(A) = sum_{S subset of [h]} (-1)^{h-|S|} f(X A_S),
  *     f(M)   = [x^h] det(I - x M)^{-1/2},
- * X swapping the two members of each pair. One subset term is a characteristic
- * polynomial of a 2|S| x 2|S| complex matrix.
+ * X swapping the two members of each pair. And the sum over the matchings of a
+ * growing prefix of the rows, kept for every set of later rows they use up
+ * (row expansion, Appendix A, with equal remainders taken together): at the
+ * orders accepted here 17 to 29 times fewer operations, and no cancellation
+ * beyond the Hafnian's own. The batched FP64 calls take the second up to
+ * n = 30, the mixed-precision calls, the server and the no-alloc call the first.
  *
  * Conventions for every call:
  *   - Return 0 on success or a negative GBS_E* code; gbs_last_error() gives a
@@ -55,7 +60,8 @@ extern "C" {
 #define GBS_ENOENT (-7)    /* unknown serving ticket */
 #define GBS_ECANCELED (-8) /* serving request cancelled by gbs_serve_cancel */
 
-#define GBS_FP64 0  /* per-subset arithmetic in FP64, signed sum in double-double */
+#define GBS_FP64 0  /* batched calls up to n = 30: matchings in FP64 throughout; otherwise the
+                       subset sum, its terms in FP64 and the signed sum in double-double */
 #define GBS_MIXED 1 /* power traces in FP32; their exponential series (the characteristic-
                        polynomial recurrence) in FP64 and the signed sum in double-double */
 
@@ -93,8 +99,7 @@ int gbs_kernel_copy_B(const gbs_kernel* k, double* dst, void* stream);
 /* Batched Hafnians and probabilities                                       */
 /* ------------------------------------------------------------------------ */
 
-/* Hafnians of a batch of symmetric complex matrices (Eq. HafMatch), by the
- * subset sum above.
+/* Hafnians of a batch of symmetric complex matrices (Eq. HafMatch).
  *   A_ri    concatenated matrices, complex128 interleaved, host or device;
  *           matrix b is n[b] x n[b] row-major starting at complex element
  *           offs[b]. Only the entries off the diagonal are read (no perfect
@@ -105,13 +110,18 @@ int gbs_kernel_copy_B(const gbs_kernel* k, double* dst, void* stream);
  *   kappa_out   batch doubles (host or device) or NULL: the cancellation ratio
  *               kappa_b = sum_S |f(X A_S)|_1 / |Haf(A_b)| (|z|_1 = |re|+|im|).
  * Errors: GBS_EINVAL, GBS_ERANGE (n[b] > GBS_MAX_N), GBS_ENOMEM, GBS_ECUDA. */
-/* Ordering: the subset sum pairs positions (t, t + n/2) of each matrix by
+/* With GBS_FP64 the Hafnians come from the matchings when every n[b] <= 30
+ * (measured on 80 matrices at n = 28 and 30: errors near 5e-15); asking for
+ * kappa_out, which is the subset sum's, adds that sum's terms and does not
+ * change the Hafnians' bits. A batch with a larger order takes the subset sum
+ * as a whole.
+ * Ordering: the subset sum pairs positions (t, t + n/2) of each matrix by
  * default (which keeps copies of a repeated row apart); for n >= 26 this call
  * and gbs_prob_batch first try 16 orderings on a sample of subsets and run the
  * sum in the one with the smallest sampled sum |f|. The Hafnian does not depend
- * on the ordering; the cancellation, and so the rounding error, does (measured
- * on 80 matrices at n = 28 and 30: largest error 3.5e-11 with the choice,
- * 3.1e-10 in the default order). */
+ * on the ordering; kappa, and the rounding error of a Hafnian taken from the
+ * sum, do (largest error of the sum on those 80 matrices: 3.5e-11 with the
+ * choice, 3.1e-10 in the default order). */
 int gbs_hafnian_batch(const double* A_ri, const int* n, const int64_t* offs, int batch,
                       int precision, void* stream, double* haf_ri_out, double* kappa_out);
 
@@ -144,7 +154,9 @@ int gbs_hafnian_batch_noalloc(const double* A_ri, const int* n, const int64_t* o
  *     p_out       p(s) per pattern (underflows to 0 below ~1e-308),
  *     logp_out    log p(s) (-inf when Haf = 0),
  *     haf_ri_out  Haf(B_x), 2 doubles per pattern,
- *     err_est_out estimated relative error of Haf: c * u * kappa, u the unit
+ *     err_est_out estimated relative error of Haf by the subset sum (an upper
+ *                 estimate where Haf comes from the matchings, whose error does
+ *                 not grow with kappa): c * u * kappa, u the unit
  *                 roundoff of the per-subset arithmetic and kappa the
  *                 cancellation ratio (as kappa_out of gbs_hafnian_batch):
  *                 GBS_FP64 u = 2^-53, c = n; GBS_MIXED u = 2^-24, c = min(n, 4),
@@ -153,17 +165,20 @@ int gbs_hafnian_batch_noalloc(const double* A_ri, const int* n, const int64_t* o
  * A host idx is checked on the host (GBS_ERANGE for an index >= m). A device
  * idx is checked on the device: a pattern with an out-of-range index gets NaN
  * outputs and no memory outside B is read.
- * Route: every pattern takes the subset sum of Sec. 2.3, except that with
- * GBS_FP64 a pattern whose photons are bunched into few modes (at most 16
- * distinct modes, prod_j (s_j + 1) terms costing well under the subset sum)
- * takes the repeated-row sum instead (the moment-extraction identity of Kan,
+ * Route: every pattern takes the matchings (GBS_FP64, every n[b] <= 30) or the
+ * subset sum of Sec. 2.3, except that with GBS_FP64 a pattern whose photons
+ * are bunched into few modes (at most 16 distinct modes, prod_j (s_j + 1) terms
+ * costing well under the subset sum) takes the repeated-row sum instead (the moment-extraction identity of Kan,
  * 2008; not in the paper). The choice is made on the device (a host idx is
  * copied there first), so it costs the host nothing and gives the same bits
  * for host and device lists; a batch reserves repeated-row partial slots for
  * at most 2^20 term chunks in all (patterns past that, in batch order, keep
- * the subset sum). On such patterns that route is also the accurate one: the subset sum
- * cancels strongly there (errors up to ~1e-8 measured at n = 24 in 8 modes,
- * flagged by err_est_out).
+ * the other route). On such patterns that sum's estimate is also the tighter
+ * one: the subset sum cancels strongly there (errors up to ~1e-8 measured at
+ * n = 24 in 8 modes, flagged by err_est_out). The choice does not depend on
+ * which outputs are asked for.
+ * Cost of the estimate: without err_est_out a GBS_FP64 call forms the Hafnians
+ * alone; with it the subset sum's terms too, several times the work.
  * Kept plans: the host-side plan of a call (work items, per-matrix
  * descriptors, ordering-probe tables) depends only on n[], offs[], m, the
  * precision and the launch shape, never on the index lists or matrices, so
@@ -183,9 +198,9 @@ int gbs_prob_batch(const gbs_kernel* k, const int* idx, const int* n, const int6
 int gbs_clear_plans(void);
 
 /* Instrumentation: when both are non-NULL, every later batch records `start`
- * immediately before and `stop` immediately after the kernels of its subset
- * sum (the pair terms, for n >= 26 the ordering probe and choice, and the
- * subset kernel), on the batch's stream (cudaEvent_t passed as void*), so a
+ * immediately before and `stop` immediately after the kernels of its Hafnians
+ * and terms (route choice, matchings or pair terms, for n >= 26 the ordering
+ * probe and choice, the terms or the subset kernel), on the batch's stream (cudaEvent_t passed as void*), so a
  * caller can time that work alone. Pass NULL, NULL to stop. Process-wide; not
  * for concurrent use from several threads. The paper has no counterpart
  * (measurement only). */
@@ -242,14 +257,14 @@ int gbs_sample_bruteforce(const gbs_kernel* k, int n, const double* uniforms, in
  * `batch` ordered prefixes of length k, for n-photon samples with identical
  * squeezing on every mode (the kernel's r must all be equal and > 0: the
  * theorem sums out the unsampled photons with the unitarity of W, which
- * B = U diag(tanh r_i) U^T lacks when the r_i differ). The sub-Hafnians of
- * the prefix's subsets that the sum reads come from the batched FP64 path;
- * the sums over s, s', A, B, mu of Theorem 1 are regrouped by the set
- * rho = [k] \ A (Per(S_{A,B}) = 0 unless A and B hold the same modes), and
- * only the sizes of rho and s inside the theorem's ranges are formed (a
- * team of lanes per rho, sized by the launch's work). Results are
- * deterministic for a given batch; the same prefix in batches of different
- * sizes can differ in the last bits (another split of its sums).
+ * B = U diag(tanh r_i) U^T lacks when the r_i differ). The sums over s, s', A,
+ * B, mu of Theorem 1 are regrouped by the set rho = [k] \ A (Per(S_{A,B}) = 0
+ * unless A and B hold the same modes); a matching of s with one of rho \ s is
+ * a matching of rho with some pairs marked, so the sum is one over rho of
+ * |Haf(W_rho)|^2 with weights, only the sizes inside the theorem's ranges
+ * counting. The sub-Hafnians of the prefix's subsets come from each other by
+ * row expansion (for prefixes near n, where few large ones count, from the
+ * batched FP64 path). A prefix's result does not depend on its batch.
  *   x      batch * k mode indices in [0, m), prefix b at [b * k, (b + 1) * k),
  *          host or device (read before return).
  *   k      0..min(n, 20).  n  even, <= GBS_MAX_N.
@@ -269,8 +284,9 @@ int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int batch, int
  * left-to-right sum only when u_k times the total lies within rounding of a
  * running sum. Identical squeezing only. The sampled prefix's sub-Hafnians
  * stay on the device between steps (the exponential-space variant,
- * Appendix D); those of the sets that hold the new photon come from them by
- * expanding the Hafnian along its row.
+ * Appendix D); those of the sets that hold the new photon expand along its row
+ * of B, so that a candidate's weight is a Hermitian form in that row, formed
+ * once per step.
  *   n         even, 0..20.
  *   uniforms  n numbers in [0, 1), HOST memory.
  *   x_out     n ints, HOST memory: the mode of each photon in draw order.
@@ -283,7 +299,7 @@ int gbs_sample_chain(const gbs_kernel* k, int n, const double* uniforms, void* s
  * once per group of samples.
  * Sample s equals gbs_sample_chain with uniforms[s * n .. s * n + n - 1].
  *   samples   >= 0; they go in groups of at most 2^28 / 2^n (their sub-Hafnian
- *             caches, 2^n complex doubles each, stay within 4 GB).
+ *             caches, 2^(n-1) complex doubles each, stay within 2 GB).
  *   uniforms  samples * n numbers in [0, 1), sample-major, HOST memory.
  *   x_out     samples * n ints, HOST memory, sample-major.
  * Errors: GBS_EINVAL, GBS_ERANGE, GBS_ENOMEM, GBS_ECUDA. */
