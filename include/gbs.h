@@ -22,8 +22,9 @@
  * growing prefix of the rows, kept for every set of later rows they use up
  * (row expansion, Appendix A, with equal remainders taken together): at the
  * orders accepted here 17 to 29 times fewer operations, and no cancellation
- * beyond the Hafnian's own. The batched FP64 calls take the second up to
- * n = 30, the mixed-precision calls, the server and the no-alloc call the first.
+ * beyond the Hafnian's own. The batched FP64 calls and the server's FP64
+ * requests take the second up to n = 30, the mixed-precision ones and the
+ * no-alloc call the first.
  *
  * Conventions for every call:
  *   - Return 0 on success or a negative GBS_E* code; gbs_last_error() gives a
@@ -339,7 +340,8 @@ typedef struct gbs_serve_opts {
   int max_slots;          /* requests resident on the device at once (0 = 256) */
   size_t mem_budget;      /* device bytes for request state (0 = 64 MiB) */
   int queue_capacity;     /* pending requests accepted before GBS_EAGAIN (0 = 65536) */
-  int subsets_per_step;   /* subset terms per request per step (0 = library choice) */
+  int subsets_per_step;   /* subset terms per request per step (0 = library choice), for requests
+                             that go by their subset sums */
   int use_graphs;         /* 0 or 1: replay an instantiated CUDA graph per step (default);
                              -1: launch each step's copies and kernels directly */
   double wait_timeout_s;  /* bound on any internal wait (0 = 10 s) */
@@ -351,8 +353,13 @@ typedef struct gbs_serve_opts {
 
 /* Start a server for kernel matrix k: a host thread admits requests into
  * device slots as slots and memory free up, and runs steps that advance every
- * resident request's subset sum together; partial sums stay on the device
- * between steps. Beside mem_budget the server keeps a pool of up to 256 MB
+ * resident request together. FP64 requests of n <= 30 go as a whole in one
+ * step (several large ones in several steps), by the batched call's
+ * matchings, with scratch from the library's pool; the others by their subset
+ * sums, whose partial sums stay on the device between steps, and so does an
+ * FP64 request for which no scratch can be had, or whose estimate's terms
+ * need the FP64 subset kernel. Every request is admitted by what its subset
+ * sum would need. Beside mem_budget the server keeps a pool of up to 256 MB
  * (less when max_slots requests of order max_n need less) for the pair sums
  * of FP64 requests of order >= 6; such a request is admitted once its pair
  * sums fit there. A request with n >= 26 is admitted once the ordering probe
@@ -399,8 +406,9 @@ int gbs_serve_cancel(gbs_server* s, int64_t ticket);
  * its completion event. */
 typedef struct gbs_serve_stats_t {
   int64_t steps;          /* steps launched */
-  int64_t items;          /* work items dispatched */
-  int64_t subsets;        /* subset terms dispatched */
+  int64_t items;          /* work items dispatched (for a request that went as a whole, as many
+                             as its subset sum has) */
+  int64_t subsets;        /* subset terms dispatched (likewise) */
   int64_t completed;      /* requests finished on the device */
   double step_wall_s;     /* summed step wall time (launch to detected completion) */
   double step_wall_max_s; /* longest step */
@@ -412,7 +420,8 @@ typedef struct gbs_serve_stats_t {
   double launch_max_s;    /* longest call that launches a step, of which: */
   double update_max_s;    /* longest update of a step graph's parameters */
   double submit_max_s;    /* longest submission of a step (graph launch, or the
-                             direct copies and launches without graphs) */
+                             direct copies and launches without graphs), not counting
+                             its whole requests' launches */
   int64_t probed;         /* requests whose ordering the probe chose (n >= 26) */
   int64_t cancelled;      /* requests cancelled while pending */
   int64_t alloc_waits;    /* admissions that found the memory budget used up and waited */

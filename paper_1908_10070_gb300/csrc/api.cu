@@ -885,6 +885,11 @@ static int clear_plans() {
   return e == cudaSuccess ? GBS_OK : cuda_fail(e, "synchronize before freeing kept plans");
 }
 
+// (pats | one empty item | order | tiles | lists, each rounded up)
+size_t batch_stage_bytes(int batch) {
+  return (sizeof(PatDesc) + sizeof(int) + sizeof(MatchTile) + sizeof(int) * kMaxN) * (size_t)batch + sizeof(WorkItem) +
+         5 * 256;
+}
 
 int run_batch(const BatchArgs& a) {
   cudaStream_t st = a.stream;
@@ -909,6 +914,7 @@ int run_batch(const BatchArgs& a) {
   // FP64: the Hafnians by partial matchings; the subset sum's terms are formed
   // (in fixed point) only for the error estimate made of their moduli. Tuning
   // runs time the subset sum itself.
+  if (a.stage && (a.precision != GBS_FP64 || maxn > kMatchMaxN)) return fail(GBS_EINVAL, "staged call");
   U.match = a.precision == GBS_FP64 && !a.cfg_override && maxn <= kMatchMaxN;
   U.terms = U.match && a.out3 != nullptr;
   // launch shape from the largest n (it dominates the cost); rounds per n
@@ -948,7 +954,7 @@ int run_batch(const BatchArgs& a) {
   U.pcfg = (U.probe32 && !a.cfg_override) ? get_cfg(GBS_MIXED, maxn) : cfg;
 
   // a kept plan of the same shape (untuned calls)
-  const bool cacheable = !a.cfg_override;
+  const bool cacheable = !a.cfg_override && !a.stage;
   PlanKey key;
   memset(&key, 0, sizeof(key));
   PlanEntry* pe = nullptr;
@@ -1000,11 +1006,12 @@ int run_batch(const BatchArgs& a) {
     if (U.match) plan_matching(a.n, batch, device_sm_count(), U, &order, &tiles);
     // (beside the terms: the items of the FP64 kernel behind them)
     if (U.terms) U.arena_b = terms_bytes(U);
+    const bool items = (U.terms && !a.stage) || !U.match;
     auto init = [&]() {
-      if (U.terms || !U.match) plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
+      if (items) plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
     };
     init();
-    if (!a.cfg_override && (U.terms || !U.match)) {
+    if (!a.cfg_override && items) {
       // A small batch gets smaller work items (fewer rounds each) for the same reason.
       for (int iter = 0; iter < 6 && plan.total() < want; ++iter) {
         bool shrunk = false;
@@ -1027,7 +1034,7 @@ int run_batch(const BatchArgs& a) {
     // order can need, up to kDevRepCap in all (patterns past that in batch
     // order keep the subset sum)
     constexpr int64_t kDevRepCap = (int64_t)1 << 20;
-    if (a.mode == BatchArgs::PROB && a.precision == GBS_FP64 && U.idx_elems > 0) {
+    if (a.mode == BatchArgs::PROB && a.precision == GBS_FP64 && U.idx_elems > 0 && !a.stage) {
       for (int b = 0; b < batch; ++b) U.dev_rep_cap += rep_max_chunks(a.n[b]);
       U.dev_rep_cap = std::min(U.dev_rep_cap, kDevRepCap);
     }
@@ -1080,18 +1087,23 @@ int run_batch(const BatchArgs& a) {
       U.up_b = U.tiles_at + al(sizeof(MatchTile) * std::max<size_t>(tiles.size(), 1));
     }
 
-    int rc = pinned_acquire(U.up_b + data_b, &host_stage, &slot);
-    if (rc) return rc;
+    if (a.stage) {
+      if (U.up_b + data_b > a.stage_b) return fail(GBS_EINVAL, "staging of %zu bytes is too small", a.stage_b);
+      host_stage = a.stage;
+    } else {
+      int rc = pinned_acquire(U.up_b + data_b, &host_stage, &slot);
+      if (rc) return rc;
+    }
     hs = (unsigned char*)host_stage;
     PatDesc* h_pats = (PatDesc*)hs;
-    if (U.terms || !U.match) plan.fill(h_pats, (WorkItem*)(hs + U.pats_b));
+    if (items) plan.fill(h_pats, (WorkItem*)(hs + U.pats_b));
     if (U.match) {
       memcpy(hs + U.order_at, order.data(), sizeof(int) * order.size());
       if (!tiles.empty()) memcpy(hs + U.tiles_at, tiles.data(), sizeof(MatchTile) * tiles.size());
     }
     for (int b = 0; b < batch; ++b) {
       PatDesc& d = h_pats[b];
-      if (U.match && !U.terms) {
+      if (!items) {
         d.n = a.n[b];
         d.item_begin = d.item_end = 0;
       }
@@ -1313,7 +1325,7 @@ int run_batch(const BatchArgs& a) {
       int blocks = device_sm_count() * per_sm;
       const int64_t need = (n_items + cfg.warps_per_block - 1) / cfg.warps_per_block;
       if (need < blocks) blocks = (int)need;
-      const bool timed = g_time_start && g_time_stop && !a.cfg_override;
+      const bool timed = g_time_start && g_time_stop && !a.cfg_override && !a.stage;
       if (timed) cudaEventRecord(g_time_start, st);
       if (dev_rep_cap) {
         RoutePlan RP;
@@ -1354,7 +1366,7 @@ int run_batch(const BatchArgs& a) {
         // 154, 80 patterns of n = 28 and 30 with it 22.2 -> 20.3 ms. Tiles that
         // fill the SMs gain nothing there (4096 patterns of n = 16: the terms
         // wait for room as long as the tiles run).
-        const bool shared = U.terms && n_items > 0;
+        const bool shared = U.terms && U.n_order > 0;
         const bool few = U.n_tiles <= device_sm_count();
         const bool beside = (shared && (U.match_b || few)) || (U.n_tiles && U.match_b);
         if (beside) side.begin(st);
@@ -1409,7 +1421,7 @@ int run_batch(const BatchArgs& a) {
         if (e != cudaSuccess) { ret = cuda_fail(e, "pairing choice launch"); break; }
       }
       if (U.match) {
-        if (U.terms && n_items > 0) {
+        if (U.terms && U.n_order > 0) {
           TermsLaunch T;
           memset(&T, 0, sizeof(T));
           T.src = L.src;
@@ -1432,13 +1444,15 @@ int run_batch(const BatchArgs& a) {
             if ((e = launch_terms(T, c, st)) != cudaSuccess) break;
           if (e != cudaSuccess) { ret = cuda_fail(e, "terms kernel launch"); break; }
           // the matrices the fixed-point terms gave back (normally none)
-          HafLaunch L2 = L;
-          L2.skip = d_ok;
-          L2.pt = nullptr;
-          L2.pt_off = nullptr;
-          L2.n_items_dev = T.fp64_items;
-          e = launch_haf_subsets(L2, a.precision, blocks, cfg.warps_per_block, st);
-          if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
+          if (n_items > 0) {
+            HafLaunch L2 = L;
+            L2.skip = d_ok;
+            L2.pt = nullptr;
+            L2.pt_off = nullptr;
+            L2.n_items_dev = T.fp64_items;
+            e = launch_haf_subsets(L2, a.precision, blocks, cfg.warps_per_block, st);
+            if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
+          }
         }
       } else {
         e = launch_pair_terms(L, st);
@@ -1519,7 +1533,7 @@ int run_batch(const BatchArgs& a) {
       F.p_out = dst[0];
       F.logp_out = dst[1];
       F.haf_out = dst[2];
-      F.err_out = dst[3];
+      (a.stage ? F.kappa_out : F.err_out) = dst[3];
     } else {
       F.haf_out = dst[2];
       F.kappa_out = dst[3];

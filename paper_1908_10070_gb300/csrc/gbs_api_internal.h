@@ -55,7 +55,17 @@ struct BatchArgs {
   double* out2 = nullptr;  // Haf (2 per entry)
   double* out3 = nullptr;  // err estimate (probabilities) or kappa (Hafnians)
   const TuneCfg* cfg_override = nullptr;
+  // The server's calls (FP64 probabilities of orders <= kMatchMaxN, device
+  // outputs): the upload is laid out in this pinned buffer, which stays as it
+  // is until the call's work is done; no plan is kept, no other pinned buffer
+  // taken and nothing is waited for. Each pattern's results depend on it
+  // alone: the lists are read in their own order, there is no repeated-row
+  // route, out3 gives kappa, and a pattern whose fixed-point terms are given
+  // up gets NaN in every output.
+  void* stage = nullptr;
+  size_t stage_b = 0;
 };
+size_t batch_stage_bytes(int batch);  // the most a staged call of `batch` patterns lays out
 
 int fail(int code, const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);

@@ -1000,7 +1000,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const Finalize
       const int n = d.n;
       // loads that do not depend on the partial sums go first
       const int xi = (want_p && d.idx_off >= 0 && lane < n) ? F.idx[d.idx_off + lane] : -1 - lane;
-      const int bad = (lane == 0 && F.status != nullptr) ? F.status[pb] : 0;
+      int bad = (lane == 0 && F.status != nullptr) ? F.status[pb] : 0;
       double rh = 0, rl = 0, ih = 0, il = 0, K = 0;
       if (!(n & 1) && n > 0) {
         const int rep = F.rep_half ? F.rep_half[pb] : 0;
@@ -1014,6 +1014,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const Finalize
           if (F.ok != nullptr && F.ok[pb] == 0) {
             double a = 0, b2 = 0, c2 = 0, e2 = 0;
             sum_partials(F.parts, d.item_begin, d.item_end, lane, a, b2, c2, e2, K);
+            if (d.item_begin == d.item_end) bad = 1;  // a served request: its subset items follow
           } else if (F.ksum != nullptr) {
             K = F.ksum[pb];
           }

@@ -10,6 +10,13 @@
 // request is spread over several steps while small ones that arrive meanwhile
 // are admitted, run beside it and finish first.
 //
+// FP64 requests of order <= 30 go as a whole in one step: their Hafnians by
+// matchings and their estimates by fixed-point terms, the batched path's
+// kernels, enqueued ahead of the step's items (384 requests of 12 <= n <= 26
+// at once, about half of them of odd n: 16 ms by items, now 4.1). They hold the same slots
+// and memory as if they went by items, which those whose terms are given up
+// and all others do.
+//
 // A request's work items, their partial-sum slots and the order in which its
 // partials are added depend only on its own n and precision, so its result is
 // bit-for-bit the same whether it runs alone or among others.
@@ -121,9 +128,19 @@ struct Slot {
   int64_t last_step = 0;   // the last step that carried its items or its finalisation
   int pt = -1;             // FP64: element offset of its pair sums in the pool (-1: none)
   bool pt_ready = false;   // its pair sums are computed (by an earlier step)
+  bool by_items = false;   // goes by its work items (see whole_request)
 };
 
 constexpr int kStepCap = 65536;  // work items per precision per step
+// FP64 requests of order <= kMatchMaxN go as a whole in one step, through the
+// batched path's matchings and fixed-point terms instead of their subset
+// items; the few whose terms are given up there go by their items afterwards.
+// A lone request took 98 us by items at n = 4, 157 at 12, 222 at 16, 0.45 ms
+// at 24, 0.80 at 26, 4.15 at 30, and takes 75, 86, 105, 0.28, 0.50 and 1.0.
+// A step takes such requests up to this many 2^h h^3 (the terms take 1 us per
+// 2.8e5, so about 2 ms; one is always taken), so that requests that arrive
+// meanwhile do not wait longer than for a step of items.
+constexpr double kWholeCost = 6e8;
 constexpr size_t kPtPoolBytes = (size_t)256 << 20;  // FP64 pair-sum pool
 
 // The GPU's global nanosecond timer, for the step graph's start and end stamps.
@@ -131,6 +148,13 @@ __global__ void stamp_kernel(unsigned long long* out) {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   *out = t;
+}
+// The end of a step of whole requests alone: the stamp, and the step's number.
+__global__ void end_kernel(unsigned long long* out, unsigned long long id) {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  out[0] = t;
+  out[1] = id;
 }
 
 struct Stage {
@@ -151,6 +175,14 @@ struct Stage {
   int n_items[2] = {0, 0};
   int n_pt_new = 0;      // slots whose pair sums this step computes
   std::vector<int> fin;  // slots finalised in this step, in selection order
+  // the slots that go as a whole in this step, their lists and orders, the
+  // staging of their upload, and their results (p | - | Haf | kappa, as in
+  // h_res, then the timer's stamps and the step's number)
+  std::vector<int> whole, w_idx, w_n;
+  std::vector<int64_t> w_offs;
+  unsigned char* h_whole = nullptr;
+  double* d_wres = nullptr;
+  double* h_wres = nullptr;
   std::chrono::steady_clock::time_point t_launch;
   // graph
   cudaGraph_t graph = nullptr;
@@ -482,6 +514,52 @@ cudaError_t build_graph(gbs_server* s, Stage& g) {
   return cudaGraphInstantiate(&g.exec, g.graph, 0);
 }
 
+// A slot whose request goes as a whole (kWholeCost): its result then depends
+// on it alone, as that of a request that goes by items does.
+bool whole_request(const Slot& sl) {
+  return sl.prec == GBS_FP64 && sl.n <= kMatchMaxN && !sl.by_items;
+}
+
+// A step of whole requests and nothing else.
+bool whole_only(const Stage& g) { return !g.whole.empty() && !g.n_items[0] && !g.n_items[1] && g.fin.empty(); }
+
+// Enqueue the step's whole requests and the copy of their results, ahead of
+// the rest of the step (no lock held: only the stage's own lists are read).
+// GBS_ENOMEM: nothing was enqueued for them but the start's stamp.
+int launch_whole(gbs_server* s, Stage& g) {
+  const int S = s->o.max_slots, cnt = (int)g.whole.size();
+  unsigned long long* d_stamp = (unsigned long long*)(g.d_wres + 5 * S);
+  cudaError_t e = cudaEventRecord(g.ev0, s->st);
+  if (e == cudaSuccess) {
+    stamp_kernel<<<1, 1, 0, s->st>>>(d_stamp);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return GBS_ECUDA;
+  BatchArgs a;
+  a.mode = BatchArgs::PROB;
+  a.B = s->k->B;
+  a.m = s->k->m;
+  a.log_norm_dev = s->k->dscal;
+  a.idx = g.w_idx.data();
+  a.n = g.w_n.data();
+  a.offs = g.w_offs.data();
+  a.batch = cnt;
+  a.precision = GBS_FP64;
+  a.stream = s->st;
+  a.out0 = g.d_wres;
+  a.out2 = g.d_wres + 2 * S;
+  a.out3 = g.d_wres + 4 * S;
+  a.stage = g.h_whole;
+  a.stage_b = batch_stage_bytes(S);
+  const int rc = run_batch(a);
+  if (rc != GBS_OK) return rc;
+  end_kernel<<<1, 1, 0, s->st>>>(d_stamp + 1, (unsigned long long)(g.id & 0x7fffffff));
+  e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(g.h_wres, g.d_wres, sizeof(double) * (5 * S + 2), cudaMemcpyDeviceToHost, s->st);
+  return e == cudaSuccess ? GBS_OK : GBS_ECUDA;
+}
+
 // Launch one prepared stage: the step header and one graph launch, or direct
 // copies and launches.
 // The longest parameter update (graph path) and the longest submission are
@@ -495,6 +573,14 @@ cudaError_t launch_stage(gbs_server* s, Stage& g) {
   const int S = s->o.max_slots;
   auto t0 = std::chrono::steady_clock::now();
   cudaError_t e;
+  if (s->o.use_graphs && whole_only(g)) {
+    // nothing for the graph: its end event and completion word alone
+    e = cudaEventRecord(g.ev, s->st);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(g.h_res + 5 * S + 2, g.d_wres + 5 * S + 2, sizeof(int), cudaMemcpyDeviceToHost, s->st);
+    note_max(s->stats.submit_max_s, t0);
+    return e;
+  }
   if (s->o.use_graphs) {
     // the whole step, its two events included, is one graph launch
     int* hdr = (int*)(g.h_up + s->off_hdr);
@@ -509,8 +595,10 @@ cudaError_t launch_stage(gbs_server* s, Stage& g) {
     note_max(s->stats.submit_max_s, t0);
     return e;
   }
-  e = cudaEventRecord(g.ev0, s->st);
-  if (e != cudaSuccess) return e;
+  if (g.whole.empty()) {  // (recorded ahead of the whole requests)
+    e = cudaEventRecord(g.ev0, s->st);
+    if (e != cudaSuccess) return e;
+  }
   {
     e = cudaMemcpyAsync(s->d_pats, g.h_up + s->off_pats, sizeof(PatDesc) * S, cudaMemcpyHostToDevice, s->st);
     if (e != cudaSuccess) return e;
@@ -691,6 +779,7 @@ void admit(gbs_server* s) {
     sl.last_step = 0;
     sl.pt = pto;
     sl.pt_ready = false;
+    sl.by_items = false;
     PatDesc& d = s->h_pats[si];
     d.src_off = 0;
     d.idx_off = (int64_t)si * GBS_MAX_N;
@@ -708,6 +797,11 @@ bool build_step(gbs_server* s, Stage& g) {
   const int S = s->o.max_slots;
   g.n_items[0] = g.n_items[1] = 0;
   g.fin.clear();
+  g.whole.clear();
+  g.w_idx.clear();
+  g.w_n.clear();
+  g.w_offs.clear();
+  double whole_cost = 0.0;
   memcpy(g.h_up + s->off_pats, s->h_pats.data(), sizeof(PatDesc) * S);
   memcpy(g.h_up + s->off_idx, s->h_idx.data(), sizeof(int) * GBS_MAX_N * S);
   WorkItem* it[2] = {(WorkItem*)(g.h_up + s->off_items[0]), (WorkItem*)(g.h_up + s->off_items[1])};
@@ -728,6 +822,20 @@ bool build_step(gbs_server* s, Stage& g) {
     const int si = (s->rr + q) % S;
     Slot& sl = s->slots[si];
     if (!sl.used || sl.finalize_sent || sl.cancelled) continue;
+    if (whole_request(sl)) {
+      const int h = sl.n / 2;
+      const double c = ldexp((double)h * h * h, h);
+      if (!g.whole.empty() && whole_cost + c > kWholeCost) continue;  // a later step's
+      whole_cost += c;
+      sl.last_step = id;
+      sl.finalize_sent = true;
+      g.whole.push_back(si);
+      g.w_n.push_back(sl.n);
+      g.w_offs.push_back((int64_t)g.w_idx.size());
+      const int* x = &s->h_idx[(size_t)si * GBS_MAX_N];
+      g.w_idx.insert(g.w_idx.end(), x, x + sl.n);
+      continue;
+    }
     sl.last_step = id;
     if (sl.pt >= 0 && !sl.pt_ready && sl.next < sl.items.size()) {
       pt_new[si] = pt_all[si];
@@ -749,7 +857,7 @@ bool build_step(gbs_server* s, Stage& g) {
   }
   s->rr = (s->rr + 1) % S;
   g.id = ++s->step_id;  // == id
-  return g.n_items[0] > 0 || g.n_items[1] > 0 || !g.fin.empty();
+  return g.n_items[0] > 0 || g.n_items[1] > 0 || !g.fin.empty() || !g.whole.empty();
 }
 
 // Return a slot's partial sums and pair-sum region (no step in flight uses them).
@@ -784,8 +892,31 @@ void complete(gbs_server* s, Stage& g) {
     s->pending.erase(sl.ticket);
     free_slot(s, sl);
   }
+  s->stats.completed += (int64_t)g.fin.size();
+  for (size_t b = 0; b < g.whole.size(); ++b) {
+    Slot& sl = s->slots[g.whole[b]];
+    const double kappa = g.h_wres[4 * S + b];
+    if (!sl.cancelled && isnan(kappa)) {  // its terms were given up: by its items from here
+      sl.by_items = true;
+      sl.finalize_sent = false;
+      continue;
+    }
+    s->stats.completed++;
+    if (!sl.cancelled) {
+      Result r;
+      r.rc = GBS_OK;
+      r.p = g.h_wres[b];
+      r.hr = g.h_wres[2 * S + 2 * b];
+      r.hi = g.h_wres[2 * S + 2 * b + 1];
+      r.err = err_estimate(sl.prec, sl.n, kappa);
+      s->done[sl.ticket] = r;
+      s->pending.erase(sl.ticket);
+    }
+    free_slot(s, sl);
+  }
   s->rcv.notify_all();
   g.fin.clear();
+  g.whole.clear();
   g.busy = false;
   s->last_done_step = std::max(s->last_done_step, g.id);
 }
@@ -868,6 +999,9 @@ bool wait_stage(gbs_server* s, Stage& g, bool block) {
 
 void serve_loop(gbs_server* s) {
   cudaSetDevice(s->device);
+  // nothing here touches a stream that another thread may be capturing
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+  cudaThreadExchangeStreamCaptureMode(&mode);
   std::unique_lock<std::mutex> lk(s->mu);
   s->last_tick = std::chrono::steady_clock::now();
   for (;;) {
@@ -890,7 +1024,22 @@ void serve_loop(gbs_server* s) {
     bool launched = false;
     if (any_work && free_stage && build_step(s, *free_stage)) {
       const auto tl0 = std::chrono::steady_clock::now();
-      const cudaError_t e = launch_stage(s, *free_stage);
+      int wrc = GBS_OK;
+      if (!free_stage->whole.empty()) {
+        // some tens of launches: clients go on submitting meanwhile
+        lk.unlock();
+        wrc = launch_whole(s, *free_stage);
+        lk.lock();
+        if (wrc == GBS_ENOMEM) {  // no scratch for them: by their items instead
+          for (int si : free_stage->whole) {
+            s->slots[si].by_items = true;
+            s->slots[si].finalize_sent = false;
+          }
+          free_stage->whole.clear();
+          wrc = GBS_OK;
+        }
+      }
+      const cudaError_t e = (wrc == GBS_OK) ? launch_stage(s, *free_stage) : cudaErrorUnknown;
       const double tl = std::chrono::duration<double>(std::chrono::steady_clock::now() - tl0).count();
       if (tl > s->stats.launch_max_s) s->stats.launch_max_s = tl;
       if (e != cudaSuccess) {
@@ -906,6 +1055,10 @@ void serve_loop(gbs_server* s) {
         s->stats.items += free_stage->n_items[p];
         const WorkItem* it = (const WorkItem*)(free_stage->h_up + s->off_items[p]);
         for (int q = 0; q < free_stage->n_items[p]; ++q) s->stats.subsets += it[q].count;
+      }
+      for (int si : free_stage->whole) {  // (what its items would have been)
+        s->stats.items += (int64_t)s->slots[si].items.size();
+        s->stats.subsets += ((int64_t)1 << (s->slots[si].n / 2)) - 1;
       }
       launched = true;
     }
@@ -925,7 +1078,9 @@ void serve_loop(gbs_server* s) {
         double dev_s = -1.0;
         if (s->o.use_graphs) {
           const unsigned long long* st = (const unsigned long long*)(old->h_res + 5 * s->o.max_slots);
-          if (st[1] >= st[0]) dev_s = 1e-9 * (double)(st[1] - st[0]);
+          const unsigned long long* wt = (const unsigned long long*)(old->h_wres + 5 * s->o.max_slots);
+          const unsigned long long t0 = old->whole.empty() ? st[0] : wt[0], t1 = whole_only(*old) ? wt[1] : st[1];
+          if (t1 >= t0) dev_s = 1e-9 * (double)(t1 - t0);
         } else {
           float dev_ms = 0.f;
           if (cudaEventElapsedTime(&dev_ms, old->ev0, old->ev) == cudaSuccess) dev_s = 1e-3 * dev_ms;
@@ -935,7 +1090,6 @@ void serve_loop(gbs_server* s) {
           s->stats.step_device_s += dev_s;
           if (dev_s > s->stats.step_device_max_s) s->stats.step_device_max_s = dev_s;
         }
-        s->stats.completed += (int64_t)old->fin.size();
         complete(s, *old);
         s->cv.notify_all();
       } else if (block) {
@@ -974,6 +1128,9 @@ void destroy_resources(gbs_server* s) {
     if (g.d_sel) cudaFree(g.d_sel);
     if (g.d_ctr) cudaFree(g.d_ctr);
     if (g.d_res) cudaFree(g.d_res);
+    if (g.h_whole) cudaFreeHost(g.h_whole);
+    if (g.h_wres) cudaFreeHost(g.h_wres);
+    if (g.d_wres) cudaFree(g.d_wres);
   }
   if (s->d_pats) cudaFree(s->d_pats);
   if (s->d_idx) cudaFree(s->d_idx);
@@ -1084,6 +1241,9 @@ extern "C" int gbs_serve_create(const gbs_kernel* k, const gbs_serve_opts* opts,
           (e = cudaMalloc(&g.d_sel, sizeof(int) * S)) != cudaSuccess ||
           (e = cudaMalloc(&g.d_ctr, 256)) != cudaSuccess ||
           (e = cudaMalloc(&g.d_res, 5 * sizeof(double) * S + 16)) != cudaSuccess ||
+          (e = cudaMallocHost(&g.h_whole, batch_stage_bytes(S))) != cudaSuccess ||
+          (e = cudaMallocHost(&g.h_wres, sizeof(double) * (5 * S + 3))) != cudaSuccess ||
+          (e = cudaMalloc(&g.d_wres, sizeof(double) * (5 * S + 3))) != cudaSuccess ||
           (e = cudaEventCreate(&g.ev)) != cudaSuccess || (e = cudaEventCreate(&g.ev0)) != cudaSuccess) {
         cudaGetLastError();
         ret = fail(GBS_ENOMEM, "stage buffers: %s", cudaGetErrorString(e));

@@ -138,3 +138,59 @@ def test_marginals_sum_across_prefix_lengths(gbs, m, n, k):
     ext = np.hstack([ext, np.tile(np.arange(m, dtype=np.int32), 3)[:, None]])
     parts = gbs.marginal_batch(K, ext, n).reshape(3, m).sum(1)
     assert np.all(whole > 0) and np.all(np.abs(parts - whole) <= 1e-12 * whole), (whole, parts)
+
+
+@pytest.mark.parametrize("kind,slots", [("haar", 256), ("haar", 3), ("blocks", 64), ("zero_modes", 64)])
+def test_server_whole_requests_match_batch(gbs, kind, slots):
+    """Requests that go as a whole (orders 2..30, several steps of them, few
+    slots), on a device of equal modes, on one whose blocks of modes differ by
+    9 orders of magnitude and on one with unsqueezed modes: the batched call's
+    results within the two estimates, estimates equal to 1e-9 (sums of up to
+    2^12 positive terms, 1e-15 each), the same bits alone and in the crowd, and
+    as many terms counted as the subset sum has."""
+    import scipy.linalg
+    import workloads as W
+
+    rng = np.random.default_rng(11)
+    if kind == "haar":
+        K = gbs.build_kernel(W.haar_unitary(60, 5), np.full(60, 0.8))
+        pats = [rng.choice(60, size=n, replace=False) for n in list(range(2, 31)) * 3 + [30, 30, 30, 28]]
+    else:
+        U = scipy.linalg.block_diag(*[W.haar_unitary(12, s) for s in (1, 2, 3)])
+        r = np.repeat([0.8, 1e-4, 1e-9] if kind == "blocks" else [0.8, 0.0, 0.5], 12)
+        K = gbs.build_kernel(U, r)
+        pats = [np.concatenate([12 * i + rng.choice(12, size=c, replace=False) for i, c in enumerate(cs)])
+                for cs in [(6, 4, 4), (8, 6, 2), (2, 2, 2), (10, 10, 8), (4, 0, 6), (0, 8, 0), (12, 0, 0), (12, 8, 10)]]
+    pats = [np.sort(x).astype(np.int32) for x in pats]
+    srv = gbs.Server(K, max_slots=slots)
+
+    def serve(xs):
+        tickets, res = [srv.submit(x) for x in xs], []
+        for t in tickets:
+            while (q := srv.poll(t)) is None:
+                pass
+            res.append(q)
+        return res
+
+    try:
+        got = serve(pats)
+        terms = srv.stats()["subsets"]
+        alone = [serve([x])[0] for x in pats[::5]]
+    finally:
+        srv.destroy()
+    assert got[::5] == alone
+    assert terms >= sum(2 ** (len(x) // 2) - 1 for x in pats if len(x) % 2 == 0)
+    idx, n, offs = gbs.pack_patterns(pats)
+    b = len(pats)
+    p, h, err = np.zeros(b), np.zeros(2 * b), np.zeros(b)
+    gbs.prob_batch(K, idx, n, offs, gbs.FP64, p_out=p, haf_out=h, err_out=err)
+    for i, (pg, hg, eg) in enumerate(got):
+        ref = complex(h[2 * i], h[2 * i + 1])
+        # each estimate is relative to its own Hafnian, and infinite for one of 0
+        tol = 1e-13 * abs(ref) + eg * abs(hg) + (err[i] * abs(ref) if ref else 0)
+        assert hg == ref or abs(hg - ref) <= tol, (i, n[i], hg, ref, eg, err[i])
+        if eg + err[i] > 1e-3:
+            continue
+        assert abs(pg - p[i]) <= 2.1 * (1e-13 + eg + err[i]) * p[i], (i, n[i], pg, p[i])
+        # (a large order's estimate is that of the ordering chosen for it, by either call)
+        assert eg == err[i] or n[i] >= 26 or abs(eg - err[i]) <= (1e-9 + eg + err[i]) * err[i], (i, n[i], eg, err[i])
