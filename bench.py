@@ -66,8 +66,9 @@ def model_flops(n: int, terms: bool = True) -> float:
 
 
 def fixed_point_peak_tflops() -> float:
-    """Peak of the terms' complex multiply-add, 4 IMAD.WIDE and 8 FFMA: measured
-    at 32 clocks a warp and SM quarter, so one a clock and quarter, 8 flops each."""
+    """Peak of the terms' complex multiply-add, measured at 32
+    clocks a warp and SM quarter with 4 IMAD.WIDE and 8 FFMA (one a clock and
+    quarter, 8 flops each; the kernel takes 3 IMAD.WIDE)."""
     return SMS * 4 * 8.0 * SM_MHZ_MAX * 1e6 / 1e12
 
 
@@ -391,7 +392,7 @@ def main():
                                 else "haf_subsets_kernel<float>"),
                      "kernel_ms": t_kern,
                      "flops_per_launch": flops,
-                     "peak_note": ("one complex multiply-add (4 IMAD.WIDE, 8 FFMA) a clock and SM quarter, "
+                     "peak_note": ("one complex multiply-add in fixed point (4 IMAD.WIDE, 8 FFMA) a clock and SM quarter, "
                                    "152 SM x 4 x 8 flop x 2.07 GHz" if fp64 else
                                    "FP32 from unit counts and clock (152 SM x 256 flop/clk x 2.07 GHz)"),
                      "measured_fp64_peak": measured_peak,

@@ -25,11 +25,13 @@
 //
 // Arithmetic. A vector entry is fixed point, (hi + lo) 2^{E_k - 27}, hi a whole
 // number of at most 2^27, lo a float of at most a half, with one exponent E_k
-// per matrix and power. A complex multiply-add is then 4 IMAD.WIDE (hi hi,
-// summed exactly in 64 bits) and 8 FFMA (hi lo and lo hi, which need 24 bits
-// only), instead of 4 DFMA: 32 clocks of a warp and SM quarter instead of 256
-// on this part (DFMA 2 a clock and SM; IMAD.WIDE 32; FFMA 128). All four
-// products as IMAD.WIDE, with lo an integer too, took 52. The series run in
+// per matrix and power. A complex multiply-add is then 3 IMAD.WIDE (hi hi:
+// re re, im im and (re + im)(re + im), summed exactly in 64 bits) and 8 FFMA
+// (hi lo and lo hi, which need 24 bits only), instead of 4 DFMA: 28 clocks of
+// a warp and SM quarter instead of 256 on this part (DFMA 2 a clock and SM;
+// IMAD.WIDE 32; FFMA 128). With four IMAD.WIDE, 80 matrices of n = 28 and 30
+// took 19.5 ms instead of 19.0 (n = 16 the same: it is bound by issue); with lo
+// an integer too, 52 clocks. The series run in
 // pairs of floats (48 FP32 operations a multiply-add), coefficient k in units
 // of 2^{e k}, e a mean growth of the E_k.
 //
@@ -52,31 +54,35 @@ constexpr int kExpUnit = 18;
 // 22 bits, which an addition converts, it cost the estimate of one 16-photon
 // pattern four bits.)
 struct FxOp {
-  int hr, hi;
+  int hr, hi, hs;
   float lr, li, fr, fi;
 };
 __device__ __forceinline__ FxOp fx_load(const int4& v) {
   FxOp o;
   o.hr = v.x;
   o.hi = v.y;
+  o.hs = v.x + v.y;
   o.lr = __int_as_float(v.z);
   o.li = __int_as_float(v.w);
   o.fr = (float)v.x;
   o.fi = (float)v.y;
   return o;
 }
-struct Fx {  // one complex sum: h + m
-  long long rh, ih;
+// One complex sum: h + m, the whole part as sums of re re, im im and
+// (re + im)(re + im) (below 2^61: 28 terms of 2^56).
+struct Fx {
+  long long p, q, s;
   float rm, im;
+  __device__ __forceinline__ long long rh() const { return p - q; }
+  __device__ __forceinline__ long long ih() const { return s - p - q; }
 };
-// c += a b; n = -a.hi
-__device__ __forceinline__ void fx_mac(Fx& c, const FxOp& a, int n, const FxOp& b) {
-  c.rh = (long long)a.hr * b.hr + c.rh;
-  c.ih = (long long)a.hr * b.hi + c.ih;
+// c += a b
+__device__ __forceinline__ void fx_mac(Fx& c, const FxOp& a, const FxOp& b) {
+  c.p = (long long)a.hr * b.hr + c.p;
+  c.q = (long long)a.hi * b.hi + c.q;
+  c.s = (long long)a.hs * b.hs + c.s;
   c.rm = fmaf(a.fr, b.lr, c.rm);
   c.im = fmaf(a.fr, b.li, c.im);
-  c.rh = (long long)n * b.hi + c.rh;
-  c.ih = (long long)a.hi * b.hr + c.ih;
   c.rm = fmaf(-a.fi, b.li, c.rm);
   c.im = fmaf(a.fi, b.lr, c.im);
   c.rm = fmaf(a.lr, b.fr, c.rm);
@@ -84,7 +90,7 @@ __device__ __forceinline__ void fx_mac(Fx& c, const FxOp& a, int n, const FxOp& 
   c.rm = fmaf(-a.li, b.fi, c.rm);
   c.im = fmaf(a.li, b.fr, c.im);
 }
-__device__ __forceinline__ Fx fx_zero() { return Fx{0, 0, 0.0f, 0.0f}; }
+__device__ __forceinline__ Fx fx_zero() { return Fx{0, 0, 0, 0.0f, 0.0f}; }
 // (hi, lo) = hi + lo with |lo| <= 1/2 (|lo| < 2^22 before); over where |hi| > 2^27.
 __device__ __forceinline__ int2 fx_pack(int hi, float lo, bool& over) {
   const float q = lo + 12582912.0f;
@@ -101,7 +107,7 @@ __device__ __forceinline__ int2 fx_round(long long h, float m, int sh, bool& ove
   return fx_pack((int)top, lo, over);
 }
 __device__ __forceinline__ int4 fx_entry(const Fx& c, int sh, bool& over) {
-  const int2 x = fx_round(c.rh, c.rm, sh, over), y = fx_round(c.ih, c.im, sh, over);
+  const int2 x = fx_round(c.rh(), c.rm, sh, over), y = fx_round(c.ih(), c.im, sh, over);
   return make_int4(x.x, y.x, x.y, y.y);
 }
 __device__ __forceinline__ bool fx_shift_ok(int sh) { return sh >= 18 && sh <= 31; }
@@ -366,10 +372,10 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
           const FxOp x0 = fx_load(row[c]), x1 = fx_load(row[c + 1]);
           const FxOp a1 = fx_load(U[2 * t + 1]), a0 = fx_load(U[2 * t]);
           const FxOp b1 = fx_load(U[N + 2 * t + 1]), b0 = fx_load(U[N + 2 * t]);
-          fx_mac(ca, x0, -x0.hi, a1);
-          fx_mac(cb, x0, -x0.hi, b1);
-          fx_mac(ca, x1, -x1.hi, a0);
-          fx_mac(cb, x1, -x1.hi, b0);
+          fx_mac(ca, x0, a1);
+          fx_mac(cb, x0, b1);
+          fx_mac(ca, x1, a0);
+          fx_mac(cb, x1, b0);
         }
         const int sh = 27 + ex[k + 1] - ex[k] - ex[1];
         V[k * 2 * N + l] = fx_entry(ca, sh, over);
@@ -397,9 +403,9 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
 #pragma unroll 2
         for (int r2 = 0; r2 < N; ++r2) {
           const FxOp xr = fx_load(x[r2]);
-          fx_mac(c, xr, -xr.hi, fx_load(y[r2 ^ 1]));
+          fx_mac(c, xr, fx_load(y[r2 ^ 1]));
         }
-        const float2 re = df_from(c.rh, c.rm, unit[k]), im = df_from(c.ih, c.im, unit[k]);
+        const float2 re = df_from(c.rh(), c.rm, unit[k]), im = df_from(c.ih(), c.im, unit[k]);
         v = make_float4(re.x, im.x, re.y, im.y);
       }
       mom[t] = v;
