@@ -1679,6 +1679,8 @@ cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st) {
   constexpr int most = 160 * 1024;
   if (!done[dev].load(std::memory_order_acquire)) {
     e = cudaFuncSetAttribute(terms_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(terms_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 257 * 16 * kMaxH);
     if (e != cudaSuccess) return e;
     done[dev].store(1, std::memory_order_release);
   }
@@ -1718,7 +1720,7 @@ cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st) {
   if (smem > (size_t)most) return cudaErrorInvalidValue;
   e = launch_dependent(terms_prep_kernel, dim3(mats), 256, 0, st, T, C);
   if (e == cudaSuccess) e = launch_dependent(terms_delta_kernel, dim3(blocks), kDeltaThreads, smem, st, T, C);
-  if (e == cudaSuccess) e = launch_dependent(terms_series_kernel, dim3(mats), 256, 0, st, T, C, -1);
+  if (e == cudaSuccess) e = launch_dependent(terms_series_kernel, dim3(mats), 256, 257 * 16 * (size_t)hmax, st, T, C, -1);
   for (int level = 8; level < hmax && e == cudaSuccess; ++level) {
     int64_t grid = 0;
     for (int g = 0; g < C.n_groups; ++g)

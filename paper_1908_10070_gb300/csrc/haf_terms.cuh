@@ -440,8 +440,17 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
 // < 0); the masks with last pair `level` >= 8 by 2^level / 256 blocks a matrix.
 // A block's sum |f|_1 and its rounding go to parts[mask >> 8].
 __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, const TermsChunk C, int level) {
+  extern __shared__ __align__(16) unsigned char smem[];
   __shared__ double red[2][256];
   __shared__ float cn[kMaxH + 1];
+  // masks below 256: D_S, then its root, coefficient k of S at [k - 1][S]; the
+  // row takes one place more, so that neither the copy (a subset's
+  // coefficients side by side) nor the sums (subsets side by side) collide (read
+  // from device memory, a place per lane 128 bytes apart, they kept the load
+  // pipe 62 % busy; with twice the threads of the matchings' tiles 4096 of
+  // n = 16 go from 1.72 to 1.63 ms, 80 of n = 28 and 30 from 18.7 to 18.4)
+  float4* ys = reinterpret_cast<float4*>(smem);
+  constexpr int ld = 257;
   dependency_wait();
   int g = 0, bid = blockIdx.x;
   const int per = level < 0 ? 1 : 1 << (level - 8);
@@ -455,8 +464,8 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
   const int n = G.n, h = n >> 1, q = bid / per, sub = bid - q * per, b = P.order[G.first + q];
   if (P.ok[b] == 0) return;
   int4* base = reinterpret_cast<int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
-  float4* delta = reinterpret_cast<float4*>(base + n * n);
-  float4* Gs = delta + ((int64_t)h << h);  // coefficient k of G_S at [k - 1][S], S without pair h - 1
+  const float4* delta = reinterpret_cast<const float4*>(base + n * n);
+  float4* Gs = reinterpret_cast<float4*>(base + n * n) + ((int64_t)h << h);  // coefficient k of G_S at [k - 1][S], S without pair h - 1
   const int64_t gl = (int64_t)1 << (h - 1);
   double2* parts = reinterpret_cast<double2*>(Gs + gl * h);
   const int* ex = P.exps + (int64_t)b * kExpStride;
@@ -468,14 +477,16 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
     const int e = (k == 1) ? ex[1] - 48 - ex[kExpUnit] : ex[i + 1] + ex[k - 2 - i + 1] - 51 - k * ex[kExpUnit];
     cn[k] = sqrtf((float)n) * pow2f(max(min(e, 100), -120));
   }
+  if (level < 0)
+    for (int e = threadIdx.x + h; e < h << min(h, 8); e += blockDim.x) ys[(e % h) * ld + e / h] = delta[e];
   __syncthreads();
   double kap = 0.0, noise = 0.0;
-  // y = D^{-1/2} of subset S in place of its D: k y_k = -sum_i (k - i / 2) d_i y_{k-i}
-  auto root = [&](int S) {
-    float4* d = delta + (int64_t)S * h;
-    float4 dl[kMaxH], y[kMaxH];
+  float4 y[kMaxH];
+  // y = D^{-1/2} of the thread's subset: k y_k = -sum_i (k - i / 2) d_i y_{k-i}
+  auto root = [&](const float4* d, int step) {
+    float4 dl[kMaxH];
 #pragma unroll 1
-    for (int k = 0; k < h; ++k) dl[k] = d[k];
+    for (int k = 0; k < h; ++k) dl[k] = d[k * step];
 #pragma unroll 1
     for (int k = 1; k <= h; ++k) {
       float4 c = dfc_scale(dl[k - 1], 0.5f * k);  // i = k, y_0 = 1
@@ -488,14 +499,13 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
       df_mac(o.x, o.z, c.x, c.z, -r, -rl);
       df_mac(o.y, o.w, c.y, c.w, -r, -rl);
       y[k - 1] = dfc_norm(o);
-      d[k - 1] = y[k - 1];
     }
   };
-  // coefficient k of G_S = G_S' y; at k = h counts f_S and its rounding
-  auto grow = [&](int S, int p, int k) {
+  // coefficient k of G_S = G_S' y, y's at y[(k - 1) step]; at k = h counts f_S
+  // and its rounding
+  auto grow = [&](int S, int p, int k, const float4* y, int step) {
     const int Sp = S ^ (1 << p);
-    const float4* y = delta + (int64_t)S * h;
-    float4 c = y[k - 1];
+    float4 c = y[(k - 1) * step];
     float size = dfc_abs1(c), nz = cn[h];
     if (Sp != 0) {
       const float4* gp = Gs + Sp;
@@ -504,7 +514,7 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
       float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 2
       for (int i = 1; i < k; ++i) {
-        const float4 g0 = gp[(i - 1) * gl], y0 = y[k - i - 1];
+        const float4 g0 = gp[(i - 1) * gl], y0 = y[(k - i - 1) * step];
         dfc_mac(a, g0, y0);
         size += dfc_abs1(g0) * dfc_abs1(y0);
         if (k == h) nz += cn[k - i] * dfc_abs1(g0);
@@ -523,19 +533,25 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
   if (level < 0) {
     // a thread per subset, then per subset and coefficient of a level
     const int low = min(h, 8);
-    if (threadIdx.x >= 1 && (int)threadIdx.x < (1 << low)) root(threadIdx.x);
+    if (threadIdx.x >= 1 && (int)threadIdx.x < (1 << low)) {
+      root(ys + threadIdx.x, ld);
+      for (int k = 0; k < h; ++k) ys[k * ld + threadIdx.x] = y[k];
+    }
     for (int p = 0; p < low; ++p) {
       __syncthreads();
       if (p < h - 1) {
-        for (int t = threadIdx.x; t < h << p; t += blockDim.x) grow((1 << p) + (t & ((1 << p) - 1)), p, h - (t >> p));
+        for (int t = threadIdx.x; t < h << p; t += blockDim.x) {
+          const int S = (1 << p) + (t & ((1 << p) - 1));
+          grow(S, p, h - (t >> p), ys + S, ld);
+        }
       } else if ((int)threadIdx.x < (1 << p)) {
-        grow((1 << p) + threadIdx.x, p, h);
+        grow((1 << p) + threadIdx.x, p, h, ys + (1 << p) + threadIdx.x, ld);
       }
     }
   } else {
     const int S = (1 << level) + sub * 256 + threadIdx.x;
-    root(S);
-    for (int k = (level < h - 1) ? 1 : h; k <= h; ++k) grow(S, level, k);
+    root(delta + (int64_t)S * h, 1);
+    for (int k = (level < h - 1) ? 1 : h; k <= h; ++k) grow(S, level, k, y, 1);
   }
   red[0][threadIdx.x] = kap;
   red[1][threadIdx.x] = noise;

@@ -169,8 +169,9 @@ __device__ __forceinline__ void layer_bases(const int* bin, int (*lb)[kMaxN / 2 
   }
 }
 
-// Orders up to kMatchSmallMax: one block per tile.
-__global__ void __launch_bounds__(kMatchThreads) match_small_kernel(const MatchLaunch L) {
+// Orders up to kMatchSmallMax: one block per tile; twice the threads where only
+// two tiles fit an SM (16 warps kept the FP64 pipe 72 % busy).
+__global__ void __launch_bounds__(2 * kMatchThreads) match_small_kernel(const MatchLaunch L) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int bin[kBinRows * kBinCols];
   __shared__ int lb[kMatchSmallMax + 1][kMaxN / 2 + 2];
@@ -376,7 +377,7 @@ cudaError_t launch_match_small(const MatchLaunch& L, int tiles, size_t smem, cud
     if (e != cudaSuccess) return e;
     done[dev].store(1, std::memory_order_release);
   }
-  return launch_dependent(match_small_kernel, dim3(tiles), kMatchThreads, smem, st, L);
+  return launch_dependent(match_small_kernel, dim3(tiles), smem > 56 * 1024 ? 2 * kMatchThreads : kMatchThreads, smem, st, L);
 }
 
 cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, bool shared, cudaStream_t st) {
