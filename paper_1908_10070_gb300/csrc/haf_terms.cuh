@@ -18,10 +18,11 @@
 //   terms_delta_kernel   D_S of every subset,
 //   terms_series_kernel  f_S = [x^h] prod over the pairs of S of D^{-1/2},
 //                        by the last pair: G_S = G_S' D_S^{-1/2}.
-// 4096 patterns of n = 16: 0.91 and 0.31 ms (powers in the same arithmetic:
-// 2.35 ms and 0.16 for pair sums); 64 of n = 28 with 16 of n = 30: 11.9 and 1.4
-// ms (40). The first kernel keeps the multipliers 55 % busy at n = 28; two
-// thirds of its lanes have a row.
+// 4096 patterns of n = 16: 0.89 and 0.25 ms (powers in the same arithmetic:
+// 2.35 ms and 0.16 for pair sums); 80 of n = 28 and 30, half each: 9.7 and 1.2
+// ms (40). The first kernel is bound by issue (0.78 instructions a clock and
+// quarter; 20 to 24 warps an SM at n = 28 instead of 16 gave 0.6 %); three
+// quarters of its lanes have a row.
 //
 // Arithmetic. A vector entry is fixed point, (hi + lo) 2^{E_k - 27}, hi a whole
 // number of at most 2^27, lo a float of at most a half, with one exponent E_k
