@@ -888,7 +888,7 @@ __global__ void __launch_bounds__(sizeof(T) == 8 ? kMaxWarpsPerBlock * 32 : 512,
 // Warp sum of parts[begin, end): lane j adds j, j+32, ... in that order (four
 // loads issued ahead of their additions), the lanes meet in a fixed
 // butterfly; lane 0 ends with the total (deterministic for a given range).
-__device__ __forceinline__ void sum_partials(const Partial* __restrict__ parts, int begin, int end,
+__device__ __forceinline__ void sum_partials(const Partial* parts, int begin, int end,
                                              int lane, double& rh, double& rl, double& ih, double& il,
                                              double& K) {
   const unsigned FULL = 0xffffffffu;

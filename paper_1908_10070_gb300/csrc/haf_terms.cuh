@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
   const int ld = n + 1;
   for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int r = e / n;
-    M[r * ld + e - r * n] = __ldg(mat + e);
+    M[r * ld + e - r * n] = mat[e];
   }
   if (threadIdx.x < kExpStride) ex[threadIdx.x] = P.exps[(int64_t)b * kExpStride + threadIdx.x];
   __syncthreads();

@@ -215,7 +215,7 @@ __device__ __forceinline__ void cfma_acc(double2& acc, double2 a, double2 b) {
 // sum_{i in T} row(i) Haf(T \ i), T odd, from a table of even sets. The terms
 // are added in increasing position order.
 template <class Row>
-__device__ __forceinline__ double2 expand(const double2* __restrict__ H, int T, const Row& row) {
+__device__ __forceinline__ double2 expand(const double2* H, int T, const Row& row) {
   double2 acc = make_double2(0.0, 0.0);
   for (int rest = T; rest; rest &= rest - 1) {
     const int i = __ffs(rest) - 1;
@@ -278,9 +278,8 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // and the sum over subsets sigma it took 3.44 ms.
 constexpr int kMargSmem = 12;
 __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, const double2* __restrict__ B, int m,
-                                                                      const int* __restrict__ x, unsigned sizes,
-                                                                      const double* __restrict__ coef,
-                                                                      double* __restrict__ q) {
+                                                                      const int* x, unsigned sizes,
+                                                                      const double* coef, double* q) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
   __shared__ double2 Bx[kMargSmem * kMargSmem];
@@ -403,11 +402,9 @@ __device__ __forceinline__ double warp_sum(double v) {
 // of the sum over rho. part[sample * tasks + task]. A mode held once (the
 // common case) has weight 2 instead of 1 on the sets without its position, so
 // half the sets are enough for it; a repeated one goes through all of them.
-__global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, const double2* __restrict__ cache,
+__global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, const double2* cache,
                                                                   int64_t cstride, const double2* __restrict__ B,
-                                                                  const int* __restrict__ x,
-                                                                  const double* __restrict__ coefs,
-                                                                  double2* __restrict__ part) {
+                                                                  const int* x, const double* coefs, double2* part) {
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
   __shared__ Repeats R;
   __shared__ int xs[kMaxK];
@@ -490,12 +487,10 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
 // The candidates' weights q[sample * m + l], a thread each (sample
 // blockIdx.y); the chunks of the gram kernel are added in their order.
 constexpr int kWeightThreads = 128;
-__global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep S, const double2* __restrict__ cache,
+__global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep S, const double2* cache,
                                                                       int64_t cstride, const double2* __restrict__ B,
-                                                                      const int* __restrict__ x,
-                                                                      const double* __restrict__ coefs,
-                                                                      const double2* __restrict__ part,
-                                                                      double* __restrict__ q) {
+                                                                      const int* x, const double* coefs,
+                                                                      const double2* part, double* q) {
   __shared__ double2 M[kMaxK * (kMaxK + 1) / 2], b[kMaxK][kWeightThreads];
   __shared__ double own[kMaxK], s_rho;
   __shared__ int xs[kMaxK], binom[kMaxK + 1][kMaxK + 1];
@@ -576,9 +571,8 @@ __global__ void chain_init_kernel(double2* __restrict__ cache, int64_t cstride, 
 // update: the sets of x_k with the odd T' that later steps read.
 //   u: n uniforms per sample; x: kMaxK sampled modes per sample.
 constexpr int kPickModes = 2048;
-__global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, const double* __restrict__ q,
-                                                                  const double* __restrict__ u, int* __restrict__ x,
-                                                                  double2* __restrict__ cache, int64_t cstride,
+__global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, const double* q, const double* u, int* x,
+                                                                  double2* cache, int64_t cstride,
                                                                   const double2* __restrict__ B) {
   __shared__ int s_pick;
   __shared__ int binom[kMaxK + 1][kMaxK + 1], xs[kMaxK];

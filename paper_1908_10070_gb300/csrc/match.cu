@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(kMatchThreads) match_layer_kernel(const MatchL
       const int cnt = bin[R * kBinCols + j], r = t * 32 + lane;
       const double2 v = next_value(
           bin, R, j, min(r, cnt - 1), has_up, [&](int dd, int rk) { return (dd > 0 ? inup : indn)[rk]; },
-          [&](int p) { return __ldg(rowA + p); });
+          [&](int p) { return rowA[p]; });
       if (r < cnt) out[bo + r] = v;
     }
     w -= all;
