@@ -1184,7 +1184,7 @@ int run_batch(const BatchArgs& a) {
   const size_t ctr_b = 256;
   const size_t status_b = al(sizeof(int) * batch);
   const size_t pstatus_b = n_sel ? al(sizeof(int) * n_probe) : 0;  // zeroed with ctr and status
-  const size_t ok_b = U.terms ? al(sizeof(int) * batch) : 0;       // zeroed too
+  const size_t ok_b = U.terms ? al(2 * sizeof(int) * batch) : 0;   // (ok | lost) zeroed too
   // matchings: a partial per matrix | scratch; terms: exponents | matrix sums | scratch
   const size_t mparts_b = U.match ? al(sizeof(Partial) * batch) : 0;
   const size_t exps_b = U.terms ? al(sizeof(int) * kExpInts * batch) : 0;
@@ -1436,6 +1436,7 @@ int run_batch(const BatchArgs& a) {
           T.status = d_status;
           T.exps = d_exps;
           T.ok = d_ok;
+          T.lost = d_ok + batch;
           T.ksum = d_ksum;
           T.fp64_items = d_ctr + 43;
           std::vector<TermsChunk> chunks;

@@ -226,7 +226,10 @@ struct TermsLaunch {
   const int* skip;         // as in HafLaunch: the repeated-row sum gives the estimate
   int* status;
   int* exps;               // kExpInts per matrix
-  int* ok;                 // zero before launch; in the end 1 where the FP64 kernel has nothing to do
+  int* ok;                 // zero before launch; 1 where prep found the matrix fit for fixed point, in the
+                           // end where the FP64 kernel has nothing to do. Blocks of a matrix branch on
+                           // it, so the kernels between those two leave it alone ..
+  int* lost;               // .. and report a matrix that leaves the range here (zero before launch)
   double* ksum;            // per matrix: sum |f|_1
   int* fp64_items;         // zero before launch; n_items where the FP64 kernel has work
 };

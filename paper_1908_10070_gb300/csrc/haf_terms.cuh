@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
   const TermsGroup G = C.g[g];
   const int n = G.n, h = n >> 1, q = (blockIdx.x - G.block) / G.parts, part = (blockIdx.x - G.block) - q * G.parts;
   const int b = P.order[G.first + q];
-  if (P.ok[b] == 0) return;  // uniform: not in fixed point, or the repeated-row sum's
+  if (P.ok[b] == 0) return;  // uniform (no block writes it here): not in fixed point, or the repeated-row sum's
   const int4* mat = reinterpret_cast<const int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
   float4* delta = reinterpret_cast<float4*>(const_cast<int4*>(mat) + n * n);
   int4* M = reinterpret_cast<int4*>(smem);
@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
   }
   __syncthreads();
   if (s_bad) {
-    if (threadIdx.x == 0) P.ok[b] = 0;
+    if (threadIdx.x == 0) P.lost[b] = 1;
     return;
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kDeltaThreads) terms_delta_kernel(const TermsL
     }
     __syncwarp();
   }
-  if (over) P.ok[b] = 0;
+  if (over) P.lost[b] = 1;
 }
 
 // The last pair's factor and the product with the subset before, a thread per
@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
   if (g == C.n_groups) return;
   const TermsGroup G = C.g[g];
   const int n = G.n, h = n >> 1, q = bid / per, sub = bid - q * per, b = P.order[G.first + q];
-  if (P.ok[b] == 0) return;
+  if (P.ok[b] == 0 || P.lost[b] != 0) return;
   int4* base = reinterpret_cast<int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
   const float4* delta = reinterpret_cast<const float4*>(base + n * n);
   float4* Gs = reinterpret_cast<float4*>(base + n * n) + ((int64_t)h << h);  // coefficient k of G_S at [k - 1][S], S without pair h - 1
@@ -589,7 +589,7 @@ __global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P, c
       continue;
     }
     double K = 0.0, noise = 0.0;
-    const bool done = P.ok[b] != 0;
+    const bool done = P.ok[b] != 0 && P.lost[b] == 0;
     if (done) {
       const int4* base = reinterpret_cast<const int4*>(C.scratch) + G.off + (int64_t)q * G.stride;
       const double2* parts = reinterpret_cast<const double2*>(base + n * n + ((int64_t)h << h) + ((int64_t)h << (h - 1)));

@@ -78,3 +78,15 @@ def test_every_kernel_launched_early_waits():
     for path in glob.glob(os.path.join(CSRC, "*.cu")):
         names |= set(re.findall(r"launch_dependent\((\w+_kernel)", open(path).read()))
     assert names and all("dependency_wait()" in kernels[n] for n in names), names
+
+
+def test_flags_that_blocks_branch_on_are_constant():
+    """A kernel whose blocks leave early on a matrix's ok flag does not write it:
+    another block of the same matrix may be reading it then, and threads of one
+    block that read different values would part before a barrier. (The kernel
+    that closes a chunk has one warp per matrix, which reads before it writes.)"""
+    kernels = {f[1]: f[3] for f in functions() if f[0] == "global"}
+    leave = [k for k, b in kernels.items() if re.search(r"if \([^;{]*P\.ok\[b\] == 0[^;{]*\) return;", b)]
+    assert "terms_delta_kernel" in leave and "terms_series_kernel" in leave
+    for k in leave:
+        assert not re.search(r"P\.ok\[[^]]*\]\s*=[^=]", kernels[k]), k
