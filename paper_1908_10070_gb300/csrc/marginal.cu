@@ -41,7 +41,8 @@
 //   Haf(B_T) = sum_{i in T, i != p} B(x_p, x_i) Haf(B_{T \ {p, i}}),
 // so a prefix's table costs at most k - 1 complex products an entry. Tables
 // hold the even sets only, at index T >> 1 (the lowest bit follows from the
-// parity), and Haf(B_T) rather than Haf(W_T): c_k absorbs tanh(r)^{-s}.
+// parity), and Haf(g B_T) (b_unit) rather than Haf(W_T): c_k absorbs
+// (g tanh(r))^{-s}.
 #include <math.h>
 #include <string.h>
 
@@ -78,16 +79,23 @@ __device__ __forceinline__ void load_binom(int (*binom)[kMaxK + 1], int rows) {
     binom[q / (kMaxK + 1)][q % (kMaxK + 1)] = c_binom.v[q / (kMaxK + 1)][q % (kMaxK + 1)];
 }
 
-// t^{-s} for s = 0..kMaxK (tanh r = t): |Haf(W_T)|^2 = t^{-|T|} |Haf(B_T)|^2.
+// q_n does not depend on t = tanh r > 0, but |Haf(B_T)|^2 ~ t^{|T|} leaves the
+// range of a double from t ~ 1e-16 on at 20 photons. So the sums work on g B
+// with a power of two g (exact) that puts g t into [1, 2) for t below 2^-16
+// (g = 1 above): every expansion along a row, which brings one factor of B,
+// multiplies by g.
+double b_unit(double t) { return t < 0x1p-16 ? ldexp(1.0, std::min(-ilogb(t), 1022)) : 1.0; }
+
+// (g t)^{-s} for s = 0..kMaxK: |Haf(W_T)|^2 = (g t)^{-|T|} |Haf(g B_T)|^2.
 // Computed once per call on the host.
 struct SizeScale {
   double s[kMaxK + 1];
 };
 
-SizeScale size_scale(double t) {
+SizeScale size_scale(double gt) {
   SizeScale sc;
   for (int i = 0; i <= kMaxK; ++i) {
-    const double h = pow(t, -0.5 * i);
+    const double h = pow(gt, -0.5 * i);
     sc.s[i] = h * h;
   }
   return sc;
@@ -112,7 +120,7 @@ unsigned rho_sizes(int k, int n) {
   return sizes;
 }
 
-// c_k(s) t^{-s}, s = 0, 2, .., k, of prefix length k = k0 + blockIdx.x at
+// c_k(s) (g t)^{-s}, s = 0, 2, .., k, of prefix length k = k0 + blockIdx.x at
 // out + k * kCoefs. The log-gammas take few distinct arguments (by mu, by
 // ja + jb and by mu + ja + jb), one thread each; a thread per term evaluated
 // seven in a row, 28 us for a launch, against 10 us now.
@@ -212,16 +220,16 @@ __device__ __forceinline__ void cfma_acc(double2& acc, double2 a, double2 b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
-// sum_{i in T} row(i) Haf(T \ i), T odd, from a table of even sets. The terms
+// g sum_{i in T} row(i) Haf(T \ i), T odd, from a table of even sets. The terms
 // are added in increasing position order.
 template <class Row>
-__device__ __forceinline__ double2 expand(const double2* H, int T, const Row& row) {
+__device__ __forceinline__ double2 expand(const double2* H, int T, double g, const Row& row) {
   double2 acc = make_double2(0.0, 0.0);
   for (int rest = T; rest; rest &= rest - 1) {
     const int i = __ffs(rest) - 1;
     cfma_acc(acc, row(i), H[(T ^ (1 << i)) >> 1]);
   }
-  return acc;
+  return make_double2(acc.x * g, acc.y * g);
 }
 
 // The modes that a prefix holds more than once: position masks and counts
@@ -277,7 +285,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // result's copy included; with index lists built on the host, batched Hafnians
 // and the sum over subsets sigma it took 3.44 ms.
 constexpr int kMargSmem = 12;
-__global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, const double2* __restrict__ B, int m,
+__global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, const double2* __restrict__ B, int m, double g,
                                                                       const int* x, unsigned sizes,
                                                                       const double* coef, double* q) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -303,7 +311,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, con
     for (int r = threadIdx.x; r < binom[k][s]; r += blockDim.x) {
       const int T = unrank(k, s, r, binom), p = __ffs(T) - 1;
       const double2* row = Bx + p * k;
-      const double2 h = expand(H, T & (T - 1), [&](int i) { return row[i]; });
+      const double2 h = expand(H, T & (T - 1), g, [&](int i) { return row[i]; });
       H[T >> 1] = h;
       if (c != 0.0) acc = fma(c * (R.n ? rho_weight(R, T, binom) : 1.0), h.x * h.x + h.y * h.y, acc);
     }
@@ -314,7 +322,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, con
 }
 
 // Longer prefixes: the tables in device memory, one launch per size.
-__global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int s, const double2* __restrict__ B, int m,
+__global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int s, const double2* __restrict__ B, int m, double g,
                                                                       const int* __restrict__ x, int batch,
                                                                       double2* __restrict__ H) {
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
@@ -331,13 +339,13 @@ __global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int
       continue;
     }
     const double2* row = B + (int64_t)xs[__ffs(T) - 1] * m;
-    Hb[T >> 1] = expand(Hb, T & (T - 1), [&](int i) { return __ldg(row + xs[i]); });
+    Hb[T >> 1] = expand(Hb, T & (T - 1), g, [&](int i) { return __ldg(row + xs[i]); });
   }
 }
 
 // q of prefix blockIdx.x from its sub-Hafnians: entry j of the classes has its
-// set's Hafnian at H[b * stride + T >> 1], or (list) at H[b * stride + j].
-__global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, SubsetClasses rho, bool list,
+// set's Hafnian at H[b * stride + T >> 1], or (list: Haf(B_T)) at H[b * stride + j].
+__global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, SubsetClasses rho, bool list, double g,
                                                                     const int* __restrict__ x,
                                                                     const double2* __restrict__ H, int64_t stride,
                                                                     const double* __restrict__ coef,
@@ -351,7 +359,9 @@ __global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, Subse
   double acc = 0.0;
   for (int64_t j = threadIdx.x; j < rho.total(); j += blockDim.x) {
     const int T = subset_of(rho, j, binom);
-    const double2 h = H[blockIdx.x * stride + (list ? j : T >> 1)];
+    double2 h = H[blockIdx.x * stride + (list ? j : T >> 1)];
+    if (list && g != 1.0)
+      for (int i = __popc(T); i > 0; i -= 2) h = make_double2(h.x * g, h.y * g);
     acc = fma(coef[__popc(T) / 2] * (R.n ? rho_weight(R, T, binom) : 1.0), h.x * h.x + h.y * h.y, acc);
   }
   const double sum = block_sum(acc, red);
@@ -403,7 +413,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // common case) has weight 2 instead of 1 on the sets without its position, so
 // half the sets are enough for it; a repeated one goes through all of them.
 __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, const double2* cache,
-                                                                  int64_t cstride, const double2* __restrict__ B,
+                                                                  int64_t cstride, const double2* __restrict__ B, double g,
                                                                   const int* x, const double* coefs, double2* part) {
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
   __shared__ Repeats R;
@@ -466,7 +476,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
           if (al == 0) continue;
           w = weight(T, __popc(T) + 1, extra) - w;
         }
-        const double2 h = expand(H, T, [&](int i) { return __ldg(row + xs[i]); });
+        const double2 h = expand(H, T, g, [&](int i) { return __ldg(row + xs[i]); });
         re = fma(w, h.x * h.x + h.y * h.y, re);
       }
     }
@@ -489,7 +499,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
 constexpr int kWeightThreads = 128;
 __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep S, const double2* cache,
                                                                       int64_t cstride, const double2* __restrict__ B,
-                                                                      const int* x, const double* coefs,
+                                                                      double g, const int* x, const double* coefs,
                                                                       const double2* part, double* q) {
   __shared__ double2 M[kMaxK * (kMaxK + 1) / 2], b[kMaxK][kWeightThreads];
   __shared__ double own[kMaxK], s_rho;
@@ -521,7 +531,10 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
   __syncthreads();
   if (S.direct && threadIdx.x == 0) find_repeats(R, xs, S.kp);
   if (l < S.m)
-    for (int i = 0; i < S.kp; ++i) b[i][threadIdx.x] = __ldg(B + (int64_t)l * S.m + xs[i]);
+    for (int i = 0; i < S.kp; ++i) {
+      const double2 v = __ldg(B + (int64_t)l * S.m + xs[i]);
+      b[i][threadIdx.x] = make_double2(v.x * g, v.y * g);
+    }
   __syncthreads();
   if (l >= S.m) return;
   int mult = 0, first = -1;
@@ -538,7 +551,7 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
     const double2* H = cache + (int64_t)smp * cstride;
     for (int r = 0; r < (int)S.odd.total(); ++r) {
       const int T = subset_of(S.odd, r, binom);
-      const double2 h = expand(H, T, [&](int i) { return b[i][threadIdx.x]; });
+      const double2 h = expand(H, T, 1.0, [&](int i) { return b[i][threadIdx.x]; });
       double w = coef[(__popc(T) + 1) / 2] * (R.n ? rho_weight(R, T, binom, extra) : 1.0);
       if (mult == 1 && !(T >> first & 1)) w *= 2.0;
       s = fma(w, h.x * h.x + h.y * h.y, s);
@@ -573,7 +586,7 @@ __global__ void chain_init_kernel(double2* __restrict__ cache, int64_t cstride, 
 constexpr int kPickModes = 2048;
 __global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, const double* q, const double* u, int* x,
                                                                   double2* cache, int64_t cstride,
-                                                                  const double2* __restrict__ B) {
+                                                                  const double2* __restrict__ B, double g) {
   __shared__ int s_pick;
   __shared__ int binom[kMaxK + 1][kMaxK + 1], xs[kMaxK];
   __shared__ double s_q[kPickModes];  // the weights, where they fit
@@ -622,7 +635,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, c
   const double2* row = B + (int64_t)pick * m;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < (int)S.grow.total(); r += gridDim.x * blockDim.x) {
     const int T = subset_of(S.grow, r, binom);
-    c[(T | (1 << S.kp)) >> 1] = expand(c, T, [&](int i) { return __ldg(row + xs[i]); });
+    c[(T | (1 << S.kp)) >> 1] = expand(c, T, g, [&](int i) { return __ldg(row + xs[i]); });
   }
 }
 
@@ -702,7 +715,9 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
     }
   }
   for (int s = 2; s <= top; s += 2) table += (double)choose(kk, s) * (s - 1);
-  const bool list = kk > kMargSmem && single < table;
+  const double g = b_unit(k->t_uniform);
+  // (the batched path computes Haf(B_T) itself: only where it stays in range)
+  const bool list = kk > kMargSmem && single < table && -0.5 * top * log2(k->t_uniform) < 900.0;
   const bool small = !list && kk <= kMargSmem;
   const int64_t stride = list ? rho.total() : small ? 0 : (int64_t)1 << (kk - 1);
   // tables of at most 2 GB at once
@@ -727,11 +742,11 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
       ret = cuda_fail(e, "marginal upload");
       break;
     }
-    coef_kernel<<<1, kMargThreads, 0, st>>>(kk, n, k->m, size_scale(k->t_uniform), d_c);
+    coef_kernel<<<1, kMargThreads, 0, st>>>(kk, n, k->m, size_scale(g * k->t_uniform), d_c);
     double* qd = q_dev ? q_out : d_q;
     if (small) {
       e = launch_dependent(marginal_small_kernel, dim3(batch), kMargThreads, 16 * ((size_t)1 << std::max(kk - 1, 0)), st, kk,
-                           B, k->m, d_x, sizes, coef, qd);
+                           B, k->m, g, d_x, sizes, coef, qd);
       if (e != cudaSuccess) { ret = cuda_fail(e, "marginal kernel"); break; }
     } else {
       std::vector<int> idx, nv;
@@ -774,10 +789,10 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
           for (int s = 0; s <= top; s += 2) {
             const int64_t work = cnt * choose(kk, s);
             marginal_layer_kernel<<<(int)std::min<int64_t>(8192, (work + kMargThreads - 1) / kMargThreads), kMargThreads,
-                                    0, st>>>(kk, s, B, k->m, d_x + b0 * kk, cnt, d_H);
+                                    0, st>>>(kk, s, B, k->m, g, d_x + b0 * kk, cnt, d_H);
           }
         }
-        marginal_sum_kernel<<<cnt, kMargThreads, 0, st>>>(kk, rho, list, d_x + b0 * kk, d_H, stride, coef, qd + b0);
+        marginal_sum_kernel<<<cnt, kMargThreads, 0, st>>>(kk, rho, list, g, d_x + b0 * kk, d_H, stride, coef, qd + b0);
       }
       if (ret != GBS_OK) break;
     }
@@ -847,7 +862,8 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
   const double2* B = (const double2*)k->B;
   std::vector<int> hx((size_t)group * kMaxK);
   int ret = GBS_OK;
-  coef_kernel<<<n, kMargThreads, 0, st>>>(1, n, m, size_scale(k->t_uniform), d_c);
+  const double g = b_unit(k->t_uniform);
+  coef_kernel<<<n, kMargThreads, 0, st>>>(1, n, m, size_scale(g * k->t_uniform), d_c);
   if ((e = cudaGetLastError()) != cudaSuccess) ret = cuda_fail(e, "chain coefficients");
   for (int s0 = 0; s0 < samples && ret == GBS_OK; s0 += group) {
     const int S = std::min(group, samples - s0);
@@ -862,14 +878,14 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
       const ChainStep& C = steps[kk];
       constexpr int wpb = kMargThreads / 32;
       e = launch_dependent(chain_gram_kernel, dim3((C.tasks + wpb - 1) / wpb, S), kMargThreads, 0, st, C, d_cache, cstride,
-                           B, d_x, d_c, d_part);
+                           B, g, d_x, d_c, d_part);
       if (e == cudaSuccess)
         e = launch_dependent(chain_weight_kernel, dim3((m + kWeightThreads - 1) / kWeightThreads, S), kWeightThreads, 0, st,
-                             C, d_cache, cstride, B, d_x, d_c, d_part, d_q);
+                             C, d_cache, cstride, B, g, d_x, d_c, d_part, d_q);
       // the draws, then the chosen modes' new sub-Hafnians into the caches
       const int nb = kk < n ? (int)std::max<int64_t>(1, std::min<int64_t>(64, (C.grow.total() + 255) / 256)) : 1;
       if (e == cudaSuccess)
-        e = launch_dependent(chain_pick_kernel, dim3(nb, S), kMargThreads, 0, st, C, d_q, d_u, d_x, d_cache, cstride, B);
+        e = launch_dependent(chain_pick_kernel, dim3(nb, S), kMargThreads, 0, st, C, d_q, d_u, d_x, d_cache, cstride, B, g);
       if (e != cudaSuccess) break;
     }
     if (e != cudaSuccess) {
