@@ -357,8 +357,7 @@ typedef struct gbs_serve_opts {
  * step (several large ones in several steps), by the batched call's
  * matchings, with scratch from the library's pool; the others by their subset
  * sums, whose partial sums stay on the device between steps, and so does an
- * FP64 request for which no scratch can be had, or whose estimate's terms
- * need the FP64 subset kernel. Every request is admitted by what its subset
+ * FP64 request for which no scratch can be had. Every request is admitted by what its subset
  * sum would need. Beside mem_budget the server keeps a pool of up to 256 MB
  * (less when max_slots requests of order max_n need less) for the pair sums
  * of FP64 requests of order >= 6; such a request is admitted once its pair

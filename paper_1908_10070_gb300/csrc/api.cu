@@ -1004,9 +1004,8 @@ int run_batch(const BatchArgs& a) {
     std::vector<int> order;
     std::vector<MatchTile> tiles;
     if (U.match) plan_matching(a.n, batch, device_sm_count(), U, &order, &tiles);
-    // (beside the terms: the items of the FP64 kernel behind them)
     if (U.terms) U.arena_b = terms_bytes(U);
-    const bool items = (U.terms && !a.stage) || !U.match;
+    const bool items = !U.match;  // of the subset sum
     auto init = [&]() {
       if (items) plan.init(a.n, batch, a.precision, cfg.warp_bytes, rounds_for_n, reserve);
     };
@@ -1051,7 +1050,7 @@ int run_batch(const BatchArgs& a) {
     U.ptoff_b = (U.pt_elems > 0) ? al(sizeof(int64_t) * batch) : 0;
     // pairing probe of the largest matrices
     PairingPlan pp;
-    if (U.n_items > 0) plan_pairing(a.n, batch, U.pprec, U.pcfg.warp_bytes, maxn / 2, &pp);
+    if (U.n_items > 0 || (U.terms && !a.stage)) plan_pairing(a.n, batch, U.pprec, U.pcfg.warp_bytes, maxn / 2, &pp);
     U.n_sel = (int)pp.sel.size();
     U.n_probe = (int)pp.pats.size();
     U.n_pitems = (int)pp.items.size();
@@ -1184,7 +1183,7 @@ int run_batch(const BatchArgs& a) {
   const size_t ctr_b = 256;
   const size_t status_b = al(sizeof(int) * batch);
   const size_t pstatus_b = n_sel ? al(sizeof(int) * n_probe) : 0;  // zeroed with ctr and status
-  const size_t ok_b = U.terms ? al(2 * sizeof(int) * batch) : 0;   // (ok | lost) zeroed too
+  const size_t ok_b = U.terms ? al(3 * sizeof(int) * batch) : 0;   // (ok | lost | done) zeroed too
   // matchings: a partial per matrix | scratch; terms: exponents | matrix sums | scratch
   const size_t mparts_b = U.match ? al(sizeof(Partial) * batch) : 0;
   const size_t exps_b = U.terms ? al(sizeof(int) * kExpInts * batch) : 0;
@@ -1428,7 +1427,6 @@ int run_batch(const BatchArgs& a) {
           T.idx = L.idx;
           T.pats = d_pats;
           T.order = (const int*)(up + U.order_at);
-          T.n_items = (int)n_items;
           T.m_bound = L.m_bound;
           T.perm = L.perm;
           T.perm_off = L.perm_off;
@@ -1437,23 +1435,14 @@ int run_batch(const BatchArgs& a) {
           T.exps = d_exps;
           T.ok = d_ok;
           T.lost = d_ok + batch;
+          T.done = d_ok + 2 * batch;
           T.ksum = d_ksum;
-          T.fp64_items = d_ctr + 43;
+          T.left = d_ctr + 43;
           std::vector<TermsChunk> chunks;
           terms_chunks(U, d_arena, &chunks);
           for (const TermsChunk& c : chunks)
             if ((e = launch_terms(T, c, st)) != cudaSuccess) break;
           if (e != cudaSuccess) { ret = cuda_fail(e, "terms kernel launch"); break; }
-          // the matrices the fixed-point terms gave back (normally none)
-          if (n_items > 0) {
-            HafLaunch L2 = L;
-            L2.skip = d_ok;
-            L2.pt = nullptr;
-            L2.pt_off = nullptr;
-            L2.n_items_dev = T.fp64_items;
-            e = launch_haf_subsets(L2, a.precision, blocks, cfg.warps_per_block, st);
-            if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
-          }
         }
       } else {
         e = launch_pair_terms(L, st);
@@ -1507,10 +1496,7 @@ int run_batch(const BatchArgs& a) {
     F.status = d_status;
     if (U.match) {
       F.match = d_mparts;
-      if (U.terms) {
-        F.ok = d_ok;
-        F.ksum = d_ksum;
-      }
+      if (U.terms) F.ksum = d_ksum;
     }
     if (dev_rep_cap && (n_items > 0 || U.n_order > 0)) {
       F.rep_half = d_rephalf;

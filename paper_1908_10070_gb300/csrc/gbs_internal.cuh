@@ -201,6 +201,8 @@ __host__ __device__ inline int terms_lanes(int s) { return s > 3 ? 2 * (s - 1) :
 __host__ __device__ inline int terms_group_bytes(int s, int h) {
   return (((h - 1) / 2 + 1) * 4 * (s - 1) + 3 * h + ((s + 3) >> 2)) * 16;
 }
+// Smallest order whose terms are formed in fixed point.
+constexpr int kTermsFixedMin = 2;
 // The matrices of one order in a chunk. Per matrix the scratch holds n^2 limbs,
 // 2^h h series coefficients D, 2^(h-1) h of G, and the sums' parts.
 struct TermsGroup {
@@ -208,10 +210,13 @@ struct TermsGroup {
   int begin;               // the group's first matrix in the chunk
   int block, parts;        // delta kernel: first block, blocks per matrix
   int region;              // delta kernel: shared bytes per warp
+  int item64, parts64;     // FP64: first item, items per matrix
   int64_t off, stride;     // in units of 16 bytes: the group's first matrix, and per matrix
 };
 struct TermsChunk {
-  int n_groups;
+  int n_groups;            // largest order first
+  int items64, small64;    // FP64: items in all, of the orders below kTermsFixedMin (numbered first)
+  int hmax64;
   void* scratch;
   TermsGroup g[kMaxN / 2];
 };
@@ -220,18 +225,19 @@ struct TermsLaunch {
   const int* idx;
   const PatDesc* pats;
   const int* order;        // even-order matrices, by order
-  int n_items, m_bound;
+  int m_bound;
   const int* perm;
   const int* perm_off;
   const int* skip;         // as in HafLaunch: the repeated-row sum gives the estimate
   int* status;
   int* exps;               // kExpInts per matrix
   int* ok;                 // zero before launch; 1 where prep found the matrix fit for fixed point, in the
-                           // end where the FP64 kernel has nothing to do. Blocks of a matrix branch on
+                           // end where the FP64 kernels have nothing to do. Blocks of a matrix branch on
                            // it, so the kernels between those two leave it alone ..
   int* lost;               // .. and report a matrix that leaves the range here (zero before launch)
+  int* done;               // FP64: blocks of the matrix that have added their share (zero before launch)
   double* ksum;            // per matrix: sum |f|_1
-  int* fp64_items;         // zero before launch; n_items where the FP64 kernel has work
+  int* left;               // zero before launch; 1 where the FP64 kernels have a matrix of a larger order
 };
 // 16-byte units of scratch of one matrix.
 int64_t terms_matrix_units(int n);
@@ -290,11 +296,9 @@ struct FinalizeLaunch {
   const int* rep_half;
   const int* rep_end;
   const Partial* rep_parts;
-  // If non-null: per matrix its Hafnian (matchings) in re_hi, im_hi; the
-  // partials of `parts` then count only for kappa, and only where ok is 0
-  // (elsewhere it is ksum, where that is given).
+  // If non-null: per matrix its Hafnian (matchings) in re_hi, im_hi, and
+  // sum |f|_1 (ksum, may be null), in the place of `parts`.
   const Partial* match;
-  const int* ok;
   const double* ksum;
   const int* batch_dev;    // if non-null, the number of entries is read here (device memory)
   const Partial* chunk_parts;  // if non-null, sum these chunk sums (chunk_off ranges) instead

@@ -1000,7 +1000,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const Finalize
       const int n = d.n;
       // loads that do not depend on the partial sums go first
       const int xi = (want_p && d.idx_off >= 0 && lane < n) ? F.idx[d.idx_off + lane] : -1 - lane;
-      int bad = (lane == 0 && F.status != nullptr) ? F.status[pb] : 0;
+      const int bad = (lane == 0 && F.status != nullptr) ? F.status[pb] : 0;
       double rh = 0, rl = 0, ih = 0, il = 0, K = 0;
       if (!(n & 1) && n > 0) {
         const int rep = F.rep_half ? F.rep_half[pb] : 0;
@@ -1011,13 +1011,7 @@ __global__ void __launch_bounds__(kFinWarps * 32) finalize_kernel(const Finalize
         } else if (F.match) {
           rh = F.match[pb].re_hi;
           ih = F.match[pb].im_hi;
-          if (F.ok != nullptr && F.ok[pb] == 0) {
-            double a = 0, b2 = 0, c2 = 0, e2 = 0;
-            sum_partials(F.parts, d.item_begin, d.item_end, lane, a, b2, c2, e2, K);
-            if (d.item_begin == d.item_end) bad = 1;  // a served request: its subset items follow
-          } else if (F.ksum != nullptr) {
-            K = F.ksum[pb];
-          }
+          if (F.ksum != nullptr) K = F.ksum[pb];
         } else if (F.chunk_parts)
           sum_partials(F.chunk_parts, F.chunk_off[pb], F.chunk_off[pb + 1], lane, rh, rl, ih, il, K);
         else
@@ -1530,6 +1524,7 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
 }
 
 #include "haf_terms.cuh"
+#include "haf_terms64.cuh"
 
 // Route choice on the device (see RoutePlan): one warp per pattern decides
 // between the subset sum and the repeated-row sum by the cost rule, then the
@@ -1678,7 +1673,10 @@ cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st) {
   static std::atomic<int> done[64];
   constexpr int most = 160 * 1024;
   if (!done[dev].load(std::memory_order_acquire)) {
-    e = cudaFuncSetAttribute(terms_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    e = cudaFuncSetAttribute(terms64_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(terms64_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * (kSeries64 + 1) * 16 * kMaxH);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(terms_delta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(terms_series_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 257 * 16 * kMaxH);
     if (e != cudaSuccess) return e;
@@ -1696,38 +1694,68 @@ cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st) {
       rounds[h] += (c + gpw - 1) / gpw;
     }
   }
+  int fixed = 0;  // the groups in fixed point: the first ones
+  while (fixed < C.n_groups && C.g[fixed].n >= kTermsFixedMin) ++fixed;
   int per = 16;  // rounds per warp
   for (; per > 1; per /= 2) {
     int64_t blocks = 0;
-    for (int g = 0; g < C.n_groups; ++g)
+    for (int g = 0; g < fixed; ++g)
       blocks += C.g[g].count * ((rounds[C.g[g].n / 2] + per * nw - 1) / (per * nw));
     if (blocks >= 16 * sms) break;
   }
-  int blocks = 0, mats = 0, hmax = 0;
+  int blocks = 0, mats = 0;
   size_t smem = 0;
-  for (int g = 0; g < C.n_groups; ++g) {
+  C.hmax64 = C.g[0].n / 2;
+  C.items64 = C.small64 = 0;
+  int64_t items_series = 0;
+  for (int g = C.n_groups - 1; g >= 0; --g) {
     TermsGroup& G = C.g[g];
     const int h = G.n / 2;
-    G.parts = (int)((rounds[h] + per * nw - 1) / (per * nw));
-    G.block = blocks;
-    blocks += G.count * G.parts;
-    mats = G.begin + G.count;
-    hmax = std::max(hmax, h);
     G.region = 0;
     for (int s = 1; s <= h; ++s) G.region = std::max(G.region, (32 / terms_lanes(s)) * terms_group_bytes(s, h));
     smem = std::max(smem, (size_t)G.n * (G.n + 1) * 16 + (size_t)nw * G.region);
+    // a round per warp: one matrix of a large order, given back alone, is to
+    // fill the chip; small orders come in numbers, and a few rounds a warp
+    // share their copy of the matrix
+    const int per64 = g < fixed ? 1 : 4;
+    G.parts64 = (int)((rounds[h] + per64 * nw - 1) / (per64 * nw));
+    G.item64 = C.items64;
+    C.items64 += G.count * G.parts64;
+    if (g >= fixed) C.small64 = C.items64;
+    items_series += h <= 7 ? (G.count + (kSeries64 >> h) - 1) / (kSeries64 >> h) : (int64_t)G.count << (h - 7);
   }
   if (smem > (size_t)most) return cudaErrorInvalidValue;
-  e = launch_dependent(terms_prep_kernel, dim3(mats), 256, 0, st, T, C);
-  if (e == cudaSuccess) e = launch_dependent(terms_delta_kernel, dim3(blocks), kDeltaThreads, smem, st, T, C);
-  if (e == cudaSuccess) e = launch_dependent(terms_series_kernel, dim3(mats), 256, 257 * 16 * (size_t)hmax, st, T, C, -1);
-  for (int level = 8; level < hmax && e == cudaSuccess; ++level) {
-    int64_t grid = 0;
-    for (int g = 0; g < C.n_groups; ++g)
-      if (C.g[g].n / 2 > level) grid += (int64_t)C.g[g].count << (level - 8);
-    e = launch_dependent(terms_series_kernel, dim3((unsigned)grid), 256, 0, st, T, C, level);
+  if (fixed > 0) {
+    TermsChunk F = C;
+    F.n_groups = fixed;
+    for (int g = 0; g < fixed; ++g) {
+      TermsGroup& G = F.g[g];
+      G.parts = (int)((rounds[G.n / 2] + per * nw - 1) / (per * nw));
+      G.block = blocks;
+      blocks += G.count * G.parts;
+      mats = G.begin + G.count;
+    }
+    const int hmax = F.g[0].n / 2;
+    e = launch_dependent(terms_prep_kernel, dim3(mats), 256, 0, st, T, F);
+    if (e == cudaSuccess) e = launch_dependent(terms_delta_kernel, dim3(blocks), kDeltaThreads, smem, st, T, F);
+    if (e == cudaSuccess) e = launch_dependent(terms_series_kernel, dim3(mats), 256, 257 * 16 * (size_t)hmax, st, T, F, -1);
+    for (int level = 8; level < hmax && e == cudaSuccess; ++level) {
+      int64_t grid = 0;
+      for (int g = 0; g < fixed; ++g)
+        if (F.g[g].n / 2 > level) grid += (int64_t)F.g[g].count << (level - 8);
+      e = launch_dependent(terms_series_kernel, dim3((unsigned)grid), 256, 0, st, T, F, level);
+    }
+    if (e == cudaSuccess) e = launch_dependent(terms_check_kernel, dim3(std::min((mats + 7) / 8, 1024)), 256, 0, st, T, F);
+    if (e != cudaSuccess) return e;
   }
-  if (e == cudaSuccess) e = launch_dependent(terms_check_kernel, dim3(std::min((mats + 7) / 8, 1024)), 256, 0, st, T, C);
+  // as many blocks as are resident by their shared memory, at most one an item
+  auto resident = [&](int64_t items, size_t bytes) {
+    const int64_t most_blocks = (int64_t)sms * std::max<int64_t>(1, std::min<int64_t>(8, (int64_t)(220 * 1024 / (bytes + 4096))));
+    return dim3((unsigned)std::min(items, most_blocks));
+  };
+  const size_t series = 2 * (kSeries64 + 1) * 16 * (size_t)C.hmax64;
+  e = launch_dependent(terms64_delta_kernel, resident(C.items64, smem), kDeltaThreads, smem, st, T, C);
+  if (e == cudaSuccess) e = launch_dependent(terms64_series_kernel, resident(items_series, series), kSeries64, series, st, T, C);
   return e;
 }
 

@@ -42,8 +42,8 @@
 // finite, exponents too far apart, or an estimate of the rounding carried along
 // with the series (several times what is met, and added over the subsets
 // without regard to sign) that comes out above 2^-33 of the sum, send the
-// matrix to the FP64 subset kernel (launched after; it returns at once when no matrix is
-// left to it).
+// matrix to the FP64 kernels (haf_terms64.cuh; launched after, they return at
+// once when no matrix is left to them).
 
 constexpr int kFxBits = 27;      // |hi| <= 2^27
 constexpr int kFxRoom = 2;       // exponents added to the float estimate of a power's largest entry
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(256) terms_series_kernel(const TermsLaunch P, 
 
 // One warp per matrix: the sum over its parts, in its own units again; a matrix
 // that left the range, or whose rounding estimate is above 2^-33 of the sum, goes
-// to the FP64 kernel.
+// to the FP64 kernels.
 __global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P, const TermsChunk C) {
   dependency_wait();
   const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P, c
     const TermsGroup& G = C.g[g];
     const int n = G.n, h = n >> 1, q = m - G.begin, b = P.order[G.first + q];
     if (P.skip != nullptr && P.skip[b] != 0) {
-      if (lane == 0) P.ok[b] = 1;  // nothing for the FP64 kernel either
+      if (lane == 0) P.ok[b] = 1;  // nothing for the FP64 kernels either
       continue;
     }
     double K = 0.0, noise = 0.0;
@@ -609,5 +609,5 @@ __global__ void __launch_bounds__(256) terms_check_kernel(const TermsLaunch P, c
       redo |= !fine;
     }
   }
-  if (redo) *P.fp64_items = P.n_items;  // (zero before the first chunk; every writer writes the same)
+  if (redo) *P.left = 1;  // (zero before the first chunk; every writer writes the same)
 }

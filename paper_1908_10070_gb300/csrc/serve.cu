@@ -11,11 +11,11 @@
 // are admitted, run beside it and finish first.
 //
 // FP64 requests of order <= 30 go as a whole in one step: their Hafnians by
-// matchings and their estimates by fixed-point terms, the batched path's
+// matchings and their estimates' terms by the Krylov vectors, the batched path's
 // kernels, enqueued ahead of the step's items (384 requests of 12 <= n <= 26
 // at once, about half of them of odd n: 16 ms by items, now 4.1). They hold the same slots
-// and memory as if they went by items, which those whose terms are given up
-// and all others do.
+// and memory as if they went by items, which all others do, and these when no
+// scratch can be had for them.
 //
 // A request's work items, their partial-sum slots and the order in which its
 // partials are added depend only on its own n and precision, so its result is
@@ -133,8 +133,7 @@ struct Slot {
 
 constexpr int kStepCap = 65536;  // work items per precision per step
 // FP64 requests of order <= kMatchMaxN go as a whole in one step, through the
-// batched path's matchings and fixed-point terms instead of their subset
-// items; the few whose terms are given up there go by their items afterwards.
+// batched path's matchings and terms instead of their subset items.
 // A lone request took 98 us by items at n = 4, 157 at 12, 222 at 16, 0.45 ms
 // at 24, 0.80 at 26, 4.15 at 30, and takes 75, 86, 105, 0.28, 0.50 and 1.0.
 // A step takes such requests up to this many 2^h h^3 (the terms take 1 us per
@@ -896,11 +895,6 @@ void complete(gbs_server* s, Stage& g) {
   for (size_t b = 0; b < g.whole.size(); ++b) {
     Slot& sl = s->slots[g.whole[b]];
     const double kappa = g.h_wres[4 * S + b];
-    if (!sl.cancelled && isnan(kappa)) {  // its terms were given up: by its items from here
-      sl.by_items = true;
-      sl.finalize_sent = false;
-      continue;
-    }
     s->stats.completed++;
     if (!sl.cancelled) {
       Result r;

@@ -1,0 +1,97 @@
+"""sum |f|_1 of the error estimate where it is formed in FP64: matrices that the
+fixed-point kernels cannot do.
+
+kappa times the modulus of the Hafnian that comes with it is that sum, whatever
+the Hafnian's own error. It adds moduli, so nothing cancels, and its relative
+error is that of the terms: sums of products of at most h = n/2 entries, with
+n roundings or so on the way to each, which grow like a square root when they
+are independent. n 2^-52 leaves more than 4 over that for two quotients."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gbs():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1908_10070_gb300 as g
+
+    return g
+
+
+def rand_sym(n, rng):
+    A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+    return (A + A.T) / 2
+
+
+def haf(gbs, mats, noalloc=False):
+    flat, n, offs = gbs.pack_matrices(mats)
+    out = torch.zeros(2 * len(mats), dtype=torch.float64, device="cuda")
+    kap = torch.zeros(len(mats), dtype=torch.float64, device="cuda")
+    f = gbs.hafnian_batch_noalloc if noalloc else gbs.hafnian_batch
+    f(torch.from_numpy(flat).cuda(), n, offs, gbs.FP64, haf_out=out, kappa_out=kap)
+    torch.cuda.synchronize()
+    o = out.cpu().numpy()
+    return o[0::2] + 1j * o[1::2], kap.cpu().numpy()
+
+
+def unequal_rows(n, rng):
+    """Rows 2^30 apart in size: fixed point has no room for them."""
+    d = np.ldexp(1.0, 15 * (1 - 2 * (rng.permutation(n) % 2)))
+    A = rand_sym(n, rng)
+    return A * d[:, None] * d[None, :], A
+
+
+@pytest.mark.parametrize("n,count", [(4, 2), (12, 3), (14, 3), (16, 5), (18, 1), (18, 6), (20, 2), (24, 2)])
+def test_matrices_without_a_fixed_point_range(gbs, n, count):
+    """Scaled rows scale the Hafnian by exact powers of two, a zero row makes it
+    0; sum |f| is the FP64 subset kernel's (both by the bound above), beside
+    matrices that stay in fixed point."""
+    rng = np.random.default_rng(n + count)
+    pairs = [unequal_rows(n, rng) for _ in range(count)]
+    zero = rand_sym(n, rng)
+    zero[1, :] = zero[:, 1] = 0
+    plain = rand_sym(n, rng)
+    mats = [p[0] for p in pairs] + [zero, plain, rand_sym(4, rng)]
+    h, kappa = haf(gbs, mats)
+    assert np.array_equal(h[:count], haf(gbs, [p[1] for p in pairs])[0])  # prod of the scales is 1
+    assert h[count] == 0 and kappa[count] == np.inf
+    assert kappa[count + 1] == haf(gbs, [plain])[1][0]
+    h0, k0 = haf(gbs, [p[0] for p in pairs], noalloc=True)
+    for b in range(count):
+        K, K0 = kappa[b] * abs(h[b]), k0[b] * abs(h0[b])
+        assert abs(K - K0) <= 2 * n * 2.0**-52 * K0, (b, K, K0)
+
+
+def test_served_requests_without_a_fixed_point_range_count_once(gbs):
+    """Blocks of modes 9 orders of magnitude apart: the batched call's results,
+    the same bits, and as many subset terms counted as the subset sum has."""
+    import scipy.linalg
+    import workloads as W
+
+    U = scipy.linalg.block_diag(*[W.haar_unitary(12, s) for s in (1, 2, 3)])
+    K = gbs.build_kernel(U, np.repeat([0.8, 1e-4, 1e-9], 12))
+    rng = np.random.default_rng(12)
+    pats = [np.sort(np.concatenate([12 * i + rng.choice(12, size=c, replace=False) for i, c in enumerate(cs)])).astype(np.int32)
+            for cs in [(6, 4, 4), (8, 6, 2), (2, 2, 2), (2, 0, 0), (10, 10, 4), (4, 0, 6), (0, 8, 0), (12, 2, 10)] * 3]
+    srv = gbs.Server(K, max_slots=16)
+    try:
+        tickets, got = [srv.submit(x) for x in pats], []
+        for t in tickets:
+            while (q := srv.poll(t)) is None:
+                pass
+            got.append(q)
+        stats = srv.stats()
+    finally:
+        srv.destroy()
+    assert stats["completed"] == len(pats)
+    assert stats["subsets"] == sum(2 ** (len(x) // 2) - 1 for x in pats)
+    idx, n, offs = gbs.pack_patterns(pats)
+    b = len(pats)
+    p, h, err = np.zeros(b), np.zeros(2 * b), np.zeros(b)
+    gbs.prob_batch(K, idx, n, offs, gbs.FP64, p_out=p, haf_out=h, err_out=err)
+    assert [q[0] for q in got] == list(p) and [q[2] for q in got] == list(err)
