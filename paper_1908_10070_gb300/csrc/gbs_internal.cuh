@@ -201,8 +201,8 @@ __host__ __device__ inline int terms_lanes(int s) { return s > 3 ? 2 * (s - 1) :
 __host__ __device__ inline int terms_group_bytes(int s, int h) {
   return (((h - 1) / 2 + 1) * 4 * (s - 1) + 3 * h + ((s + 3) >> 2)) * 16;
 }
-// Smallest order whose terms are formed in fixed point.
-constexpr int kTermsFixedMin = 2;
+// Smallest order whose terms are formed in fixed point (haf_terms64.cuh: why).
+constexpr int kTermsFixedMin = 14;
 // The matrices of one order in a chunk. Per matrix the scratch holds n^2 limbs,
 // 2^h h series coefficients D, 2^(h-1) h of G, and the sums' parts.
 struct TermsGroup {

@@ -1,6 +1,15 @@
-// The same moduli in FP64 (included by haf_subsets.cu after haf_terms.cuh), for
-// the matrices that the fixed-point kernels could not do or gave back: sum |f|
-// is within 1e-15 of its value, as the powers gave it.
+// The same moduli in FP64 (included by haf_subsets.cu after haf_terms.cuh):
+// for the orders below kTermsFixedMin, and for the matrices that the
+// fixed-point kernels could not do or gave back.
+//
+// Below order 14 kappa from the fixed-point sum is off by more than kappa from
+// the subset sum was, whose Hafnian brings the larger part of its error
+// (largest of 240 Haar and random matrices an order, subset sum / fixed point /
+// now: n = 4 2.0e-15 / 1.2e-14 / 4e-16, n = 8 1.2e-14 / 2.2e-14 / 2e-15, n = 10
+// 2.4e-14 / 3.6e-14 / 4e-15; n = 12, medians, up to 3.8e-15 / 3.2e-15 / 2e-16).
+// From 14 on it is off by less (n = 14 7.6e-13 / 1.9e-14; n = 16 9.3e-13 /
+// 1.1e-14; n = 24 1.2e-11 / 1.1e-14). Here sum |f| is within 1e-15 of its
+// value, as the powers gave it.
 //
 // The same Krylov vectors and series as there (a third of the products of the
 // powers of a subset's matrix at order 16, a quarter at 30), on the matrix
@@ -8,8 +17,9 @@
 // so the layout only has to keep its lanes filled: rows as lanes, then a
 // subset's series per lane. Two launches whatever the order: a block takes 128
 // neighbouring masks and recomputes the series of the prefixes they share (a
-// quarter of the Krylov products at order 30) instead of a launch per level. Both strided over by as many blocks as are resident, which leave
-// at once when no matrix is left to them (the usual case).
+// quarter of the Krylov products at order 30) instead of a launch per level.
+// As many blocks as are resident stride over the items of either, and leave at
+// once when no matrix is left to them (the usual case).
 
 constexpr int kCoefs64 = (kMatchMaxN / 2 + 5) / 6;  // most coefficients per lane (6 lanes a subset at least)
 constexpr int kSeries64 = 128;                      // threads (columns) of a block of the series kernel

@@ -1,5 +1,5 @@
-"""sum |f|_1 of the error estimate where it is formed in FP64: matrices that the
-fixed-point kernels cannot do.
+"""sum |f|_1 of the error estimate where it is formed in FP64: the small orders,
+and matrices that the fixed-point kernels cannot do.
 
 kappa times the modulus of the Hafnian that comes with it is that sum, whatever
 the Hafnian's own error. It adds moduli, so nothing cancels, and its relative
@@ -37,6 +37,37 @@ def haf(gbs, mats, noalloc=False):
     torch.cuda.synchronize()
     o = out.cpu().numpy()
     return o[0::2] + 1j * o[1::2], kap.cpu().numpy()
+
+
+def moduli(A):
+    """sum_S |f(X A_S)|_1 from the power traces, in long double (64 bits or more)."""
+    n = len(A)
+    h = n // 2
+    pos = [p // 2 + (h if p % 2 else 0) for p in range(n)]
+    A = A[np.ix_(pos, pos)].astype(np.clongdouble)
+    A[np.arange(n), np.arange(n)] = 0
+    total = np.longdouble(0)
+    for S in range(1, 1 << h):
+        rows = [2 * p + q for p in range(h) if S >> p & 1 for q in (0, 1)]
+        M = A[np.ix_([r ^ 1 for r in rows], rows)]
+        power, tr, c = M, [None], [np.clongdouble(1)]
+        for k in range(1, h + 1):
+            tr.append(np.trace(power))
+            c.append(sum(tr[i] * c[k - i] for i in range(1, k + 1)) / (2 * k))
+            power = (power[:, :, None] * M[None, :, :]).sum(1)
+        total += abs(c[h].real) + abs(c[h].imag)
+    return total
+
+
+@pytest.mark.parametrize("n,count", [(2, 1), (2, 300), (4, 1), (4, 70), (6, 33), (8, 17), (10, 9), (12, 1), (12, 5)])
+def test_small_orders_keep_double_precision(gbs, n, count):
+    """Blocks of one and of many matrices, the last one partly filled."""
+    rng = np.random.default_rng(100 * n + count)
+    mats = [rand_sym(n, rng) for _ in range(count)]
+    h, kappa = haf(gbs, mats)
+    for b in sorted({0, 1 % count, count // 2, count - 1}):
+        K = moduli(mats[b])
+        assert abs(kappa[b] * abs(h[b]) - K) <= n * 2.0**-52 * K, (b, kappa[b] * abs(h[b]), K)
 
 
 def unequal_rows(n, rng):
