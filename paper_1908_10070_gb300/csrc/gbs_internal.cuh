@@ -18,8 +18,8 @@ namespace gbs {
 // before those writes), so the read-only path is not for it: plain pointers
 // without __restrict__, which lets the compiler take that path, or __ldcg;
 // __ldg and __restrict__ are for B, the caller's inputs and uploads alone,
-// complete before the call's first kernel. The wait returns at once after an
-// ordinary launch. In calls of many short kernels this takes 2 us off a
+// complete before the first kernel of such a chain has begun. The wait returns
+// at once after an ordinary launch. In calls of many short kernels this takes 2 us off a
 // launch: 64 chain samples of 16 photons (50 launches) 716 -> 616 us, 301
 // matrices of n <= 22 (16) 154 -> 127, one 16-photon pattern 141 -> 126. No
 // kernel asks for its successor early: blocks that wait then hold shared

@@ -41,8 +41,8 @@
 //   Haf(B_T) = sum_{i in T, i != p} B(x_p, x_i) Haf(B_{T \ {p, i}}),
 // so a prefix's table costs at most k - 1 complex products an entry. Tables
 // hold the even sets only, at index T >> 1 (the lowest bit follows from the
-// parity), and Haf(g B_T) (b_unit) rather than Haf(W_T): c_k absorbs
-// (g tanh(r))^{-s}.
+// parity), and Haf(B_T) rather than Haf(W_T): c_k absorbs tanh(r)^{-s} (for a
+// tiny r both with g B, see b_unit).
 #include <math.h>
 #include <string.h>
 
@@ -80,11 +80,24 @@ __device__ __forceinline__ void load_binom(int (*binom)[kMaxK + 1], int rows) {
 }
 
 // q_n does not depend on t = tanh r > 0, but |Haf(B_T)|^2 ~ t^{|T|} leaves the
-// range of a double from t ~ 1e-16 on at 20 photons. So the sums work on g B
-// with a power of two g (exact) that puts g t into [1, 2) for t below 2^-16
-// (g = 1 above): every expansion along a row, which brings one factor of B,
-// multiplies by g.
+// range of a double from t ~ 1e-16 on at 20 photons. Below 2^-16 the sums
+// therefore read g B, a copy made for the call with a power of two g (exact)
+// that puts g t into [1, 2); above, g = 1 and they read B itself. (Multiplying
+// by g wherever a set's Hafnian is formed cost ordinary calls up to 10 %.)
 double b_unit(double t) { return t < 0x1p-16 ? ldexp(1.0, std::min(-ilogb(t), 1022)) : 1.0; }
+__global__ void scale_kernel(const double* __restrict__ B, double* __restrict__ gB, int64_t count, double g) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x)
+    gB[i] = g * B[i];
+}
+// What the sums read: k's B, or its copy at `copy` (b_copy_bytes of scratch).
+size_t b_copy_bytes(const gbs_kernel* k) { return b_unit(k->t_uniform) == 1.0 ? 0 : 16 * (size_t)k->m * k->m; }
+const double* scaled_B(const gbs_kernel* k, void* copy, cudaStream_t st) {
+  const double g = b_unit(k->t_uniform);
+  if (g == 1.0) return k->B;
+  const int64_t count = 2 * (int64_t)k->m * k->m;
+  scale_kernel<<<(int)std::min<int64_t>(8192, (count + 255) / 256), 256, 0, st>>>(k->B, (double*)copy, count, g);
+  return (const double*)copy;
+}
 
 // (g t)^{-s} for s = 0..kMaxK: |Haf(W_T)|^2 = (g t)^{-|T|} |Haf(g B_T)|^2.
 // Computed once per call on the host.
@@ -92,7 +105,8 @@ struct SizeScale {
   double s[kMaxK + 1];
 };
 
-SizeScale size_scale(double gt) {
+SizeScale size_scale(double t) {
+  const double gt = b_unit(t) * t;
   SizeScale sc;
   for (int i = 0; i <= kMaxK; ++i) {
     const double h = pow(gt, -0.5 * i);
@@ -220,16 +234,16 @@ __device__ __forceinline__ void cfma_acc(double2& acc, double2 a, double2 b) {
   acc.y = fma(a.y, b.x, acc.y);
 }
 
-// g sum_{i in T} row(i) Haf(T \ i), T odd, from a table of even sets. The terms
+// sum_{i in T} row(i) Haf(T \ i), T odd, from a table of even sets. The terms
 // are added in increasing position order.
 template <class Row>
-__device__ __forceinline__ double2 expand(const double2* H, int T, double g, const Row& row) {
+__device__ __forceinline__ double2 expand(const double2* H, int T, const Row& row) {
   double2 acc = make_double2(0.0, 0.0);
   for (int rest = T; rest; rest &= rest - 1) {
     const int i = __ffs(rest) - 1;
     cfma_acc(acc, row(i), H[(T ^ (1 << i)) >> 1]);
   }
-  return make_double2(acc.x * g, acc.y * g);
+  return acc;
 }
 
 // The modes that a prefix holds more than once: position masks and counts
@@ -285,7 +299,7 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 // result's copy included; with index lists built on the host, batched Hafnians
 // and the sum over subsets sigma it took 3.44 ms.
 constexpr int kMargSmem = 12;
-__global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, const double2* __restrict__ B, int m, double g,
+__global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, const double2* __restrict__ B, int m,
                                                                       const int* x, unsigned sizes,
                                                                       const double* coef, double* q) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -311,7 +325,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, con
     for (int r = threadIdx.x; r < binom[k][s]; r += blockDim.x) {
       const int T = unrank(k, s, r, binom), p = __ffs(T) - 1;
       const double2* row = Bx + p * k;
-      const double2 h = expand(H, T & (T - 1), g, [&](int i) { return row[i]; });
+      const double2 h = expand(H, T & (T - 1), [&](int i) { return row[i]; });
       H[T >> 1] = h;
       if (c != 0.0) acc = fma(c * (R.n ? rho_weight(R, T, binom) : 1.0), h.x * h.x + h.y * h.y, acc);
     }
@@ -322,7 +336,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_small_kernel(int k, con
 }
 
 // Longer prefixes: the tables in device memory, one launch per size.
-__global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int s, const double2* __restrict__ B, int m, double g,
+__global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int s, const double2* __restrict__ B, int m,
                                                                       const int* __restrict__ x, int batch,
                                                                       double2* __restrict__ H) {
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
@@ -339,13 +353,13 @@ __global__ void __launch_bounds__(kMargThreads) marginal_layer_kernel(int k, int
       continue;
     }
     const double2* row = B + (int64_t)xs[__ffs(T) - 1] * m;
-    Hb[T >> 1] = expand(Hb, T & (T - 1), g, [&](int i) { return __ldg(row + xs[i]); });
+    Hb[T >> 1] = expand(Hb, T & (T - 1), [&](int i) { return __ldg(row + xs[i]); });
   }
 }
 
 // q of prefix blockIdx.x from its sub-Hafnians: entry j of the classes has its
-// set's Hafnian at H[b * stride + T >> 1], or (list: Haf(B_T)) at H[b * stride + j].
-__global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, SubsetClasses rho, bool list, double g,
+// set's Hafnian at H[b * stride + T >> 1], or (list) at H[b * stride + j].
+__global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, SubsetClasses rho, bool list,
                                                                     const int* __restrict__ x,
                                                                     const double2* __restrict__ H, int64_t stride,
                                                                     const double* __restrict__ coef,
@@ -359,9 +373,7 @@ __global__ void __launch_bounds__(kMargThreads) marginal_sum_kernel(int k, Subse
   double acc = 0.0;
   for (int64_t j = threadIdx.x; j < rho.total(); j += blockDim.x) {
     const int T = subset_of(rho, j, binom);
-    double2 h = H[blockIdx.x * stride + (list ? j : T >> 1)];
-    if (list && g != 1.0)
-      for (int i = __popc(T); i > 0; i -= 2) h = make_double2(h.x * g, h.y * g);
+    const double2 h = H[blockIdx.x * stride + (list ? j : T >> 1)];
     acc = fma(coef[__popc(T) / 2] * (R.n ? rho_weight(R, T, binom) : 1.0), h.x * h.x + h.y * h.y, acc);
   }
   const double sum = block_sum(acc, red);
@@ -413,7 +425,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // common case) has weight 2 instead of 1 on the sets without its position, so
 // half the sets are enough for it; a repeated one goes through all of them.
 __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, const double2* cache,
-                                                                  int64_t cstride, const double2* __restrict__ B, double g,
+                                                                  int64_t cstride, const double2* __restrict__ B,
                                                                   const int* x, const double* coefs, double2* part) {
   __shared__ int binom[kMaxK + 1][kMaxK + 1];
   __shared__ Repeats R;
@@ -476,7 +488,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
           if (al == 0) continue;
           w = weight(T, __popc(T) + 1, extra) - w;
         }
-        const double2 h = expand(H, T, g, [&](int i) { return __ldg(row + xs[i]); });
+        const double2 h = expand(H, T, [&](int i) { return __ldg(row + xs[i]); });
         re = fma(w, h.x * h.x + h.y * h.y, re);
       }
     }
@@ -499,7 +511,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_gram_kernel(ChainStep S, c
 constexpr int kWeightThreads = 128;
 __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep S, const double2* cache,
                                                                       int64_t cstride, const double2* __restrict__ B,
-                                                                      double g, const int* x, const double* coefs,
+                                                                      const int* x, const double* coefs,
                                                                       const double2* part, double* q) {
   __shared__ double2 M[kMaxK * (kMaxK + 1) / 2], b[kMaxK][kWeightThreads];
   __shared__ double own[kMaxK], s_rho;
@@ -531,10 +543,7 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
   __syncthreads();
   if (S.direct && threadIdx.x == 0) find_repeats(R, xs, S.kp);
   if (l < S.m)
-    for (int i = 0; i < S.kp; ++i) {
-      const double2 v = __ldg(B + (int64_t)l * S.m + xs[i]);
-      b[i][threadIdx.x] = make_double2(v.x * g, v.y * g);
-    }
+    for (int i = 0; i < S.kp; ++i) b[i][threadIdx.x] = __ldg(B + (int64_t)l * S.m + xs[i]);
   __syncthreads();
   if (l >= S.m) return;
   int mult = 0, first = -1;
@@ -551,7 +560,7 @@ __global__ void __launch_bounds__(kWeightThreads) chain_weight_kernel(ChainStep 
     const double2* H = cache + (int64_t)smp * cstride;
     for (int r = 0; r < (int)S.odd.total(); ++r) {
       const int T = subset_of(S.odd, r, binom);
-      const double2 h = expand(H, T, 1.0, [&](int i) { return b[i][threadIdx.x]; });
+      const double2 h = expand(H, T, [&](int i) { return b[i][threadIdx.x]; });
       double w = coef[(__popc(T) + 1) / 2] * (R.n ? rho_weight(R, T, binom, extra) : 1.0);
       if (mult == 1 && !(T >> first & 1)) w *= 2.0;
       s = fma(w, h.x * h.x + h.y * h.y, s);
@@ -586,7 +595,7 @@ __global__ void chain_init_kernel(double2* __restrict__ cache, int64_t cstride, 
 constexpr int kPickModes = 2048;
 __global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, const double* q, const double* u, int* x,
                                                                   double2* cache, int64_t cstride,
-                                                                  const double2* __restrict__ B, double g) {
+                                                                  const double2* __restrict__ B) {
   __shared__ int s_pick;
   __shared__ int binom[kMaxK + 1][kMaxK + 1], xs[kMaxK];
   __shared__ double s_q[kPickModes];  // the weights, where they fit
@@ -635,7 +644,7 @@ __global__ void __launch_bounds__(kMargThreads) chain_pick_kernel(ChainStep S, c
   const double2* row = B + (int64_t)pick * m;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < (int)S.grow.total(); r += gridDim.x * blockDim.x) {
     const int T = subset_of(S.grow, r, binom);
-    c[(T | (1 << S.kp)) >> 1] = expand(c, T, g, [&](int i) { return __ldg(row + xs[i]); });
+    c[(T | (1 << S.kp)) >> 1] = expand(c, T, [&](int i) { return __ldg(row + xs[i]); });
   }
 }
 
@@ -715,18 +724,16 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
     }
   }
   for (int s = 2; s <= top; s += 2) table += (double)choose(kk, s) * (s - 1);
-  const double g = b_unit(k->t_uniform);
-  // (the batched path computes Haf(B_T) itself: only where it stays in range)
-  const bool list = kk > kMargSmem && single < table && -0.5 * top * log2(k->t_uniform) < 900.0;
+  const bool list = kk > kMargSmem && single < table;
   const bool small = !list && kk <= kMargSmem;
   const int64_t stride = list ? rho.total() : small ? 0 : (int64_t)1 << (kk - 1);
   // tables of at most 2 GB at once
   const int64_t group = small ? batch : std::max<int64_t>(1, std::min<int64_t>(batch, ((int64_t)1 << 27) / stride));
   auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
   const size_t H_b = al(16 * (size_t)(small ? 0 : group * stride)), c_b = al(8 * (size_t)(kMaxK + 1) * kCoefs);
-  const size_t x_b = al(4 * hx.size()), q_b = al(8 * (size_t)batch);
+  const size_t x_b = al(4 * hx.size()), q_b = al(8 * (size_t)batch), B_b = al(b_copy_bytes(k));
   void* tmp = nullptr;
-  cudaError_t e = scratch_alloc(&tmp, H_b + c_b + x_b + q_b, st);
+  cudaError_t e = scratch_alloc(&tmp, H_b + c_b + x_b + q_b + B_b, st);
   if (e != cudaSuccess) return fail(GBS_ENOMEM, "marginal scratch: %s", cudaGetErrorString(e));
   unsigned char* t = (unsigned char*)tmp;
   double2* d_H = (double2*)t;
@@ -734,7 +741,7 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
   int* d_x = (int*)(t + H_b + c_b);
   double* d_q = (double*)(t + H_b + c_b + x_b);
   const bool q_dev = is_device_ptr(q_out);
-  const double2* B = (const double2*)k->B;
+  const double2* B = (const double2*)scaled_B(k, t + H_b + c_b + x_b + q_b, st);
   const double* coef = d_c + (size_t)kk * kCoefs;
   int ret = GBS_OK;
   do {
@@ -742,11 +749,11 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
       ret = cuda_fail(e, "marginal upload");
       break;
     }
-    coef_kernel<<<1, kMargThreads, 0, st>>>(kk, n, k->m, size_scale(g * k->t_uniform), d_c);
+    coef_kernel<<<1, kMargThreads, 0, st>>>(kk, n, k->m, size_scale(k->t_uniform), d_c);
     double* qd = q_dev ? q_out : d_q;
     if (small) {
       e = launch_dependent(marginal_small_kernel, dim3(batch), kMargThreads, 16 * ((size_t)1 << std::max(kk - 1, 0)), st, kk,
-                           B, k->m, g, d_x, sizes, coef, qd);
+                           B, k->m, d_x, sizes, coef, qd);
       if (e != cudaSuccess) { ret = cuda_fail(e, "marginal kernel"); break; }
     } else {
       std::vector<int> idx, nv;
@@ -773,8 +780,7 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
           if (idx.empty()) idx.push_back(0);
           BatchArgs a;
           a.mode = BatchArgs::PROB;
-          a.B = k->B;
-          a.B32 = k->B32;
+          a.B = (const double*)B;
           a.m = k->m;
           a.log_norm_dev = k->dscal;
           a.idx = idx.data();
@@ -789,10 +795,10 @@ extern "C" int gbs_marginal_batch(const gbs_kernel* k, const int* x, int kk, int
           for (int s = 0; s <= top; s += 2) {
             const int64_t work = cnt * choose(kk, s);
             marginal_layer_kernel<<<(int)std::min<int64_t>(8192, (work + kMargThreads - 1) / kMargThreads), kMargThreads,
-                                    0, st>>>(kk, s, B, k->m, g, d_x + b0 * kk, cnt, d_H);
+                                    0, st>>>(kk, s, B, k->m, d_x + b0 * kk, cnt, d_H);
           }
         }
-        marginal_sum_kernel<<<cnt, kMargThreads, 0, st>>>(kk, rho, list, g, d_x + b0 * kk, d_H, stride, coef, qd + b0);
+        marginal_sum_kernel<<<cnt, kMargThreads, 0, st>>>(kk, rho, list, d_x + b0 * kk, d_H, stride, coef, qd + b0);
       }
       if (ret != GBS_OK) break;
     }
@@ -848,9 +854,9 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
   }
   const size_t cache_b = al(16 * (size_t)(group * cstride)), x_b = al(4 * (size_t)group * kMaxK);
   const size_t c_b = al(8 * (size_t)(kMaxK + 1) * kCoefs), q_b = al(8 * (size_t)group * m);
-  const size_t part_b = al(16 * (size_t)group * tasks), u_b = al(8 * (size_t)group * n);
+  const size_t part_b = al(16 * (size_t)group * tasks), u_b = al(8 * (size_t)group * n), B_b = al(b_copy_bytes(k));
   void* tmp = nullptr;
-  cudaError_t e = scratch_alloc(&tmp, cache_b + x_b + c_b + q_b + part_b + u_b, st);
+  cudaError_t e = scratch_alloc(&tmp, cache_b + x_b + c_b + q_b + part_b + u_b + B_b, st);
   if (e != cudaSuccess) return fail(GBS_ENOMEM, "chain scratch: %s", cudaGetErrorString(e));
   unsigned char* t = (unsigned char*)tmp;
   double2* d_cache = (double2*)t;
@@ -859,11 +865,10 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
   double* d_q = (double*)(t += c_b);
   double2* d_part = (double2*)(t += q_b);
   double* d_u = (double*)(t += part_b);
-  const double2* B = (const double2*)k->B;
+  const double2* B = (const double2*)scaled_B(k, t + u_b, st);
   std::vector<int> hx((size_t)group * kMaxK);
   int ret = GBS_OK;
-  const double g = b_unit(k->t_uniform);
-  coef_kernel<<<n, kMargThreads, 0, st>>>(1, n, m, size_scale(g * k->t_uniform), d_c);
+  coef_kernel<<<n, kMargThreads, 0, st>>>(1, n, m, size_scale(k->t_uniform), d_c);
   if ((e = cudaGetLastError()) != cudaSuccess) ret = cuda_fail(e, "chain coefficients");
   for (int s0 = 0; s0 < samples && ret == GBS_OK; s0 += group) {
     const int S = std::min(group, samples - s0);
@@ -878,14 +883,14 @@ extern "C" int gbs_sample_chain_batch(const gbs_kernel* k, int n, int samples, c
       const ChainStep& C = steps[kk];
       constexpr int wpb = kMargThreads / 32;
       e = launch_dependent(chain_gram_kernel, dim3((C.tasks + wpb - 1) / wpb, S), kMargThreads, 0, st, C, d_cache, cstride,
-                           B, g, d_x, d_c, d_part);
+                           B, d_x, d_c, d_part);
       if (e == cudaSuccess)
         e = launch_dependent(chain_weight_kernel, dim3((m + kWeightThreads - 1) / kWeightThreads, S), kWeightThreads, 0, st,
-                             C, d_cache, cstride, B, g, d_x, d_c, d_part, d_q);
+                             C, d_cache, cstride, B, d_x, d_c, d_part, d_q);
       // the draws, then the chosen modes' new sub-Hafnians into the caches
       const int nb = kk < n ? (int)std::max<int64_t>(1, std::min<int64_t>(64, (C.grow.total() + 255) / 256)) : 1;
       if (e == cudaSuccess)
-        e = launch_dependent(chain_pick_kernel, dim3(nb, S), kMargThreads, 0, st, C, d_q, d_u, d_x, d_cache, cstride, B, g);
+        e = launch_dependent(chain_pick_kernel, dim3(nb, S), kMargThreads, 0, st, C, d_q, d_u, d_x, d_cache, cstride, B);
       if (e != cudaSuccess) break;
     }
     if (e != cudaSuccess) {
