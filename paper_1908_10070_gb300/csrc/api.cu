@@ -1271,7 +1271,7 @@ int run_batch(const BatchArgs& a) {
   HafLaunch L;
   memset(&L, 0, sizeof(L));
   int ret = GBS_OK;
-  SideWork side;  // joined before the scratch is freed
+  SideWork side, rep_side;  // joined before the scratch is freed
   void* h_outs = nullptr;  // pinned copy of the output staging (host outputs)
   int oslot = -1;
   const size_t out_sz[4] = {sizeof(double) * batch, sizeof(double) * batch, 2 * sizeof(double) * batch,
@@ -1346,6 +1346,28 @@ int run_batch(const BatchArgs& a) {
         e = launch_route_plan(RP, st);
         if (e != cudaSuccess) { ret = cuda_fail(e, "route choice launch"); break; }
         L.skip = d_rephalf;
+        // Beside the larger orders' chain of layers, which is launched (90 us of
+        // nearly empty kernels at order 24) also when the repeated-row sum takes
+        // every matrix.
+        if (U.match && U.match_b) rep_side.begin(st);
+        else rep_side.here(st);
+        // the patterns the device chose for the repeated-row sum (the item
+        // count is read on the device; the grid covers the reservation)
+        RepLaunch R;
+        R.B = a.B;
+        R.idx = d_idx;
+        R.pats = d_pats;
+        R.n_items = (int)dev_rep_cap;
+        R.n_items_dev = d_ctr + 56;
+        R.m_bound = L.m_bound;
+        R.counter = d_ctr + 58;
+        R.status = d_status;
+        R.parts = d_repparts;
+        R.rep_half = d_rephalf;
+        R.rep_end = d_repend;
+        R.batch = batch;
+        e = launch_haf_repeated(R, rep_side.stream());
+        if (e != cudaSuccess) { ret = cuda_fail(e, "repeated-row kernel launch"); break; }
       }
       if (U.match) {
         MatchLaunch M;
@@ -1450,26 +1472,8 @@ int run_batch(const BatchArgs& a) {
         e = launch_haf_subsets(L, a.precision, blocks, cfg.warps_per_block, st);
         if (e != cudaSuccess) { ret = cuda_fail(e, "subset kernel launch"); break; }
       }
-      if (dev_rep_cap) {
-        // the patterns the device chose for the repeated-row sum (the item
-        // count is read on the device; the grid covers the reservation)
-        RepLaunch R;
-        R.B = a.B;
-        R.idx = d_idx;
-        R.pats = d_pats;
-        R.n_items = (int)dev_rep_cap;
-        R.n_items_dev = d_ctr + 56;
-        R.m_bound = L.m_bound;
-        R.counter = d_ctr + 58;
-        R.status = d_status;
-        R.parts = d_repparts;
-        R.rep_half = d_rephalf;
-        R.rep_end = d_repend;
-        R.batch = batch;
-        e = launch_haf_repeated(R, st);
-        if (e != cudaSuccess) { ret = cuda_fail(e, "repeated-row kernel launch"); break; }
-      }
       e = side.join();
+      if (e == cudaSuccess) e = rep_side.join();
       if (e != cudaSuccess) { ret = cuda_fail(e, "side stream"); break; }
       if (timed) cudaEventRecord(g_time_stop, st);
     }

@@ -1234,36 +1234,46 @@ __global__ void pairing_select_kernel(const PairingSelect S) {
 // kRepLow digit combinations) and high ones; the low ones again into two
 // groups of T1 and T2 combinations.
 constexpr int kRepLow = 256;
-struct RepWarp {
+constexpr int kRepWarps = 4;  // warps of a block, which takes one item at a time
+struct RepItem {
   double2 B[kRepMaxDistinct * kRepMaxDistinct];  // B_v, row stride kRepMaxDistinct
   double2 C[kRepLow];           // x^T B_v x / 2 over the low modes, per combination
-  double2 S1[kMaxN + 2];        // per combination of the first group: its x . y, plus the high modes' share
-  double2 S2[kRepLow / 2];      // per combination of the second group: its x . y
-  double2 y[kRepMaxDistinct];   // B_v x over the high modes, per low mode
   double w[kRepLow];            // prod (-1)^nu_j C(c_j, nu_j) over the low modes
-  int c[kRepMaxDistinct];                         // multiplicities c_j
-  int mode[kRepMaxDistinct];                      // distinct modes v_j
+  struct {                      // per warp:
+    double2 S1[kMaxN + 2];      // per combination of the first group: its x . y, plus the high modes' share
+    double2 S2[kRepLow / 2];    // per combination of the second group: its x . y
+    double2 y[kRepMaxDistinct]; // B_v x over the high modes, per low mode
+  } warp[kRepWarps];
+  double sum[5][kRepWarps][32]; // the lanes' sums
+  int c[kRepMaxDistinct];       // multiplicities c_j
+  int mode[kRepMaxDistinct];    // distinct modes v_j
 };
 
-// Warp sum of compensated accumulators (fixed butterfly, double-double) into
-// one item partial.
+// Warp sum of compensated accumulators (fixed tree, double-double) into one
+// item partial: the real parts in the lower half of the warp, the imaginary
+// ones in the upper half.
 __device__ __forceinline__ void store_warp_partial(Comp<double> re, Comp<double> im, double kap, int lane,
                                                    Partial* out) {
   const unsigned FULL = 0xffffffffu;
-  double rh = re.hi, rl = re.lo, ih = im.hi, il = im.lo;
-  for (int off = 16; off > 0; off >>= 1) {
-    const double orh = __shfl_xor_sync(FULL, rh, off), orl = __shfl_xor_sync(FULL, rl, off);
-    const double oih = __shfl_xor_sync(FULL, ih, off), oil = __shfl_xor_sync(FULL, il, off);
+  const bool up = lane >= 16;
+  double hi = up ? im.hi : re.hi, lo = up ? im.lo : re.lo;
+  double ohi = __shfl_xor_sync(FULL, up ? re.hi : im.hi, 16), olo = __shfl_xor_sync(FULL, up ? re.lo : im.lo, 16);
+  kap += __shfl_xor_sync(FULL, kap, 16);
+  dd_add(hi, lo, ohi, olo);
+  for (int off = 8; off > 0; off >>= 1) {
+    ohi = __shfl_xor_sync(FULL, hi, off);
+    olo = __shfl_xor_sync(FULL, lo, off);
     kap += __shfl_xor_sync(FULL, kap, off);
-    dd_add(rh, rl, orh, orl);
-    dd_add(ih, il, oih, oil);
+    dd_add(hi, lo, ohi, olo);
   }
+  ohi = __shfl_sync(FULL, hi, 16);
+  olo = __shfl_sync(FULL, lo, 16);
   if (lane == 0) {
     Partial pr;
-    pr.re_hi = rh;
-    pr.re_lo = rl;
-    pr.im_hi = ih;
-    pr.im_lo = il;
+    pr.re_hi = hi;
+    pr.re_lo = lo;
+    pr.im_hi = ohi;
+    pr.im_lo = olo;
     pr.kappa = kap;
     pr.pad[0] = pr.pad[1] = pr.pad[2] = 0.0;
     *out = pr;
@@ -1280,9 +1290,9 @@ __device__ __forceinline__ void sum_add(Comp<double>& a, double v) {
 
 // Terms t0 <= t < t0 + count for D distinct modes: digits nu_j of t (mixed
 // radix c_j + 1, j = 0 fastest), x_j = c_j - 2 nu_j, the weight prod (-1)^nu_j
-// C(c_j, nu_j), Q = x^T B_v x / 2, Q^h by squaring, and the term times
-// 2 / (2^n h!) (1 / (2^n h!) for the middle term t = (T - 1) / 2, which is its
-// own mirror).
+// C(c_j, nu_j), Q = x^T B_v x / 2, Q^h by squaring (half for the middle term
+// t = (T - 1) / 2, which is its own mirror). The sums' common factor
+// 2 / (2^n h!) is left to the caller.
 //
 // Q = C[l] + (x . y over the low modes) + (the high modes alone), l the low
 // digits: C depends on the pattern only, y and the high share on the high
@@ -1293,17 +1303,27 @@ __device__ __forceinline__ void sum_add(Comp<double>& a, double v) {
 // bounds it: 512 patterns of n = 24 in 8 modes (2^15 terms each) went from
 // 3.5 to 1.75 ms (whole call). The sum keeps its rounding errors (Knuth's two-sum, once a
 // component and term), as it did.
-__device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN + 1], int D, int h, int t0,
-                                          int count, int T, double scale, int lane, Comp<double>& re,
+//
+// The block's warps share C and w and take the values of the high digits in
+// turn, a class H mod 4 each (another one from item to item, as `turn` says:
+// the classes with one value more are not one SM quarter's). One warp
+// an item left a few long ones alone on their SM quarters: a call for 64
+// patterns of 24 photons in 4 modes (128 items, 21 values of H each) took 366
+// us, 298 with the quadratic form per term, and takes 137; 512 patterns of 24
+// in 8 modes 1698 -> 1672.
+__device__ __forceinline__ void rep_terms(RepItem& W, const int (*binom)[kMaxN + 1], int D, int h, int t0,
+                                          int count, int T, int turn, Comp<double>& re,
                                           Comp<double>& im, double& kap) {
   const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, cls = ((threadIdx.x >> 5) + turn) & (kRepWarps - 1);
+  auto& V = W.warp[threadIdx.x >> 5];
   // low modes [0, dl), the first group [0, d1)
   int dl = 1, TL = W.c[0] + 1;
   while (dl < D && TL * (W.c[dl] + 1) <= kRepLow) TL *= W.c[dl++] + 1;
   int d1 = 1, T1 = W.c[0] + 1;
   while (d1 < dl && T1 * (W.c[d1] + 1) <= 32) T1 *= W.c[d1++] + 1;
   const int T2 = TL / T1;
-  for (int l = lane; l < TL; l += 32) {
+  for (int l = threadIdx.x; l < TL; l += kRepWarps * 32) {
     double w = 1.0, qr = 0.0, qi = 0.0;
     int rem = l;
     for (int j = 0; j < dl; ++j) {
@@ -1328,8 +1348,10 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
     W.w[l] = w;
     W.C[l] = make_double2(qr, qi);
   }
+  __syncthreads();
   double kp = 0.0;
-  for (int H = t0 / TL; (int64_t)H * TL < t0 + count; ++H) {
+  const int H0 = t0 / TL;
+  for (int H = H0 + ((cls - H0) & (kRepWarps - 1)); (int64_t)H * TL < t0 + count; H += kRepWarps) {
     const int base = H * TL;
     // the high digits' weight; lane j < dl takes y_j, lane j >= dl the high
     // mode j's x_j (B_jj x_j / 2 + sum_{k > j} B_jk x_k)
@@ -1349,7 +1371,7 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
       }
     }
     __syncwarp();
-    if (lane < dl) W.y[lane] = make_double2(ar, ai);
+    if (lane < dl) V.y[lane] = make_double2(ar, ai);
     // lanes outside [dl, D) hold xl = 0
     double hr = ar * xl, hi = ai * xl;
     for (int off = 8; off > 0; off >>= 1) {
@@ -1367,17 +1389,17 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
         const int cj = W.c[j];
         const double xj = (double)(cj - 2 * (r % (cj + 1)));
         r /= (cj + 1);
-        const double2 y = W.y[j];
+        const double2 y = V.y[j];
         sr = fma(xj, y.x, sr);
         si = fma(xj, y.y, si);
       }
-      (first ? W.S1[l] : W.S2[l - T1]) = make_double2(sr, si);
+      (first ? V.S1[l] : V.S2[l - T1]) = make_double2(sr, si);
     }
     __syncwarp();
     const int end = min(TL, t0 + count - base);
     for (int l = max(t0 - base, 0) + lane; l < end; l += 32) {
       const int l2 = l / T1, l1 = l - l2 * T1;
-      const double2 c = W.C[l], s1 = W.S1[l1], s2 = W.S2[l2];
+      const double2 c = W.C[l], s1 = V.S1[l1], s2 = V.S2[l2];
       const double qr = c.x + (s1.x + s2.x), qi = c.y + (s1.y + s2.y);
       double pr = 1.0, pi = 0.0, br = qr, bi = qi;
       bool one = true;  // p = 1 (uniform: the exponent is)
@@ -1408,26 +1430,17 @@ __device__ __forceinline__ void rep_terms(RepWarp& W, const int (*binom)[kMaxN +
     }
     __syncwarp();
   }
-  // the common factor 2 / (2^n h!)
-  const double g = 2.0 * scale;
-  auto scaled = [&](Comp<double>& a) {
-    const double p = a.hi * g;
-    a.lo = fma(a.hi, g, -p) + a.lo * g;
-    a.hi = p;
-  };
-  scaled(re);
-  scaled(im);
-  kap += kp * g;
+  kap = kp;
 }
 
-// Persistent warps over repeated-row work items. Per item: the matrix's index
+// Persistent blocks over repeated-row work items. Per item: the matrix's index
 // list (lane i holds x_i), its distinct modes and multiplicities by
-// __match_any_sync (order of first occurrence), B_v gathered into the warp's
-// shared slot, then the item's terms.
-__global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
+// __match_any_sync (order of first occurrence), B_v gathered into shared
+// memory, then the item's terms.
+__global__ void __launch_bounds__(kRepWarps * 32) haf_repeated_kernel(const RepLaunch R) {
   extern __shared__ __align__(16) unsigned char rep_smem[];
-  RepWarp* ws = reinterpret_cast<RepWarp*>(rep_smem);
-  __shared__ int binom[kMaxN + 1][kMaxN + 1];
+  RepItem& W = *reinterpret_cast<RepItem*>(rep_smem);
+  __shared__ int binom[kMaxN + 1][kMaxN + 1], s_it;
   dependency_wait();
   // the grid covers the reservation; with no item (no bunched pattern) every
   // block leaves before building its table (uniform over the block)
@@ -1444,12 +1457,13 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
   __syncthreads();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  RepWarp& W = ws[threadIdx.x >> 5];
   const double2* src2 = reinterpret_cast<const double2*>(R.B);
   for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(R.counter, 1);
-    it = __shfl_sync(FULL, it, 0);
+    // (everything up to the sums is the same in every warp)
+    if (threadIdx.x == 0) s_it = atomicAdd(R.counter, 1);
+    __syncthreads();
+    const int it = s_it;
+    __syncthreads();
     if (it >= n_items) break;
     WorkItem w;
     // route choice on the device: the pattern whose partial range holds
@@ -1472,10 +1486,9 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
     w.s_last = 0;
     w.aux = 0;
     if (half <= 0 || c < 0 || c >= chunks) {  // never for a consistent plan
-      if (lane == 0) R.status[lo] = 1;
+      if (threadIdx.x == 0) R.status[lo] = 1;
       const Comp<double> z = {0.0, 0.0};
-      store_warp_partial(z, z, 0.0, lane, R.parts + it);
-      __syncwarp();
+      if (threadIdx.x < 32) store_warp_partial(z, z, 0.0, lane, R.parts + it);
       continue;
     }
     const PatDesc d = R.pats[w.pat];
@@ -1493,33 +1506,59 @@ __global__ void __launch_bounds__(128) haf_repeated_kernel(const RepLaunch R) {
     if (__any_sync(FULL, bad) || D > kRepMaxDistinct) {
       // an out-of-range index (NaN output) or a matrix this route was not
       // planned for: flag it, leave a zero partial, read nothing
-      if (lane == 0) R.status[w.pat] = 1;
+      if (threadIdx.x == 0) R.status[w.pat] = 1;
       const Comp<double> z = {0.0, 0.0};
-      store_warp_partial(z, z, 0.0, lane, R.parts + w.part);
-      __syncwarp();
+      if (threadIdx.x < 32) store_warp_partial(z, z, 0.0, lane, R.parts + w.part);
       continue;
     }
-    if (leader) {
+    if (leader && threadIdx.x < 32) {
       const int j = __popc(leaders & ((1u << lane) - 1u));
       W.mode[j] = v;
       W.c[j] = __popc(same);
     }
-    __syncwarp();
-    for (int e = lane; e < D * D; e += 32) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < D * D; e += kRepWarps * 32) {
       const int j = e / D, k = e - j * D;
       W.B[j * kRepMaxDistinct + k] = __ldg(src2 + d.src_off + (int64_t)W.mode[j] * d.ld + W.mode[k]);
     }
-    __syncwarp();
+    __syncthreads();
     int T = 1;
     for (int j = 0; j < D; ++j) T *= W.c[j] + 1;
-    double hf = 1.0;
-    for (int i = 2; i <= h; ++i) hf *= (double)i;  // exact: h! < 2^53 for h <= 16
-    const double scale = ldexp(1.0 / hf, -n);
     Comp<double> re = {0.0, 0.0}, im = {0.0, 0.0};
     double kap = 0.0;
-    rep_terms(W, binom, D, h, w.rank0, w.count, T, scale, lane, re, im, kap);
-    store_warp_partial(re, im, kap, lane, R.parts + w.part);
-    __syncwarp();
+    rep_terms(W, binom, D, h, w.rank0, w.count, T, it, re, im, kap);
+    // the four classes in their order, lane by lane, then the lanes
+    {
+      const int cls = ((threadIdx.x >> 5) + it) & (kRepWarps - 1);
+      W.sum[0][cls][lane] = re.hi;
+      W.sum[1][cls][lane] = re.lo;
+      W.sum[2][cls][lane] = im.hi;
+      W.sum[3][cls][lane] = im.lo;
+      W.sum[4][cls][lane] = kap;
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      Comp<double> a = {W.sum[0][0][lane], W.sum[1][0][lane]}, b = {W.sum[2][0][lane], W.sum[3][0][lane]};
+      double q = W.sum[4][0][lane];
+      for (int c2 = 1; c2 < kRepWarps; ++c2) {
+        sum_add(a, W.sum[0][c2][lane]);
+        a.lo += W.sum[1][c2][lane];
+        sum_add(b, W.sum[2][c2][lane]);
+        b.lo += W.sum[3][c2][lane];
+        q += W.sum[4][c2][lane];
+      }
+      double hf = 1.0;
+      for (int i = 2; i <= h; ++i) hf *= (double)i;  // exact: h! < 2^53 for h <= 16
+      const double f = 2.0 * ldexp(1.0 / hf, -n);
+      auto scaled = [&](Comp<double>& v2) {
+        const double p = v2.hi * f;
+        v2.lo = fma(v2.hi, f, -p) + v2.lo * f;
+        v2.hi = p;
+      };
+      scaled(a);
+      scaled(b);
+      store_warp_partial(a, b, q * f, lane, R.parts + w.part);
+    }
   }
 }
 
@@ -1632,17 +1671,17 @@ cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  constexpr int smem = 4 * (int)sizeof(RepWarp);
+  constexpr int smem = (int)sizeof(RepItem);
   static std::atomic<int> done[64];
   if (!done[dev].load(std::memory_order_acquire)) {
     const cudaError_t e = cudaFuncSetAttribute(haf_repeated_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     done[dev].store(1, std::memory_order_release);
   }
-  int blocks = (R.n_items + 3) / 4;
-  const int cap = (sms > 0 ? sms : 1) * (int)std::min<size_t>(8, (size_t)220 * 1024 / smem);
+  int blocks = R.n_items;
+  const int cap = (sms > 0 ? sms : 1) * (int)std::min<size_t>(8, (size_t)200 * 1024 / smem);
   if (blocks > cap) blocks = cap;
-  return launch_dependent(haf_repeated_kernel, dim3(blocks), 128, smem, st, R);
+  return launch_dependent(haf_repeated_kernel, dim3(blocks), kRepWarps * 32, smem, st, R);
 }
 
 cudaError_t launch_pairing_select(const PairingSelect& S, cudaStream_t st) {
