@@ -1388,7 +1388,10 @@ int run_batch(const BatchArgs& a) {
         // fill the SMs gain nothing there (4096 patterns of n = 16: the terms
         // wait for room as long as the tiles run).
         const bool shared = U.terms && U.n_order > 0;
-        const bool few = U.n_tiles <= device_sm_count();
+        // Up to order 4 they are shorter than the side stream's events (one
+        // pattern with its estimate, beside or after: n = 2 50.8 and 46.6 us,
+        // n = 4 52.8 and 50.4, n = 6 63.9 and 65.5, n = 10 79.9 and 87.8).
+        const bool few = U.n_tiles <= device_sm_count() && maxn > 4;
         const bool beside = (shared && (U.match_b || few)) || (U.n_tiles && U.match_b);
         if (beside) side.begin(st);
         else side.here(st);
@@ -1462,8 +1465,9 @@ int run_batch(const BatchArgs& a) {
           T.left = d_ctr + 43;
           std::vector<TermsChunk> chunks;
           terms_chunks(U, d_arena, &chunks);
+          // (a second chunk's scratch is the first one's)
           for (const TermsChunk& c : chunks)
-            if ((e = launch_terms(T, c, st)) != cudaSuccess) break;
+            if ((e = launch_terms(T, c, st, chunks.size() == 1 ? side.stream() : st)) != cudaSuccess) break;
           if (e != cudaSuccess) { ret = cuda_fail(e, "terms kernel launch"); break; }
         }
       } else {

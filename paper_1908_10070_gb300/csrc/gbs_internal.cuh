@@ -437,8 +437,9 @@ cudaError_t launch_match_large(const MatchLaunch& L, MatchChunk C, bool shared, 
 
 // Defined in haf_subsets.cu
 cudaError_t launch_haf_repeated(const RepLaunch& R, cudaStream_t st);
-// The terms of a chunk's matrices, and the check.
-cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st);
+// The terms of a chunk's matrices, and the check. The orders below
+// kTermsFixedMin go to `small_st` where the chunk has others too.
+cudaError_t launch_terms(const TermsLaunch& T, TermsChunk C, cudaStream_t st, cudaStream_t small_st);
 cudaError_t launch_route_plan(const RoutePlan& R, cudaStream_t st);
 cudaError_t launch_haf_subsets(const HafLaunch& L, int precision, int blocks, int warps_per_block,
                                cudaStream_t st);

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(kDeltaThreads) terms64_delta_kernel(const Term
   }
   dependency_wait();
   __syncthreads();
-  const int items = *P.left ? C.items64 : C.small64;
+  const int items = C.small64 < C.items64 && *P.left ? C.items64 : C.small64;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     int g = C.n_groups - 1;  // (items are numbered from the smallest order on)
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kSeries64) terms64_series_kernel(const TermsLa
   constexpr int ld = kSeries64 + 1, bits = 7;
   dependency_wait();
   __syncthreads();
-  const bool left = *P.left != 0;
+  const bool left = C.small64 < C.items64 && *P.left != 0;
   const int col = threadIdx.x;
   // coefficient k of a column at [k - 1][column]: D_S^{-1/2}, and G_S
   double2* ys = reinterpret_cast<double2*>(smem);
