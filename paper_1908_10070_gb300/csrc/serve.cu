@@ -528,10 +528,12 @@ bool whole_only(const Stage& g) { return !g.whole.empty() && !g.n_items[0] && !g
 int launch_whole(gbs_server* s, Stage& g) {
   const int S = s->o.max_slots, cnt = (int)g.whole.size();
   unsigned long long* d_stamp = (unsigned long long*)(g.d_wres + 5 * S);
-  cudaError_t e = cudaEventRecord(g.ev0, s->st);
-  if (e == cudaSuccess) {
+  cudaError_t e = cudaSuccess;
+  if (s->o.use_graphs) {  // (a graph's steps are timed by stamps, direct ones by events)
     stamp_kernel<<<1, 1, 0, s->st>>>(d_stamp);
     e = cudaGetLastError();
+  } else {
+    e = cudaEventRecord(g.ev0, s->st);
   }
   if (e != cudaSuccess) return GBS_ECUDA;
   BatchArgs a;
@@ -552,8 +554,10 @@ int launch_whole(gbs_server* s, Stage& g) {
   a.stage_b = batch_stage_bytes(S);
   const int rc = run_batch(a);
   if (rc != GBS_OK) return rc;
-  end_kernel<<<1, 1, 0, s->st>>>(d_stamp + 1, (unsigned long long)(g.id & 0x7fffffff));
-  e = cudaGetLastError();
+  if (s->o.use_graphs) {
+    end_kernel<<<1, 1, 0, s->st>>>(d_stamp + 1, (unsigned long long)(g.id & 0x7fffffff));
+    e = cudaGetLastError();
+  }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(g.h_wres, g.d_wres, sizeof(double) * (5 * S + 2), cudaMemcpyDeviceToHost, s->st);
   return e == cudaSuccess ? GBS_OK : GBS_ECUDA;
@@ -572,10 +576,11 @@ cudaError_t launch_stage(gbs_server* s, Stage& g) {
   const int S = s->o.max_slots;
   auto t0 = std::chrono::steady_clock::now();
   cudaError_t e;
-  if (s->o.use_graphs && whole_only(g)) {
-    // nothing for the graph: its end event and completion word alone
+  if (whole_only(g)) {
+    // nothing beside the whole requests: the end event, and the completion
+    // word where a graph's step would bring it
     e = cudaEventRecord(g.ev, s->st);
-    if (e == cudaSuccess)
+    if (e == cudaSuccess && s->o.use_graphs)
       e = cudaMemcpyAsync(g.h_res + 5 * S + 2, g.d_wres + 5 * S + 2, sizeof(int), cudaMemcpyDeviceToHost, s->st);
     note_max(s->stats.submit_max_s, t0);
     return e;
