@@ -5,9 +5,11 @@ collision-free patterns of n = 16 photons, FP64 path, one batched call per step.
 `value` = patterns / device time of the step with inputs resident in HBM;
 `e2e` = the same through the C ABI with host index lists and host outputs.
 
-Also reported (`extra`): the mixed FP32 path on the same workload, the mixed-n
-collision workload (M = 144), the large instances (M = 900, n = 28 and 30) and
-the serving loop (Poisson stream, p50/p99 latency), unless --quick.
+Also measured, unless --quick: the mixed FP32 path on the same workload, the
+mixed-n collision workload (M = 144), the large instances (M = 900, n = 28 and
+30), bunched patterns, the serving loop (Poisson stream, p50/p99 latency) and
+the samplers. They go to standard error, a JSON object a line; standard output
+is the one short line of the headline.
 
 `--impl reference` times the CPU oracle (plain C, FP64 subset sum with repeated
 products, OpenMP over patterns) on a bounded sample of the same workload.
@@ -59,17 +61,25 @@ def term_macs(n: int) -> int:
                for s in range(1, h + 1))
 
 
-def model_flops(n: int, terms: bool = True) -> float:
-    """Flops of one FP64 result, 8 per complex multiply-add: the matchings (FP64
-    pipe) and, with the error estimate, the terms (whole numbers and FP32)."""
-    return 8.0 * (matching_macs(n) + (term_macs(n) if terms else 0))
+FIXED_MIN = 14  # smallest order whose terms are formed in fixed point
+
+
+def fixed_point_flops(n: int) -> float:
+    """Flops (8 per complex multiply-add) of one FP64 result with its estimate that
+    run in whole numbers and FP32: the terms of the larger orders."""
+    return 8.0 * term_macs(n) if n >= FIXED_MIN else 0.0
+
+
+def fp64_flops(n: int) -> float:
+    """Those that run on the FP64 pipe: the matchings, and a small order's terms."""
+    return 8.0 * (matching_macs(n) + (term_macs(n) if n < FIXED_MIN else 0))
 
 
 def fixed_point_peak_tflops() -> float:
-    """Peak of the terms' complex multiply-add, measured at 32
-    clocks a warp and SM quarter with 4 IMAD.WIDE and 8 FFMA (one a clock and
-    quarter, 8 flops each; the kernel takes 3 IMAD.WIDE)."""
-    return SMS * 4 * 8.0 * SM_MHZ_MAX * 1e6 / 1e12
+    """Peak of the terms' complex multiply-add: 3 IMAD.WIDE and 8 FFMA take 28 clocks
+    of a warp and SM quarter (IMAD.WIDE 32 lanes a clock and SM, FFMA 128), for 32
+    multiply-adds of 8 flops."""
+    return SMS * 4 * 8.0 * 32.0 / 28.0 * SM_MHZ_MAX * 1e6 / 1e12
 
 
 def fp64_peak_tflops() -> float:
@@ -270,6 +280,15 @@ def reference_arm(args):
     print(json.dumps(line), flush=True)
 
 
+def emit(line, extra):
+    """The other workloads to standard error, one JSON object a line, then the
+    headline alone to standard output (with the others in it the line grew to
+    tens of kilobytes, which a reader of the last few lost)."""
+    for key, value in extra.items():
+        print(json.dumps({key: value}), file=sys.stderr, flush=True)
+    print(json.dumps(line), flush=True)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -365,10 +384,11 @@ def main():
     e2e_s = (time.perf_counter() - t0) / e2e_steps
     assert np.array_equal(hh, hf.cpu().numpy()), "host and device paths disagree"
 
-    # the FP64 route: its terms set the time (whole numbers and FP32); the
-    # float kernel is counted by one N x N complex product per subset
+    # the FP64 route: its terms (whole numbers and FP32) set the time, beside
+    # the matchings on the FP64 pipe, each against its own peak; the float
+    # kernel is counted by one N x N complex product per subset
     fp64 = prec == gbs.FP64
-    flops = (model_flops(16) if fp64 else 64.0 * 2 ** 5 * 64 * 11) * b
+    flops = (fixed_point_flops(16) if fp64 else 64.0 * 2 ** 5 * 64 * 11) * b
     peak = fixed_point_peak_tflops() if fp64 else fp32_peak_tflops()
     achieved = flops / (t_kern * 1e-3) / 1e12
     # the FP64 pipe's measured throughput (DFMA microbenchmark in the library),
@@ -386,36 +406,34 @@ def main():
                    "autotuned_rounds_per_item": tuned_rounds},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                      "frac": achieved / peak,
-                     "traffic": None,
                      "hafnian_terms_per_s": b * (2 ** 8 - 1) / (t_kern * 1e-3),
                      "kernel": ("terms_delta_kernel, terms_series_kernel, match_small_kernel" if fp64
                                 else "haf_subsets_kernel<float>"),
                      "kernel_ms": t_kern,
                      "flops_per_launch": flops,
-                     "peak_note": ("one complex multiply-add in fixed point (4 IMAD.WIDE, 8 FFMA) a clock and SM quarter, "
-                                   "152 SM x 4 x 8 flop x 2.07 GHz" if fp64 else
+                     "peak_note": ("terms: a warp's complex multiply-add in fixed point (3 IMAD.WIDE, 8 FFMA) in 28 "
+                                   "clocks of an SM quarter, 152 SM x 4 x 32 x 8 flop / 28 x 2.07 GHz" if fp64 else
                                    "FP32 from unit counts and clock (152 SM x 256 flop/clk x 2.07 GHz)"),
                      "measured_fp64_peak": measured_peak,
                      "matching_flops_frac_of_measured_fp64_peak":
-                         (8.0 * matching_macs(16) * b / (t_kern * 1e-3) / 1e12 / measured_peak) if fp64 else None,
+                         (fp64_flops(16) * b / (t_kern * 1e-3) / 1e12 / measured_peak) if fp64 else None,
                      "measured_peak_note": "gbs_measure_fp64_peak (independent DFMA chains on every SM), "
                                            "SM clock %s MHz during it" % pclk_s.get("sm_mhz")},
         "e2e": {"value": world * b / e2e_s, "unit": UNIT, "h2d_bytes_per_step": int(idx.nbytes),
                 "d2h_bytes_per_step": int(hp.nbytes + hl.nbytes + hh.nbytes + he.nbytes)},
-        # per step, FP64: the route choice, the matchings, the terms' preparation,
-        # two kernels and check, the subset kernel behind them, the repeated-row
-        # kernel, finalisation; mixed: the subset kernel, finalisation
-        "gpu_launches": (9 if prec == gbs.FP64 else 2) * args.steps,
+        # per step, FP64: the route choice, the repeated-row kernel, the matchings,
+        # the terms' preparation, two kernels and check, the two FP64 kernels
+        # behind them, finalisation; mixed: the subset kernel, finalisation
+        "gpu_launches": (10 if prec == gbs.FP64 else 2) * args.steps,
         "clocks": clk.summary(),
     }
     if rank == 0 and not args.no_cpu_baseline and world == 1 and prec == gbs.FP64:
         line["cpu_baseline"] = cpu_baseline(pats, U, r)
     # the other workloads, serving and the samplers: one-GPU runs only (a
     # multi-rank run holds every GPU meanwhile)
-    if rank == 0 and not args.quick and world == 1:
-        line["extra"] = extras(gbs, torch, measured_peak)
+    extra = extras(gbs, torch, measured_peak) if rank == 0 and not args.quick and world == 1 else {}
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        emit(line, extra)
     if dist:
         dist.destroy_process_group()
 
@@ -558,11 +576,11 @@ def profile_chain(args, torch, gbs):
 
 def extras(gbs, torch, measured_peak):
     out = {}
-    peak = fixed_point_peak_tflops()
 
-    def frac(fl, ms):  # matchings and terms against the terms' multiply-add rate
-        a = fl / (ms * 1e-3) / 1e12
-        return {"achieved_tflops": a, "frac_of_fixed_point_peak": a / peak}
+    def frac(pats, ms):  # the terms in fixed point, and what runs on the FP64 pipe, each against its own peak
+        fx, f64 = (sum(f(len(p)) for p in pats) / (ms * 1e-3) / 1e12 for f in (fixed_point_flops, fp64_flops))
+        return {"fixed_point_tflops": fx, "frac_of_fixed_point_peak": fx / fixed_point_peak_tflops(),
+                "fp64_tflops": f64, "frac_of_measured_fp64_peak": f64 / measured_peak if measured_peak else None}
 
     # mixed path on the headline workload
     U, r, pats = W.workload(WORKLOAD)
@@ -583,9 +601,8 @@ def extras(gbs, torch, measured_peak):
         gbs.autotune(nn, gbs.MIXED)
     t64, k64, h64, e64 = timed_batch(gbs, torch, K, pats, gbs.FP64)
     t32, k32, h32, e32 = timed_batch(gbs, torch, K, pats, gbs.MIXED)
-    fl = sum(model_flops(len(p)) for p in pats)
     out["mixed_m144"] = {"fp64_probs_per_s": len(pats) / (t64 * 1e-3), "fp64_ms": t64, "fp64_kernel_ms": k64,
-                         "fp64_roofline": frac(fl, k64),
+                         "fp64_roofline": frac(pats, k64),
                          "mixed_probs_per_s": len(pats) / (t32 * 1e-3), "mixed_ms": t32,
                          **error_columns(ref, h64, e64, "fp64"), **error_columns(ref, h32, e32, "mixed"),
                          "cpu_baseline": oracle_rate(pats, U, r)}
@@ -597,10 +614,9 @@ def extras(gbs, torch, measured_peak):
     gbs.autotune(30, gbs.FP64)
     t64, k64, h64, e64 = timed_batch(gbs, torch, K, pats, gbs.FP64, reps=2)
     t32, k32, h32, e32 = timed_batch(gbs, torch, K, pats, gbs.MIXED, reps=2)
-    fl = sum(model_flops(len(p)) for p in pats)
     out["large_m900"] = {"probs_per_s": len(pats) / (t64 * 1e-3), "ms": t64, "kernel_ms": k64,
                          "subset_terms_per_s": sum(2 ** (len(p) // 2) for p in pats) / (k64 * 1e-3),
-                         "roofline": frac(fl, k64),
+                         "roofline": frac(pats, k64),
                          "mixed_probs_per_s": len(pats) / (t32 * 1e-3), "mixed_ms": t32,
                          **error_columns(ref, h64, e64, "fp64"), **error_columns(ref, h32, e32, "mixed"),
                          "cpu_baseline": oracle_rate(pats[:16], U, r, target_s=8.0)}
