@@ -1048,7 +1048,8 @@ void serve_loop(gbs_server* s) {
         break;
       }
       free_stage->busy = true;
-      free_stage->t_launch = std::chrono::steady_clock::now();
+      // (whole requests run while their launches are still being enqueued)
+      free_stage->t_launch = free_stage->whole.empty() ? std::chrono::steady_clock::now() : tl0;
       s->stats.steps++;
       for (int p = 0; p < 2; ++p) {
         s->stats.items += free_stage->n_items[p];

@@ -126,3 +126,23 @@ def test_served_requests_without_a_fixed_point_range_count_once(gbs):
     p, h, err = np.zeros(b), np.zeros(2 * b), np.zeros(b)
     gbs.prob_batch(K, idx, n, offs, gbs.FP64, p_out=p, haf_out=h, err_out=err)
     assert [q[0] for q in got] == list(p) and [q[2] for q in got] == list(err)
+
+
+@pytest.mark.parametrize("graphs", [1, -1])
+def test_server_wall_time_covers_device_time(gbs, graphs):
+    """A step's wall time runs from the start of its launch to its detected
+    completion, so it is no shorter than its time on the device."""
+    import workloads as W
+
+    K = gbs.build_kernel(W.haar_unitary(60, 5), np.full(60, 0.8))
+    rng = np.random.default_rng(4)
+    srv = gbs.Server(K, use_graphs=graphs)
+    try:
+        for n in (4, 12, 16, 20, 24) * 4:
+            t = srv.submit(np.sort(rng.choice(60, size=n, replace=False)).astype(np.int32))
+            while srv.poll(t) is None:
+                pass
+        stats = srv.stats()
+    finally:
+        srv.destroy()
+    assert stats["step_wall_s"] >= stats["step_device_s"] > 0, stats
