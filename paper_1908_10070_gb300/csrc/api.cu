@@ -172,32 +172,39 @@ void pinned_release(int slot, cudaStream_t st) {
 // side streams: a call's independent kernels run beside its main stream
 // ------------------------------------------------------------------------
 // A lane is a non-blocking stream with the events that order it after a point
-// of the caller's stream (fork) and that stream after its work (join). Lanes
-// are taken for the time it takes to enqueue, so a handful serve any number of
-// threads; when none is free, or the caller's stream is being captured (a lane
-// may be in use outside the capture), the work goes to the caller's stream.
+// of the caller's stream (fork) and that stream after its work (join). A lane
+// stays with the caller's stream that took it (work of two streams in one lane
+// would make one wait for what the other waits for); the least recently used
+// ones go to new streams once there are kSideLanes. While another thread
+// enqueues through a stream's lane, or when the stream is being captured (a
+// lane may be in use outside the capture), the work goes to the caller's
+// stream.
 struct SideLane {
   int device = 0;
+  cudaStream_t owner = nullptr;  // the caller's stream (its handle alone), and which of its lanes
+  int index = 0;
+  uint64_t used = 0;
   cudaStream_t stream = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
   bool busy = false;
 };
-constexpr int kSideLanes = 8;  // per process; never freed (streams of devices that are in use)
+constexpr int kSideLanes = 16;  // per process; never freed (streams of devices that are in use)
 static std::mutex g_side_mu;
 static std::vector<SideLane*> g_side;
+static uint64_t g_side_clock = 0;
 
 class SideWork {
  public:
-  // Orders the lane after what `st` holds so far; stream() is the lane's, or
-  // `st` itself when there is none to be had.
-  void begin(cudaStream_t st) {
+  // Orders lane `index` of `st` after what `st` holds so far; stream() is the
+  // lane's, or `st` itself when there is none to be had.
+  void begin(cudaStream_t st, int index) {
     st_ = st;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
       cudaGetLastError();
       return;
     }
-    lane_ = acquire();
+    lane_ = acquire(st, index);
     if (!lane_) return;
     if (cudaEventRecord(lane_->fork, st) != cudaSuccess || cudaStreamWaitEvent(lane_->stream, lane_->fork, 0) != cudaSuccess) {
       cudaGetLastError();
@@ -218,16 +225,35 @@ class SideWork {
   ~SideWork() { join(); }
 
  private:
-  static SideLane* acquire() {
+  static SideLane* acquire(cudaStream_t st, int index) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_side_mu);
-    for (SideLane* l : g_side)
-      if (!l->busy && l->device == dev) {
-        l->busy = true;
-        return l;
+    SideLane* pick = nullptr;  // the stream's own, or the least recently used of the device
+    for (SideLane* l : g_side) {
+      if (l->device != dev) continue;
+      if (l->owner == st && l->index == index) {
+        pick = l->busy ? nullptr : l;
+        if (!pick) return nullptr;
+        break;
       }
-    if ((int)g_side.size() >= kSideLanes) return nullptr;
+      if (!l->busy && (!pick || l->used < pick->used)) pick = l;
+    }
+    if (!pick || pick->owner != st || pick->index != index) {
+      if ((int)g_side.size() < kSideLanes)
+        if (SideLane* l = create(dev)) {
+          g_side.push_back(l);
+          pick = l;
+        }
+      if (!pick) return nullptr;
+      pick->owner = st;
+      pick->index = index;
+    }
+    pick->busy = true;
+    pick->used = ++g_side_clock;
+    return pick;
+  }
+  static SideLane* create(int dev) {
     SideLane* l = new (std::nothrow) SideLane();
     if (!l) return nullptr;
     l->device = dev;
@@ -240,8 +266,6 @@ class SideWork {
       delete l;
       return nullptr;
     }
-    l->busy = true;
-    g_side.push_back(l);
     return l;
   }
   void release() {
@@ -1349,7 +1373,7 @@ int run_batch(const BatchArgs& a) {
         // Beside the larger orders' chain of layers, which is launched (90 us of
         // nearly empty kernels at order 24) also when the repeated-row sum takes
         // every matrix.
-        if (U.match && U.match_b) rep_side.begin(st);
+        if (U.match && U.match_b) rep_side.begin(st, 1);
         else rep_side.here(st);
         // the patterns the device chose for the repeated-row sum (the item
         // count is read on the device; the grid covers the reservation)
@@ -1393,7 +1417,7 @@ int run_batch(const BatchArgs& a) {
         // n = 4 52.8 and 50.4, n = 6 63.9 and 65.5, n = 10 79.9 and 87.8).
         const bool few = U.n_tiles <= device_sm_count() && maxn > 4;
         const bool beside = (shared && (U.match_b || few)) || (U.n_tiles && U.match_b);
-        if (beside) side.begin(st);
+        if (beside) side.begin(st, 0);
         else side.here(st);
         if (U.n_tiles) e = launch_match_small(M, U.n_tiles, U.tile_smem, side.stream());
         if (e == cudaSuccess && U.match_b) {
