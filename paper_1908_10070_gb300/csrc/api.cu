@@ -1578,6 +1578,7 @@ int run_batch(const BatchArgs& a) {
     }
   } while (0);
   side.join();
+  rep_side.join();
   pinned_release(slot, st);
   if (!hit && pe) plan_uploaded(pe, ret == GBS_OK);
   plan_release(pe);

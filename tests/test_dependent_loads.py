@@ -90,3 +90,14 @@ def test_flags_that_blocks_branch_on_are_constant():
     assert "terms_delta_kernel" in leave and "terms_series_kernel" in leave
     for k in leave:
         assert not re.search(r"P\.ok\[[^]]*\]\s*=[^=]", kernels[k]), k
+
+
+def test_side_streams_are_joined_before_the_scratch_is_freed():
+    """Also on errors: after the launches' block and ahead of scratch_free, which
+    frees in the order of the caller's stream alone."""
+    s = open(os.path.join(CSRC, "api.cu")).read()
+    body = s[s.index("int run_batch("):]
+    lanes = re.search(r"SideWork ([\w, ]+);", body).group(1).split(", ")
+    end = body[body.index("} while (0);"):]
+    end = end[:end.index("scratch_free(dmem")]
+    assert len(lanes) == 2 and all(re.search(r"^  %s\.join\(\);" % v, end, re.M) for v in lanes), lanes
