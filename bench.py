@@ -61,7 +61,7 @@ def term_macs(n: int) -> int:
                for s in range(1, h + 1))
 
 
-FIXED_MIN = 14  # smallest order whose terms are formed in fixed point
+FIXED_MIN = 12  # smallest order whose terms are formed in fixed point
 
 
 def fixed_point_flops(n: int) -> float:

@@ -202,7 +202,7 @@ __host__ __device__ inline int terms_group_bytes(int s, int h) {
   return (((h - 1) / 2 + 1) * 4 * (s - 1) + 3 * h + ((s + 3) >> 2)) * 16;
 }
 // Smallest order whose terms are formed in fixed point (haf_terms64.cuh: why).
-constexpr int kTermsFixedMin = 14;
+constexpr int kTermsFixedMin = 12;
 // The matrices of one order in a chunk. Per matrix the scratch holds n^2 limbs,
 // 2^h h series coefficients D, 2^(h-1) h of G, and the sums' parts.
 struct TermsGroup {

@@ -2,14 +2,16 @@
 // for the orders below kTermsFixedMin, and for the matrices that the
 // fixed-point kernels could not do or gave back.
 //
-// Below order 14 kappa from the fixed-point sum is off by more than kappa from
-// the subset sum was, whose Hafnian brings the larger part of its error
-// (largest of 240 Haar and random matrices an order, subset sum / fixed point /
-// now: n = 4 2.0e-15 / 1.2e-14 / 4e-16, n = 8 1.2e-14 / 2.2e-14 / 2e-15, n = 10
-// 2.4e-14 / 3.6e-14 / 4e-15; n = 12, medians, up to 3.8e-15 / 3.2e-15 / 2e-16).
-// From 14 on it is off by less (n = 14 7.6e-13 / 1.9e-14; n = 16 9.3e-13 /
-// 1.1e-14; n = 24 1.2e-11 / 1.1e-14). Here sum |f| is within 1e-15 of its
-// value, as the powers gave it.
+// Below order 12 kappa from the fixed-point sum is off by more than kappa from
+// the subset sum was, whose Hafnian brings the larger part of its error (60
+// matrices of four kinds an order, Haar and random; largest, subset sum / fixed
+// point / now: n = 4 2.0e-15 / 1.2e-14 / 4e-16, n = 8 1.2e-14 / 2.2e-14 / 2e-15,
+// n = 10 2.4e-14 / 3.6e-14 / 3e-15). From 12 on it is off by less, in the mean,
+// the root mean square and the largest of each kind (n = 12 at most 7.2e-15,
+// 2.1e-14, 1.5e-13 / 3.5e-15, 4.5e-15, 1.4e-14; largest at n = 16 9.3e-13 /
+// 1.1e-14, at 24 1.2e-11 / 1.1e-14), and FP64 would take twice the time (1024
+// of n = 12 318 us instead of 165, 399 by the subset sum). Here sum |f| is
+// within 1e-15 of its value, as the powers gave it.
 //
 // The same Krylov vectors and series as there (a third of the products of the
 // powers of a subset's matrix at order 16, a quarter at 30), on the matrix
@@ -40,8 +42,8 @@ __device__ __forceinline__ void zmac(double2& c, double2 a, double2 b) {
 // of terms_delta_kernel. The root is taken by the subset's lanes for the larger
 // orders, an eighth more work than by one thread of the series kernel, whose
 // chain was twice as long for it (a lone matrix of order 24: 635 -> 500 us);
-// small orders come in numbers and have short chains (1024 of order 12 took
-// 355 us with the root here, 303 there).
+// small orders come in numbers and have short chains (4096 of order 8 took 245
+// us with the root here, 207 there).
 __global__ void __launch_bounds__(kDeltaThreads) terms64_delta_kernel(const TermsLaunch P, const TermsChunk C) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int binom[kMaxH + 1][kMaxH + 1], rows[kMaxN], s_max;

@@ -18,5 +18,5 @@ def test_work_counts_split_by_pipe():
     for n in range(2, 31, 2):
         total = bench.fixed_point_flops(n) + bench.fp64_flops(n)
         assert total == 8 * (bench.matching_macs(n) + bench.term_macs(n))
-        assert (bench.fixed_point_flops(n) > 0) == (n >= 14)
+        assert (bench.fixed_point_flops(n) > 0) == (n >= 12)
     assert abs(bench.fixed_point_peak_tflops() / (152 * 4 * 32 / 28 * 8 * 2.07e-3) - 1) < 1e-12

@@ -59,7 +59,7 @@ def moduli(A):
     return total
 
 
-@pytest.mark.parametrize("n,count", [(2, 1), (2, 300), (4, 1), (4, 70), (6, 33), (8, 17), (10, 9), (12, 1), (12, 5)])
+@pytest.mark.parametrize("n,count", [(2, 1), (2, 300), (4, 1), (4, 70), (6, 33), (8, 17), (10, 1), (10, 9)])
 def test_small_orders_keep_double_precision(gbs, n, count):
     """Blocks of one and of many matrices, the last one partly filled."""
     rng = np.random.default_rng(100 * n + count)
