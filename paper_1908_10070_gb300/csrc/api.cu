@@ -655,7 +655,7 @@ struct BatchLayout {
 };
 
 // Scratch of the matching route's larger orders: the matrices of a call go in
-// chunks of at most this many bytes (one matrix of order 32 takes 34 MB). A
+// chunks of at most this many bytes (one matrix of order 30 takes 13 MB). A
 // chunk costs about 25 launches, against 4 ms of work in 512 MB of order 28.
 constexpr size_t kMatchBudget = (size_t)512 << 20;
 
@@ -936,7 +936,7 @@ int run_batch(const BatchArgs& a) {
   (hmode ? U.src_elems : U.idx_elems) = elems;
   const int maxn = U.maxn;
   // FP64: the Hafnians by partial matchings; the subset sum's terms are formed
-  // (in fixed point) only for the error estimate made of their moduli. Tuning
+  // (in fixed point, some in FP64) only for the error estimate made of their moduli. Tuning
   // runs time the subset sum itself.
   if (a.stage && (a.precision != GBS_FP64 || maxn > kMatchMaxN)) return fail(GBS_EINVAL, "staged call");
   U.match = a.precision == GBS_FP64 && !a.cfg_override && maxn <= kMatchMaxN;

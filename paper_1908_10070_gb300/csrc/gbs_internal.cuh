@@ -368,10 +368,15 @@ struct RepLaunch {
 // pattern finds its distinct modes and multiplicities and applies the cost
 // rule: the repeated-row sum when the
 // pattern has a repeated mode, at most d_max[n] distinct modes, T <= 2^30 and
-// 4 ceil(T / 2) (d^2 + 3d + 60) < subset_cost[n]. The last block to finish
+// 4 ceil(T / 2) (d^2 + 3d + 60) < subset_cost[n]. (The rule weighs both sums
+// as they were when it was fitted. A term now costs about 40 operations
+// whatever d, and a pattern that stays takes the matchings, so orders 8..16
+// with about n / 2 distinct modes take this route at up to 2.5 times the
+// matchings' operations; it is kept because it fixes which estimate, and which
+// bits, a pattern gets.) The last block to finish
 // then assigns partial ranges in pattern order: a pattern keeps the route
 // only while the running total of chunks stays within cap (later ones fall
-// back to the subset sum), so the choice is the same for the same batch.
+// back to the batch's other route), so the choice is the same for the same batch.
 struct RoutePlan {
   const int* idx;
   const PatDesc* pats;
@@ -380,7 +385,7 @@ struct RoutePlan {
   int cap;                 // repeated-row partial slots available
   double subset_cost[kMaxN + 1];
   int d_max[kMaxN + 1];
-  int* rep_half;           // out, per pattern: terms summed (ceil(T / 2)), 0 = subset sum
+  int* rep_half;           // out, per pattern: terms summed (ceil(T / 2)), 0 = the other route
   int* rep_end;            // out, per pattern: end of its partial range (non-decreasing)
   int* rep_total;          // out: partial slots used (the repeated-row item count)
   unsigned* blocks_done;   // zero before launch
@@ -394,7 +399,7 @@ struct RoutePlan {
 constexpr int kMatchMaxN = 30;       // batches with larger orders keep the subset sum
 constexpr int kMatchSmallMax = 18;   // largest order whose layers live in shared memory
 constexpr int kMatchThreads = 256;
-constexpr int kMatchTileBytes = 112 * 1024;  // two blocks an SM
+constexpr int kMatchTileBytes = 104 * 1024;  // two blocks an SM, with 6.3 KB of static tables each
 constexpr int kMatchTail = 9;        // the last layers of larger orders go back to shared memory
 struct MatchTile {
   int n, lp, first, count;  // matrices order[first, first + count)
