@@ -1052,10 +1052,10 @@ int run_batch(const BatchArgs& a) {
       return fail(GBS_ENOMEM, "too many work items (%lld)", (long long)U.n_items);
 
     // FP64 probabilities: the route choice (repeated-row sum for bunched
-    // patterns) is made on the device (route_plan_kernel) before the subset
+    // patterns) is made on the device (route_plan_kernel) ahead of the other
     // sum; repeated-row partial slots are reserved for the most each pattern's
     // order can need, up to kDevRepCap in all (patterns past that in batch
-    // order keep the subset sum)
+    // order keep the other route)
     constexpr int64_t kDevRepCap = (int64_t)1 << 20;
     if (a.mode == BatchArgs::PROB && a.precision == GBS_FP64 && U.idx_elems > 0 && !a.stage) {
       for (int b = 0; b < batch; ++b) U.dev_rep_cap += rep_max_chunks(a.n[b]);

@@ -1614,7 +1614,7 @@ __global__ void __launch_bounds__(256) route_plan_kernel(const RoutePlan R) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  if (__ldcg(R.n_chosen) == 0) {  // every pattern keeps the subset sum: no ranges to assign
+  if (__ldcg(R.n_chosen) == 0) {  // every pattern keeps the other route: no ranges to assign
     if (threadIdx.x == 0) *R.rep_total = 0;
     return;
   }
